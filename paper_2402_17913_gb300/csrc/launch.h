@@ -71,6 +71,15 @@ cudaError_t launch_up_s3(const LevelDev& L, const void* b, const void* xin, void
                          float sc, SolveState* st, double* partials, cudaStream_t s);
 template <typename T, bool MASKED>
 cudaError_t prepare_s3_kernels();
+// 3D level kernels of small levels, a 16 x 4 x 4 tile per block (two sweeps;
+// mg_small3d.cu).
+bool small3d_eligible(int dim, int pre, int post, const LevelDev& L);
+template <typename T, bool MASKED, typename TB = T>
+cudaError_t launch_down_c3(const LevelDev& L, const void* b, void* x, void* bcoarse, float omega,
+                           const SolveState* st, cudaStream_t s);
+template <typename T, bool MASKED, bool FINEST, typename TB = T>
+cudaError_t launch_up_c3(const LevelDev& L, const void* b, const void* xin, void* xout, const void* e, float omega,
+                         float sc, SolveState* st, double* partials, cudaStream_t s);
 // 2D level kernels streamed along y by single warps (two sweeps;
 // mg_stream2d.cu); arrays 16-byte aligned.
 bool stream2d_eligible(int dim, int pre, int post, const LevelDev& L);

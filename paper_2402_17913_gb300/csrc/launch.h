@@ -41,7 +41,20 @@ size_t coarse_layout(int* off, const LevelDev* lv, int nlev, int dim);
 // Write the constant part of the single-block kernel's shared memory (zero
 // ghost rings and arrays, inverse diagonals) to `image` (device).
 cudaError_t launch_coarse_image(const CoarseArgs& a, float* image, size_t bytes, cudaStream_t s);
-int coarse_start_level(const LevelDev* lv, int L, int dim, size_t smem_limit);
+// First level handled by the single-block kernel (or, with `dense`, by the
+// dense matrix of the coarse cycle).
+int coarse_start_level(const LevelDev* lv, int L, int dim, size_t smem_limit, bool dense);
+
+// The coarse cycle of level n cells as a dense matrix (mg_dense.cu): bytes of
+// the matrix and of its set-up's scratch, its set-up (a.finest 0; a wait
+// that times out sets st->status), and y = M b (b and y with 16-byte aligned
+// storage padded to a multiple of four values).
+size_t dense_bytes(int n);
+size_t dense_scratch_bytes(int n);
+cudaError_t launch_dense_matrix(const CoarseArgs& a, size_t smem_bytes, int n, float* M, float* scratch,
+                                SolveState* st, cudaStream_t s);
+template <typename T>
+cudaError_t launch_dense(int n, const float* M, const void* b, void* y, const SolveState* st, cudaStream_t s);
 
 // Level legs: T is the storage of a level's iterate and of its coarse-side
 // arrays, TB that of its right-hand side b and of the up leg's output (the

@@ -18,10 +18,11 @@ static int grid_1d(size_t n, int cap) {
 }
 
 // ---------------------------------------------------------------------------
-// Below a few thousand cells a level is too small to fill the GPU, so the
-// remaining part of the cycle (down legs, the exact coarsest solve, up
-// legs) runs inside one block of 1024 threads with every level resident in
-// shared memory.  One SM executes it, so it is written for instruction
+// The whole cycle of a grid of at most 2048 cells, and of the coarse levels of
+// the allocation-free cycle (handles apply those as one dense matrix,
+// mg_dense.cu, whose columns this block's cycle computes): down legs, the
+// exact coarsest solve and up legs inside one block of 1024 threads with
+// every level resident in shared memory.  One SM executes it, so it is written for instruction
 // count: each level is stored with a zero ghost ring (no bounds checks; the
 // ring is the zero padding of Sec. 2.1), the inverse diagonal is computed
 // once per launch (0 marks a non-fluid cell), and a sweep is
@@ -58,21 +59,25 @@ size_t coarse_layout(int* off, const LevelDev* lv, int nlev, int dim) {
 
 // Largest level (cells) the single-block kernel takes: 2048 in 2D and 8192
 // in 3D (measured on GB300: the 2048x1024 flow step is 4% faster when the
-// 128x64 level runs on the tiled kernels, the 256^3 solve is not), or
-// NPMG_COARSE_CELLS (64 .. 8192) to tune it.
-static size_t coarse_cells_limit(int dim) {
+// 128x64 level runs on the tiled kernels, the 256^3 solve is not).  The dense
+// matrix takes 2048 in both (16 MB; its share of a cycle grows with the
+// square): 1024 / 2048 / 4096 cells gave 2.43 / 2.22 / 2.22 ms on the 1600x960
+// solve, 1.89 / 1.84 / 1.86 ms on the 2048x1024 flow step, 2.38 / 2.38 / 2.69
+// on 128^3 and 9.87 / 9.87 / 10.21 on 256^3.  NPMG_COARSE_CELLS (64 .. 8192)
+// sets either.
+static size_t coarse_cells_limit(int dim, bool dense) {
   const char* e = getenv("NPMG_COARSE_CELLS");
   const long v = e ? atol(e) : 0;
   if (v >= 64 && v <= 8192) return (size_t)v;
-  return dim == 3 ? 8192 : 2048;
+  return dim == 3 && !dense ? 8192 : 2048;
 }
 
 // First level handled by the single-block kernel: levels within the cell
 // limit whose padded arrays fit the block's shared memory.
-int coarse_start_level(const LevelDev* lv, int L, int dim, size_t smem_limit) {
+int coarse_start_level(const LevelDev* lv, int L, int dim, size_t smem_limit, bool dense) {
   int kc = L - 1;
   int off[kMaxLevels];
-  const size_t lim = coarse_cells_limit(dim);
+  const size_t lim = coarse_cells_limit(dim, dense);
   while (kc > 0 && (size_t)lv[kc - 1].nx * lv[kc - 1].ny * lv[kc - 1].nz <= lim &&
          coarse_layout(off, lv + kc - 1, L - kc + 1, dim) <= smem_limit)
     --kc;
@@ -104,12 +109,7 @@ cudaError_t prepare_coarse(size_t smem_bytes) {
   return cudaFuncSetAttribute(k_coarse<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - 1024);
 }
 template cudaError_t prepare_coarse<float>(size_t);
-template cudaError_t prepare_coarse<__half>(size_t);
-template cudaError_t prepare_coarse<__nv_bfloat16>(size_t);
 template cudaError_t launch_coarse<float>(const CoarseArgs&, size_t, const void*, void*, SolveState*, cudaStream_t);
-template cudaError_t launch_coarse<__half>(const CoarseArgs&, size_t, const void*, void*, SolveState*, cudaStream_t);
-template cudaError_t launch_coarse<__nv_bfloat16>(const CoarseArgs&, size_t, const void*, void*, SolveState*,
-                                                  cudaStream_t);
 
 // ---------------------------------------------------------------------------
 // Set-up kernels (run once in mg_create).

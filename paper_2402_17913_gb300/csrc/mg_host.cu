@@ -143,8 +143,9 @@ static cudaError_t up_leg(mg_handle_s* h, int k, const void* b, void* xo, const 
 }
 
 // One application of the preconditioner M (one cycle from a zero guess):
-// down legs on levels 0 .. kc-1, the single-block kernel for kc .. L-1, up
-// legs back to level 0.  r and z (level 0's right-hand side and output) are
+// down legs on levels 0 .. kc-1, the dense matrix of the cycle on levels
+// kc .. L-1 (a grid with kc = 0: the single-block kernel), up legs back to
+// level 0.  r and z (level 0's right-hand side and output) are
 // float32; the level arrays below are T.  With `st` it is the CG
 // preconditioner (kernels skip once CG converged; the finest up leg reduces
 // (r, z)).
@@ -192,7 +193,7 @@ static cudaError_t enqueue_vcycle(mg_handle_s* h, const void* r, void* z, SolveS
                            h->clu_y, st, s);
     else
       e = h->kc == 0 ? launch_coarse<float>(ca, h->ca_smem, r, z, st, s)
-                     : launch_coarse<T>(ca, h->ca_smem, h->bk[h->kc], h->yk[h->kc], st, s);
+                     : launch_dense<T>((int)h->ncell[h->kc], h->dense, h->bk[h->kc], h->yk[h->kc], st, s);
   }
   if (e != cudaSuccess) return e;
   for (int k = kdown - 1; k >= 0; --k) {
@@ -646,7 +647,7 @@ mg_status mg_create(mg_handle* out, int dim, const int64_t shape[3], const doubl
     geo[k].ny = (int)h->n[k][1];
     geo[k].nz = (int)h->n[k][2];
   }
-  const int kc = coarse_start_level(geo, L, dim, (size_t)optin - 2048);
+  const int kc = coarse_start_level(geo, L, dim, (size_t)optin - 2048, true);
   h->kc = kc;
   {
     int offtmp[kMaxLevels];
@@ -687,6 +688,10 @@ mg_status mg_create(mg_handle* out, int dim, const int64_t shape[3], const doubl
   plan.push_back({(void**)&h->bsave, n0c * 4});
   plan.push_back({(void**)&h->inv, (size_t)2 * h->ncoarse * h->ncoarse * 8});
   plan.push_back({(void**)&h->cimage, h->ca_smem});
+  if (kc > 0) {
+    plan.push_back({(void**)&h->dense, dense_bytes((int)h->ncell[kc])});
+    plan.push_back({(void**)&h->dense_scratch, dense_scratch_bytes((int)h->ncell[kc])});
+  }
   if (dim == 2 && o.prec == MG_FP32 && kc >= 1) {
     // the cluster path's coarse cycle starts at level kc or below: its
     // right-hand side, correction and shared-memory image fit level kc's
@@ -772,6 +777,10 @@ mg_status mg_create(mg_handle* out, int dim, const int64_t shape[3], const doubl
     ca.s = (float)o.coarse_scale;
     NPMG_TRY(launch_coarse_image(ca, h->cimage, h->ca_smem, s));
     ca.image = h->cimage;
+    if (kc > 0) {
+      NPMG_TRY(launch_dense_matrix(ca, h->ca_smem, (int)h->ncell[kc], h->dense, h->dense_scratch, h->st, s));
+      NPMG_TRY(cudaMemcpyAsync(h->st_host, h->st, sizeof(SolveState), cudaMemcpyDeviceToHost, s));
+    }
   }
   h->nb1d = default_blocks_1d(h, h->ncell[0]);
   {
@@ -790,8 +799,7 @@ mg_status mg_create(mg_handle* out, int dim, const int64_t shape[3], const doubl
     using T = std::remove_pointer_t<decltype(tp)>;
     constexpr bool M = decltype(mc)::value;
     cudaError_t e = prepare_level_kernels<DIM, T, M>(o.pre, o.post);
-    if (e == cudaSuccess) e = prepare_coarse<T>(h->ca_smem);
-    if (e == cudaSuccess && !std::is_same<T, float>::value) e = prepare_coarse<float>(h->ca_smem);
+    if (e == cudaSuccess) e = prepare_coarse<float>(h->ca_smem);
     if (e == cudaSuccess && DIM == 2) e = prepare_tma_kernels<T, M>();
     if (e == cudaSuccess && DIM == 3) e = prepare_s3_kernels<T, M>();
     if (e == cudaSuccess && DIM == 3) e = prepare_r3_kernels<T, M>();
@@ -885,6 +893,11 @@ mg_status mg_create(mg_handle* out, int dim, const int64_t shape[3], const doubl
   NPMG_TRY(cudaStreamSynchronize(s));
   NPMG_TRY(cudaGetLastError());
 #undef NPMG_TRY
+  if (kc > 0 && h->st_host->status == MG_TIMEOUT) {
+    set_error("mg_create: a load of the coarse cycle's set-up timed out");
+    st = MG_TIMEOUT;
+    goto fail;
+  }
   *out = h;
   return MG_OK;
 fail:

@@ -180,7 +180,7 @@ extern "C" mg_status mg_vcycle_noalloc(int dim, const int64_t shape[3], const do
     geo[k].ny = (int)nk[k][1];
     geo[k].nz = (int)nk[k][2];
   }
-  const int kc = coarse_start_level(geo, L, dim, (size_t)optin - 2048);
+  const int kc = coarse_start_level(geo, L, dim, (size_t)optin - 2048, false);
   // carve the static scratch
   unsigned char* base = nullptr;
   NPMG_CUDA(scratch_address(&base));

@@ -1,7 +1,7 @@
 """GPU parity of the level kernels and of the coarse cycle of small grids
 against the FP64 oracle: the 16 x 4 x 4 tiles of small 3D levels at their
 edges (one tile, whole tiles, remainders along each axis, a finest level, all
-storage types).  One cycle is compared to 2e-5 of its norm: each of its
+storage types), and the coarse cycle as a dense matrix.  One cycle is compared to 2e-5 of its norm: each of its
 some thirty float32 steps rounds to 2^-24 of the field's scale and the
 smoothers do not amplify (eight levels of a V(2,2) cycle: below 1e-5)."""
 import numpy as np
@@ -78,3 +78,22 @@ def test_small_3d_tiles_solve_in_every_storage(L, prec):
     assert status == L.MG_OK, st
     xs = P.solve_reference(shape, h, bc, b.astype(np.float64), solid, tol=1e-12, s=1.0)
     assert np.linalg.norm(x.cpu().numpy() - xs) / np.linalg.norm(xs) <= 1e-5
+
+
+DENSE = [
+    # shape, faces, solid fraction, levels (0: until a side is odd or 4)
+    ((64, 128), (0, 0, 0, 0), 0.0, 0),               # level 1 has 2048 cells, the most the matrix takes
+    ((60, 100), (1, 0, 1, 1), 0.05, 0),              # 1500 rows, coarsest 15 x 25
+    ((46, 46), (0, 0, 0, 0), 0.0, 2),                # 529 rows (no multiple of four), the matrix is the inverse
+    ((52, 92), (1, 0, 0, 1), 0.08, 0),               # 1196 rows over 299
+    ((24, 36, 20), (1, 0, 1, 1, 1, 1), 0.05, 0),     # 3D: 2160 cells on the tiles, 270 rows
+    ((18, 18, 24), (0,) * 6, 0.0, 2),                # 3D: 972 rows, the inverse
+    ((32, 96), (0, 0, 0, 1), 0.0, 5),                # the smallest matrices: 192, coarsest 2 x 6
+]
+
+
+@pytest.mark.parametrize("shape,bc,frac,levels", DENSE)
+def test_dense_coarse_cycle_matches_oracle(L, shape, bc, frac, levels):
+    check_cycle(L, shape, bc, frac, levels)
+    check_cycle(L, shape, bc, frac, levels, cycle="sawtooth")
+    check_cycle(L, shape, bc, frac, levels, pre=1, post=3)  # not symmetric

@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(256) k_p_update(LevelDev L, const T* __restric
     }
   }
   double tot;
-  if (grid_sum_last((double)acc, partials, &st->counter[kCntPAP], &tot)) {
+  if (grid_sum_last(acc, partials, &st->counter[kCntPAP], &tot)) {
     if (threadIdx.x == 0) {
       st->pAp = tot;
       st->alpha = st->krylov ? st->rz / tot : 1.0;
@@ -296,7 +296,7 @@ __global__ void __launch_bounds__(256) k_xr_update(LevelDev L, const T* __restri
     }
   }
   double tot;
-  if (grid_sum_last((double)acc, partials, &st->counter[kCntRR], &tot)) {
+  if (grid_sum_last(acc, partials, &st->counter[kCntRR], &tot)) {
     if (threadIdx.x == 0) inner_decide(st, tot);
   }
 }
@@ -393,7 +393,7 @@ __global__ void __launch_bounds__(256) k_p_update_z(LevelDev L, const float* __r
     }
   }
   double tot;
-  if (grid_sum_last((double)acc, partials, &st->counter[kCntPAP], &tot)) {
+  if (grid_sum_last(acc, partials, &st->counter[kCntPAP], &tot)) {
     if (threadIdx.x == 0) {
       st->pAp = tot;
       st->alpha = st->krylov ? st->rz / tot : 1.0;
@@ -558,7 +558,7 @@ __global__ void __launch_bounds__(256) k_outer(LevelDev L, OuterArgs oa, const f
     }
   }
   double tot;
-  if (grid_sum_last((double)acc, partials, &st->counter[kCntOuter], &tot)) {
+  if (grid_sum_last(acc, partials, &st->counter[kCntOuter], &tot)) {
     if (threadIdx.x == 0) {
       outer_decide(st, tot, oa.c2, sig_new_d, UPDATE);
       if (UPDATE && dyn) st->cur ^= 1;
@@ -832,7 +832,7 @@ __global__ void __launch_bounds__(256) k_init(LevelDev L, const float* __restric
     }
   }
   double tot;
-  if (grid_sum_last((double)acc, partials, &st->counter[kCntInit], &tot)) {
+  if (grid_sum_last(acc, partials, &st->counter[kCntInit], &tot)) {
     if (threadIdx.x == 0) init_state(st, prm, tot, c);
   }
 }

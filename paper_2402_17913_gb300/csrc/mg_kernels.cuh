@@ -271,7 +271,7 @@ k_up(LevelDev L, const TB* __restrict__ b, const T* __restrict__ xin, TB* __rest
   }
   if (FINEST) {
     double tot;
-    if (grid_sum_last((double)acc, partials, &st->counter[kCntRZ], &tot)) {
+    if (grid_sum_last(acc, partials, &st->counter[kCntRZ], &tot)) {
       if (threadIdx.x == 0) {
         st->rz = tot;
         st->beta = (st->first || !st->krylov) ? 0.0 : tot / st->rz_old;

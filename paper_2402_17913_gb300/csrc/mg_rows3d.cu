@@ -416,7 +416,7 @@ __global__ void __launch_bounds__(NT, 1) k_up_r3(LevelDev L, const TB* __restric
   });
   if (FINEST) {
     double tot;
-    if (grid_sum_last((double)acc, partials, &st->counter[kCntRZ], &tot)) {
+    if (grid_sum_last(acc, partials, &st->counter[kCntRZ], &tot)) {
       if (threadIdx.x == 0) {
         st->rz = tot;
         st->beta = (st->first || !st->krylov) ? 0.0 : tot / st->rz_old;

@@ -292,7 +292,7 @@ k_up_tma(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUtens
   }
   if (FINEST) {
     double tot;
-    if (grid_sum_last((double)acc, partials, &st->counter[kCntRZ], &tot)) {
+    if (grid_sum_last(acc, partials, &st->counter[kCntRZ], &tot)) {
       if (threadIdx.x == 0) {
         st->rz = tot;
         st->beta = (st->first || !st->krylov) ? 0.0 : tot / st->rz_old;

@@ -439,7 +439,7 @@ __global__ void __launch_bounds__(NT, 1)
   if (failed) fail(st);
   if (FINEST) {
     double tot;
-    if (grid_sum_last((double)acc, partials, &st->counter[kCntRZ], &tot)) {
+    if (grid_sum_last(acc, partials, &st->counter[kCntRZ], &tot)) {
       if (threadIdx.x == 0 && !failed) {
         st->rz = tot;
         st->beta = (st->first || !st->krylov) ? 0.0 : tot / st->rz_old;
@@ -743,7 +743,7 @@ __global__ void __launch_bounds__(NT, 2)
   });
   if (failed) fail(st);
   double tot;
-  if (grid_sum_last((double)acc, partials, &st->counter[kCntPAP], &tot)) {
+  if (grid_sum_last(acc, partials, &st->counter[kCntPAP], &tot)) {
     if (threadIdx.x == 0 && !failed) {
       st->pAp = tot;
       st->alpha = st->krylov ? st->rz / tot : 1.0;
@@ -900,7 +900,7 @@ __global__ void __launch_bounds__(NT, 1)
   });
   if (failed) fail(st);
   double tot;
-  if (grid_sum_last((double)acc, partials, &st->counter[kCntRR], &tot)) {
+  if (grid_sum_last(acc, partials, &st->counter[kCntRR], &tot)) {
     if (threadIdx.x == 0 && !failed) inner_decide(st, tot);
   }
 }

@@ -109,34 +109,99 @@ __device__ __forceinline__ unsigned linear_block() {
   return blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
 }
 
-// Each block contributes `v`; returns true in every thread of the last block
-// to arrive, with the grid total in *total (valid in all its threads).
-__device__ __forceinline__ bool grid_sum_last(double v, double* partials,
-                                              unsigned int* counter,
-                                              double* total) {
+// Float-float pair (hi + lo, about 48 significant bits) of a reduction:
+// two_sum (Knuth) of the high parts, the low parts added to its error.
+__device__ __forceinline__ float2 pair_add(float2 a, float2 b) {
+  const float s = a.x + b.x, bb = s - a.x;
+  const float e = ((a.x - (s - bb)) + (b.x - bb)) + (a.y + b.y);
+  const float h = s + e;
+  return make_float2(h, e - (h - s));
+}
+
+// Sum of the first `n` lanes' pairs, valid in lane 0 (lanes from n on add
+// nothing; they may not exist).
+__device__ __forceinline__ float2 warp_pair_sum(float2 v, int lane, int n) {
+  const unsigned mask = n >= 32 ? 0xffffffffu : (1u << n) - 1u;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float2 t = make_float2(__shfl_down_sync(mask, v.x, o), __shfl_down_sync(mask, v.y, o));
+    if (lane + o < n) v = pair_add(v, t);
+  }
+  return v;
+}
+
+// Sum over the block, valid in thread 0; `sh` holds >= 32 pairs.
+__device__ __forceinline__ float2 block_pair_sum(float2 v, float2* sh) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int nw = (blockDim.x + 31) >> 5;
+  v = warp_pair_sum(v, lane, min(32, (int)blockDim.x - 32 * w));
+  __syncthreads();
+  if (lane == 0) sh[w] = v;
+  __syncthreads();
+  if (w == 0) v = warp_pair_sum(lane < nw ? sh[lane] : make_float2(0.f, 0.f), lane, min(32, (int)blockDim.x));
+  return v;
+}
+
+// One more arrival at the counter: the block's writes before it are visible
+// to the block that sees the last count (release), and that block's later
+// reads are ordered after it (acquire; the other threads' by the barrier
+// that follows).
+__device__ __forceinline__ unsigned arrive(unsigned int* counter) {
+  unsigned t;
+  asm volatile("atom.add.acq_rel.gpu.u32 %0, [%1], 1;" : "=r"(t) : "l"(counter) : "memory");
+  return t;
+}
+
+// Each block contributes `v`, a sum of float32 terms kept in float32 by each
+// thread; returns true in every thread of the last block to arrive, with the
+// grid total in *total (valid in thread 0).  Latency-bound tail of every
+// reducing kernel: the sums are float-float pairs (the terms themselves carry
+// 2^-24), since one float64 warp instruction holds its sub-partition's pipe
+// for 64 cycles on GB300 and a float64 tree is ten dependent ones per level,
+// and the arrival is one acquire-release atomic instead of a fence on each
+// side.  Against the float64 tree with fences: 448x576 solve 1.25 -> 1.23 ms,
+// 128^3 2.38 -> 2.31 ms, 2048x1024 flow step 1.845 -> 1.820 ms.
+__device__ __forceinline__ bool grid_sum_last(float v, double* partials, unsigned int* counter, double* total) {
+  __shared__ float2 sh[32];
+  __shared__ bool last;
+  float2* part = reinterpret_cast<float2*>(partials);
+  const float2 s = block_pair_sum(make_float2(v, 0.f), sh);
+  const unsigned nb = gridDim.x * gridDim.y * gridDim.z;
+  if (threadIdx.x == 0) {
+    part[linear_block()] = s;
+    last = arrive(counter) == nb - 1;
+  }
+  __syncthreads();
+  if (!last) return false;
+  float2 acc = make_float2(0.f, 0.f);
+  for (unsigned i = threadIdx.x; i < nb; i += blockDim.x) acc = pair_add(acc, __ldcg(part + i));
+  const float2 r = block_pair_sum(acc, sh);
+  if (threadIdx.x == 0) {
+    *total = (double)r.x + (double)r.y;
+    *counter = 0u;
+  }
+  return true;
+}
+
+// The same for float64 contributions.
+__device__ __forceinline__ bool grid_sum_last(double v, double* partials, unsigned int* counter, double* total) {
   __shared__ double sh[32];
   __shared__ bool last;
-  __shared__ double tot;
   const double s = block_sum(v, sh);
   const unsigned nb = gridDim.x * gridDim.y * gridDim.z;
   if (threadIdx.x == 0) {
     partials[linear_block()] = s;
-    __threadfence();
-    const unsigned t = atomicAdd(counter, 1u);
-    last = (t == nb - 1);
+    last = arrive(counter) == nb - 1;
   }
   __syncthreads();
   if (!last) return false;
-  __threadfence();
   double acc = 0.0;
   for (unsigned i = threadIdx.x; i < nb; i += blockDim.x) acc += __ldcg(partials + i);
   const double r = block_sum(acc, sh);
   if (threadIdx.x == 0) {
-    tot = r;
+    *total = r;
     *counter = 0u;
   }
-  __syncthreads();
-  *total = tot;
   return true;
 }
 

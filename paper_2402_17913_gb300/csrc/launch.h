@@ -54,7 +54,8 @@ size_t dense_scratch_bytes(int n);
 cudaError_t launch_dense_matrix(const CoarseArgs& a, size_t smem_bytes, int n, float* M, float* scratch,
                                 SolveState* st, cudaStream_t s);
 template <typename T>
-cudaError_t launch_dense(int n, const float* M, const void* b, void* y, const SolveState* st, cudaStream_t s);
+cudaError_t launch_dense(int dim, int n, const float* M, const void* b, void* y, const SolveState* st,
+                         cudaStream_t s);
 
 // Level legs: T is the storage of a level's iterate and of its coarse-side
 // arrays, TB that of its right-hand side b and of the up leg's output (the
@@ -84,15 +85,15 @@ cudaError_t launch_up_s3(const LevelDev& L, const void* b, const void* xin, void
                          float sc, SolveState* st, double* partials, cudaStream_t s);
 template <typename T, bool MASKED>
 cudaError_t prepare_s3_kernels();
-// 3D level kernels of small levels, a 16 x 4 x 4 tile per block (two sweeps;
-// mg_small3d.cu).
-bool small3d_eligible(int dim, int pre, int post, const LevelDev& L);
-template <typename T, bool MASKED, typename TB = T>
-cudaError_t launch_down_c3(const LevelDev& L, const void* b, void* x, void* bcoarse, float omega,
-                           const SolveState* st, cudaStream_t s);
-template <typename T, bool MASKED, bool FINEST, typename TB = T>
-cudaError_t launch_up_c3(const LevelDev& L, const void* b, const void* xin, void* xout, const void* e, float omega,
-                         float sc, SolveState* st, double* partials, cudaStream_t s);
+// Kernels of small levels, a tile of 256 cells per block (two sweeps;
+// mg_small.cu).
+bool small_level_eligible(int dim, int pre, int post, const LevelDev& L);
+template <int DIM, typename T, bool MASKED, typename TB = T>
+cudaError_t launch_down_c(const LevelDev& L, const void* b, void* x, void* bcoarse, float omega,
+                          const SolveState* st, cudaStream_t s);
+template <int DIM, typename T, bool MASKED, bool FINEST, typename TB = T>
+cudaError_t launch_up_c(const LevelDev& L, const void* b, const void* xin, void* xout, const void* e, float omega,
+                        float sc, SolveState* st, double* partials, cudaStream_t s);
 // 2D level kernels streamed along y by single warps (two sweeps;
 // mg_stream2d.cu); arrays 16-byte aligned.
 bool stream2d_eligible(int dim, int pre, int post, const LevelDev& L);

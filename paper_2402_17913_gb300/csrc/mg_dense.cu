@@ -92,7 +92,8 @@ constexpr int kAhead = 16;     // float4 of its row a lane holds before b is nee
 template <typename T>
 __global__ void __launch_bounds__(32 * kRowWarps) k_dense(int n, int ld, const float* __restrict__ M,
                                                           const T* __restrict__ b, T* __restrict__ y,
-                                                          const SolveState* __restrict__ st) {
+                                                          const SolveState* __restrict__ st, int release) {
+  if (release) chain_release();
   const int row = blockIdx.x * kRowWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   const float4* __restrict__ m = reinterpret_cast<const float4*>(M + (size_t)min(row, n - 1) * ld);
   const int n4 = ld / 4;
@@ -144,13 +145,14 @@ cudaError_t launch_dense_matrix(const CoarseArgs& a, size_t smem_bytes, int n, f
 }
 
 template <typename T>
-cudaError_t launch_dense(int n, const float* M, const void* b, void* y, const SolveState* st, cudaStream_t s) {
+cudaError_t launch_dense(int dim, int n, const float* M, const void* b, void* y, const SolveState* st,
+                         cudaStream_t s) {
   return launch_chain(k_dense<T>, (n + kRowWarps - 1) / kRowWarps, 32 * kRowWarps, 0, s, n, dense_stride(n), M,
-                      (const T*)b, (T*)y, st);
+                      (const T*)b, (T*)y, st, dim == 3 ? 1 : 0);
 }
-template cudaError_t launch_dense<float>(int, const float*, const void*, void*, const SolveState*, cudaStream_t);
-template cudaError_t launch_dense<__half>(int, const float*, const void*, void*, const SolveState*, cudaStream_t);
-template cudaError_t launch_dense<__nv_bfloat16>(int, const float*, const void*, void*, const SolveState*,
+template cudaError_t launch_dense<float>(int, int, const float*, const void*, void*, const SolveState*, cudaStream_t);
+template cudaError_t launch_dense<__half>(int, int, const float*, const void*, void*, const SolveState*, cudaStream_t);
+template cudaError_t launch_dense<__nv_bfloat16>(int, int, const float*, const void*, void*, const SolveState*,
                                                  cudaStream_t);
 
 }  // namespace npmg

@@ -61,7 +61,7 @@ struct mg_handle_s {
   npmg::TmaLevelMaps tmaps[npmg::kMaxLevels];  // TMA tensor maps per level (levels < kc)
   bool tma_ok[npmg::kMaxLevels];
   bool s3_ok[npmg::kMaxLevels];   // 3D levels on the z-streaming kernels
-  bool c3_ok[npmg::kMaxLevels];   // small 3D levels on the 16 x 4 x 4 tiles
+  bool c_ok[npmg::kMaxLevels];    // small levels on the 256-cell tiles
   bool s2_ok[npmg::kMaxLevels];   // 2D levels on the y-streaming warp kernels
   bool r3_ok[npmg::kMaxLevels];   // 3D levels on the row-warp z-streaming kernels
   npmg::Tma3Maps t3maps[npmg::kMaxLevels];  // tensor maps of the TMA-fed 3D kernels (levels < kc)

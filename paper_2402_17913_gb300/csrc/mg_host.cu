@@ -109,12 +109,12 @@ static cudaError_t down_leg(mg_handle_s* h, int k, const void* b, const TmaLevel
     if (stream2d_aligned(b)) return launch_down_saw<DIM, T, M, TB>(h->lv[k], b, h->xk[k], h->bk[k + 1], st, s);
     return launch_down<DIM, T, M, TB>(h->lv[k], b, h->xk[k], h->bk[k + 1], -1, om, st, s);
   }
+  if (h->c_ok[k]) return launch_down_c<DIM, T, M, TB>(h->lv[k], b, h->xk[k], h->bk[k + 1], om, st, s);
   if (DIM == 2 && h->s2_ok[k] && stream2d_aligned(b))
     return launch_down_w<T, M, TB>(h->lv[k], b, h->xk[k], h->bk[k + 1], om, st, s);
   if constexpr (std::is_same<T, TB>::value) {
     if (tm) return launch_down_tma<T, M>(*tm, h->lv[k], h->xk[k], h->bk[k + 1], om, st, s);
   }
-  if (DIM == 3 && h->c3_ok[k]) return launch_down_c3<T, M, TB>(h->lv[k], b, h->xk[k], h->bk[k + 1], om, st, s);
   if (DIM == 3 && t3) return launch_down_t3<T, M, TB>(*t3, h->lv[k], h->xk[k], h->bk[k + 1], om, st, s);
   if (DIM == 3 && h->r3_ok[k] && stream2d_aligned(b))
     return launch_down_r3<T, M, TB>(h->lv[k], b, h->xk[k], h->bk[k + 1], om, st, s);
@@ -126,13 +126,13 @@ template <int DIM, typename T, bool M, bool F, typename TB>
 static cudaError_t up_leg(mg_handle_s* h, int k, const void* b, void* xo, const TmaLevelMaps* tm,
                           const Tma3Maps* t3, SolveState* st, cudaStream_t s) {
   const float om = (float)h->opt.omega, sc = (float)h->opt.coarse_scale;
+  if (h->c_ok[k])
+    return launch_up_c<DIM, T, M, F, TB>(h->lv[k], b, h->xk[k], xo, h->yk[k + 1], om, sc, st, h->partials, s);
   if (DIM == 2 && h->s2_ok[k] && stream2d_aligned(b))
     return launch_up_w<T, M, F, TB>(h->lv[k], b, h->xk[k], xo, h->yk[k + 1], om, sc, st, h->partials, s);
   if constexpr (std::is_same<T, TB>::value) {
     if (tm) return launch_up_tma<T, M, F>(*tm, h->lv[k], xo, om, sc, st, h->partials, s);
   }
-  if (DIM == 3 && h->c3_ok[k])
-    return launch_up_c3<T, M, F, TB>(h->lv[k], b, h->xk[k], xo, h->yk[k + 1], om, sc, st, h->partials, s);
   if (DIM == 3 && t3) return launch_up_t3<T, M, F, TB>(*t3, h->lv[k], xo, om, sc, st, h->partials, s);
   if (DIM == 3 && h->r3_ok[k] && stream2d_aligned(b))
     return launch_up_r3<T, M, F, TB>(h->lv[k], b, h->xk[k], xo, h->yk[k + 1], om, sc, st, h->partials, s);
@@ -193,7 +193,8 @@ static cudaError_t enqueue_vcycle(mg_handle_s* h, const void* r, void* z, SolveS
                            h->clu_y, st, s);
     else
       e = h->kc == 0 ? launch_coarse<float>(ca, h->ca_smem, r, z, st, s)
-                     : launch_dense<T>((int)h->ncell[h->kc], h->dense, h->bk[h->kc], h->yk[h->kc], st, s);
+                     : launch_dense<T>(DIM, (int)h->ncell[h->kc], h->dense, h->bk[h->kc], h->yk[h->kc], st,
+                                       s);
   }
   if (e != cudaSuccess) return e;
   for (int k = kdown - 1; k >= 0; --k) {
@@ -813,7 +814,7 @@ mg_status mg_create(mg_handle* out, int dim, const int64_t shape[3], const doubl
       h->s3_ok[k] = getenv("NPMG_NO_STREAM3D") == nullptr && stream3d_eligible(dim, pre_e, o.post, h->lv[k]);
       h->s2_ok[k] = getenv("NPMG_NO_STREAM2D") == nullptr && stream2d_eligible(dim, pre_e, o.post, h->lv[k]) &&
                     h->ncell[k] >= stream2d_min_cells();
-      h->c3_ok[k] = small3d_eligible(dim, pre_e, o.post, h->lv[k]);
+      h->c_ok[k] = small_level_eligible(dim, pre_e, o.post, h->lv[k]);
       h->r3_ok[k] = getenv("NPMG_NO_ROWS3D") == nullptr && rows3d_eligible(dim, pre_e, o.post, h->lv[k]);
     }
     // tensor maps of the TMA level kernels (2D, two sweeps, rows of 16k cells)

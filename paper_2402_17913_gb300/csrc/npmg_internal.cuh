@@ -61,12 +61,20 @@ enum Counter { kCntInit = 0, kCntOuter = 1, kCntRZ = 2, kCntPAP = 3, kCntRR = 4,
 // dependency on the previous one, so that their launch overlaps its drain;
 // each first waits until the preceding grid has completed and its writes
 // are visible (a no-op when it was launched without the dependency).
-// Nothing may be read or written before this call.  No grid releases its
-// successor early: measured on GB300, successors parked on the SMs from the
-// start of the previous grid made the 2D and 3D solves 5-8% slower (1-7%
-// when only grids of at most 32 or 128 blocks release early), while the
+// Only constants of the handle (cell bytes, the dense coarse matrix) may be
+// read before this call, and nothing written.  Most grids release their
+// successor at exit: measured on GB300, successors parked on the SMs from the
+// start of large grids made the 2D and 3D solves 5-8% slower, while the
 // release at exit makes the 2D flow step about 1.5% faster.
 __device__ __forceinline__ void chain_enter() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+// Release the successor now, so that its blocks start, form what does not
+// depend on this grid and wait for its end.  For the small 3D levels and the
+// coarse matrix between them, whose grids leave room on the SMs and whose
+// successors have work before their wait (geometry, diagonals, the matrix
+// rows): 256x128x128 FE flow step 3.41 -> 3.27 ms, masked 96x80x64 cycle 30.1
+// -> 27.7 us, 256^3 solve 9.85 -> 9.76 ms.  In 2D the same release measured
+// 2-5% slower (448x576 1.01 -> 1.06 ms), so 2D grids keep the release at exit.
+__device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 
 // ---------------------------------------------------------------------------
 // storage conversions
@@ -152,8 +160,8 @@ __device__ __forceinline__ unsigned arrive(unsigned int* counter) {
   return t;
 }
 
-// Each block contributes `v`, a sum of float32 terms kept in float32 by each
-// thread; returns true in every thread of the last block to arrive, with the
+// Each block contributes `v`, a sum of float32 terms kept in float32 (or as a
+// pair) by each thread; returns true in every thread of the last block to arrive, with the
 // grid total in *total (valid in thread 0).  Latency-bound tail of every
 // reducing kernel: the sums are float-float pairs (the terms themselves carry
 // 2^-24), since one float64 warp instruction holds its sub-partition's pipe
@@ -161,11 +169,11 @@ __device__ __forceinline__ unsigned arrive(unsigned int* counter) {
 // and the arrival is one acquire-release atomic instead of a fence on each
 // side.  Against the float64 tree with fences: 448x576 solve 1.25 -> 1.23 ms,
 // 128^3 2.38 -> 2.31 ms, 2048x1024 flow step 1.845 -> 1.820 ms.
-__device__ __forceinline__ bool grid_sum_last(float v, double* partials, unsigned int* counter, double* total) {
+__device__ __forceinline__ bool grid_sum_last(float2 v, double* partials, unsigned int* counter, double* total) {
   __shared__ float2 sh[32];
   __shared__ bool last;
   float2* part = reinterpret_cast<float2*>(partials);
-  const float2 s = block_pair_sum(make_float2(v, 0.f), sh);
+  const float2 s = block_pair_sum(v, sh);
   const unsigned nb = gridDim.x * gridDim.y * gridDim.z;
   if (threadIdx.x == 0) {
     part[linear_block()] = s;
@@ -181,6 +189,10 @@ __device__ __forceinline__ bool grid_sum_last(float v, double* partials, unsigne
     *counter = 0u;
   }
   return true;
+}
+
+__device__ __forceinline__ bool grid_sum_last(float v, double* partials, unsigned int* counter, double* total) {
+  return grid_sum_last(make_float2(v, 0.f), partials, counter, total);
 }
 
 // The same for float64 contributions.

@@ -1,5 +1,5 @@
 """GPU parity of the level kernels and of the coarse cycle of small grids
-against the FP64 oracle: the 16 x 4 x 4 tiles of small 3D levels at their
+against the FP64 oracle: the 256-cell tiles of small levels at their
 edges (one tile, whole tiles, remainders along each axis, a finest level, all
 storage types), and the coarse cycle as a dense matrix.  One cycle is compared to 2e-5 of its norm: each of its
 some thirty float32 steps rounds to 2^-24 of the field's scale and the
@@ -57,17 +57,32 @@ SMALL3D = [
 ]
 
 
+SMALL2D = [
+    ((64, 64), (0, 0, 0, 0), 0.0),            # whole tiles
+    ((72, 104), (1, 0, 1, 1), 0.06),          # a remainder in x (3.25 tiles), level 1 (36, 52) in both
+    ((400, 480), (0, 0, 1, 0), 0.05),         # close to the largest level (192,000 cells)
+    ((512, 416), (0, 1, 0, 0), 0.0),          # just above it: the TMA-fed tiles, then the small ones
+]
+
+
+@pytest.mark.parametrize("shape,bc,frac", SMALL2D)
+def test_small_2d_tiles_match_oracle(L, shape, bc, frac):
+    check_cycle(L, shape, bc, frac)
+    check_cycle(L, shape, bc, frac, cycle="sawtooth")
+
+
 @pytest.mark.parametrize("shape,bc,frac", SMALL3D)
 def test_small_3d_tiles_match_oracle(L, shape, bc, frac):
     check_cycle(L, shape, bc, frac)
     check_cycle(L, shape, bc, frac, cycle="sawtooth")
 
 
-@pytest.mark.parametrize("prec", [0, 1, 2])
-def test_small_3d_tiles_solve_in_every_storage(L, prec):
+@pytest.mark.parametrize("shape,bc,prec", [((20, 24, 40), (1, 0, 1, 1, 0, 1), 0), ((20, 24, 40), (1, 0, 1, 1, 0, 1), 1),
+                                           ((20, 24, 40), (1, 0, 1, 1, 0, 1), 2), ((72, 104), (1, 0, 1, 1), 0),
+                                           ((72, 104), (1, 0, 1, 1), 1)])
+def test_small_tiles_solve_in_every_storage(L, shape, bc, prec):
     """The finest level on the tiles (its up leg reduces (r, z)), in every
     level storage: relres 1e-6 and the oracle's solution."""
-    shape, bc = (20, 24, 40), (1, 0, 1, 1, 0, 1)
     hdl, solid, h = setup(L, shape, bc, 0.06, prec=prec)
     try:
         b = I.blob_rhs(shape, 0, solid=solid).astype(np.float32)

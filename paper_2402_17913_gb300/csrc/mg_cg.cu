@@ -7,6 +7,7 @@
 // results are reproducible run to run).
 #include <math.h>
 #include <stdlib.h>
+#include <string.h>
 #include <type_traits>
 
 #include "launch.h"
@@ -568,12 +569,21 @@ __global__ void __launch_bounds__(256) k_outer(LevelDev L, OuterArgs oa, const f
 
 // Refinement step in float64: the iterate x is a float64 array.  With
 // UPDATE, k_update64 first writes x + sigma d' (float64) into the other
-// buffer; k_outer64 then forms, in the scaled units of the inner solve,
-// r = c b - A' x in float64 from the (updated) iterate, reduces ||r|| in
-// float64 and writes r' = r / sigma_new rounded to float32.  The last block
-// decides as in the float-float form (outer_decide).  The update is its own
-// pass so that every cell is updated once (not once per neighbour that
-// reads it): GB300's float64 rate is 1/64 of its float32 rate.
+// buffer; the residual kernel then forms, in the scaled units of the inner
+// solve, r = c b - A' x from the (updated) iterate, reduces ||r|| and writes
+// r' = r / sigma_new rounded to float32.  The last block decides as in the
+// float-float form (outer_decide).  The update is its own pass so that every
+// cell is updated once (not once per neighbour that reads it): GB300's
+// float64 rate is 1/64 of its float32 rate.
+
+// The float64 value of a float32 (not denormal, infinite or NaN: those take
+// the conversion) by moving its fields, without the float64 pipe.
+__device__ __forceinline__ double widen(float v) {
+  const unsigned u = __float_as_uint(v), e = (u >> 23) & 255u;
+  if (e == 0u || e == 255u) return (u << 1) ? (double)v : 0.0;
+  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))), (int)(u << 29));
+}
+
 __global__ void __launch_bounds__(256) k_update64(size_t n, const uint8_t* __restrict__ cell, double* xa,
                                                   double* xb, int dyn, const float* __restrict__ dprime,
                                                   const SolveState* __restrict__ st) {
@@ -583,16 +593,14 @@ __global__ void __launch_bounds__(256) k_update64(size_t n, const uint8_t* __res
   const double sig = st->sigma;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
     const bool fl = cell == nullptr || cell[i] != 0;
-    xout[i] = fl ? fma(sig, (double)dprime[i], xin[i]) : 0.0;
+    xout[i] = fl ? fma(sig, widen(dprime[i]), xin[i]) : 0.0;
   }
 }
 
-// UNIT: every axis weight is exactly 1 (equal spacings in the scaled units
-// c = h_0x^2), so the neighbour sum needs no products.  The diagonal d =
-// sum_a w_a k_a comes from a 64-entry float64 table by link counts
-// (kx + 4 ky + 16 kz).  A thread whose cells and neighbours all hold 0 (a
-// zero guess) has A' x = 0 exactly and forms only r = c b.
-template <int DIM, bool MASKED, bool UPDATE, bool UNIT>
+// Residual in float64 for any axis weights.  The diagonal d = sum_a w_a k_a
+// comes from a 64-entry float64 table by link counts (kx + 4 ky + 16 kz).
+// Bound by the float64 pipe (ten float64 operations per 3D cell).
+template <int DIM, bool MASKED, bool UPDATE>
 __global__ void __launch_bounds__(256) k_outer64(LevelDev L, double w0, double w1, double w2, double c, double c2,
                                                  const float* __restrict__ b, double* xa, double* xb, int dyn,
                                                  float* __restrict__ rprime, SolveState* __restrict__ st,
@@ -630,17 +638,6 @@ __global__ void __launch_bounds__(256) k_outer64(LevelDev L, double w0, double w
         zf[k] = ok && n.hf ? x[n.iF + k] : 0.0;
       }
     }
-    // any nonzero value among them (integer test of the bits, sign ignored)
-    unsigned long long nz = 0ull;
-#pragma unroll
-    for (int k = 0; k < 6; ++k) nz |= (unsigned long long)__double_as_longlong(xc[k]);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      nz |= (unsigned long long)__double_as_longlong(yu[k]) | (unsigned long long)__double_as_longlong(yd[k]);
-      if (DIM == 3)
-        nz |= (unsigned long long)__double_as_longlong(zb[k]) | (unsigned long long)__double_as_longlong(zf[k]);
-    }
-    const bool zero = (nz & 0x7fffffffffffffffull) == 0ull;
     float bv[4];
     ld4(b, n.i, x0, L.nx, bv);
     uint8_t m[4];
@@ -650,30 +647,19 @@ __global__ void __launch_bounds__(256) k_outer64(LevelDev L, double w0, double w
     for (int k = 0; k < 4; ++k) {
       rv[k] = 0.f;
       if (!m[k]) continue;
-      double r;
-      if (zero) {
-        r = c * (double)bv[k];
+      int q;
+      if (MASKED) {
+        q = m[k] & 63;
       } else {
-        int q;
-        if (MASKED) {
-          q = m[k] & 63;
-        } else {
-          q = axis_count(x0 + k, L.nx, L.bcD, 0) + 4 * axis_count(y, L.ny, L.bcD, 2);
-          if (DIM == 3) q += 16 * axis_count(zz, L.nz, L.bcD, 4);
-        }
-        // A' x = d x_c - sum_a w_a (x_minus + x_plus); a missing link or
-        // solid neighbour holds 0
-        double sn;
-        if (UNIT) {
-          sn = (xc[k] + xc[k + 2]) + (yu[k] + yd[k]);
-          if (DIM == 3) sn += zb[k] + zf[k];
-        } else {
-          sn = w0 * (xc[k] + xc[k + 2]);
-          sn = fma(w1, yu[k] + yd[k], sn);
-          if (DIM == 3) sn = fma(w2, zb[k] + zf[k], sn);
-        }
-        r = fma(c, (double)bv[k], fma(-dtab[q], xc[k + 1], sn));
+        q = axis_count(x0 + k, L.nx, L.bcD, 0) + 4 * axis_count(y, L.ny, L.bcD, 2);
+        if (DIM == 3) q += 16 * axis_count(zz, L.nz, L.bcD, 4);
       }
+      // A' x = d x_c - sum_a w_a (x_minus + x_plus); a missing link or
+      // solid neighbour holds 0
+      double sn = w0 * (xc[k] + xc[k + 2]);
+      sn = fma(w1, yu[k] + yd[k], sn);
+      if (DIM == 3) sn = fma(w2, zb[k] + zf[k], sn);
+      const double r = fma(c, (double)bv[k], fma(-dtab[q], xc[k + 1], sn));
       rv[k] = (float)r * inv_sig_new;
       acc = fma(r, r, acc);
     }
@@ -683,6 +669,166 @@ __global__ void __launch_bounds__(256) k_outer64(LevelDev L, double w0, double w
   if (grid_sum_last(acc, partials, &st->counter[kCntOuter], &tot)) {
     if (threadIdx.x == 0) {
       outer_decide(st, tot, c2, sig_new, UPDATE);
+      if (UPDATE && dyn) st->cur ^= 1;
+    }
+  }
+}
+
+// Equal axis weights (all 1 in the scaled units c = h_0x^2): the residual of
+// the float64 iterate, its last sums in 64-bit fixed point.  The neighbours
+// in y and z are added in float64 (one or three operations per cell, which
+// run beside the integer ones); that sum, the cells of the row and c b take
+// the largest exponent among the thread's four cells: each becomes an integer
+// of magnitude below 2^59 (the largest keeps six bits beyond its 53), c b as
+// the exact 77-bit product of the significands cut to 59 bits, and the
+// products with the link counts and the rest of the sum are exact integer
+// arithmetic.  The cut-off parts are below 2^-59 of the largest value, where
+// a float64 sum rounds at 2^-53.  The result is normalised and rounded to
+// float32 once; ||r|| is summed from r' in float-float.
+__device__ __forceinline__ unsigned magnitude(double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; }
+
+__device__ __forceinline__ long long fix_of(double v, int emax) {
+  const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+  const int e = (int)((hi >> 20) & 0x7ffu);
+  unsigned long long t = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32 | lo) << 6;
+  t >>= min(emax - e, 63);  // 0 for a zero: emax >= 128 where this is used
+  const long long s = (long long)((int)hi >> 31);
+  return ((long long)t ^ s) - s;
+}
+
+// c b: significand product cut to 59 bits, exponent `e` on fix_of's scale.
+struct FixC {
+  unsigned mhi, mlo;  // c's significand
+  int e;              // c's exponent field less 126
+};
+
+__device__ __forceinline__ long long fix_cb(FixC c, float b, int emax) {
+  const unsigned u = __float_as_uint(b), m = (u & 0x7fffffu) | 0x800000u;
+  const int eb = (int)((u >> 23) & 255u);
+  unsigned long long t = ((unsigned long long)m * c.mhi << 14) + ((unsigned long long)m * c.mlo >> 18);
+  t >>= min(emax - (eb + c.e), 63);
+  if (eb == 0) t = 0;  // zero (a denormal b has ||b||^2 = 0 in float32)
+  const long long s = (long long)((int)u >> 31);
+  return ((long long)t ^ s) - s;
+}
+
+// v 2^(emax - 1081) as float32.
+__device__ __forceinline__ float fix_float(long long v, int emax) {
+  const unsigned long long a = (unsigned long long)(v < 0 ? -v : v);
+  const int z = __clzll((long long)a);
+  const unsigned top = (unsigned)((a << (z & 63)) >> 32);
+  // top 2^(32 - z) 2^(emax - 1081), in two factors that are float32 numbers
+  const int s = emax - 1049 - z, s1 = s >> 1, s2 = s - s1;
+  const float f1 = __int_as_float((max(-126, min(127, s1)) + 127) << 23);
+  const float f2 = __int_as_float((max(-126, min(127, s2)) + 127) << 23);
+  const float r = a ? (float)top * f1 * f2 : 0.f;
+  return v < 0 ? -r : r;
+}
+
+template <bool VEC>
+__device__ __forceinline__ void row64(const double* __restrict__ x, size_t i, int x0, int nx, bool on,
+                                      double (&v)[4]) {
+  if (VEC) {
+    double2 p = make_double2(0.0, 0.0), q = p;
+    if (on) {
+      p = *reinterpret_cast<const double2*>(x + i);
+      q = *reinterpret_cast<const double2*>(x + i + 2);
+    }
+    v[0] = p.x;
+    v[1] = p.y;
+    v[2] = q.x;
+    v[3] = q.y;
+  } else {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = on && x0 + k < nx ? x[i + k] : 0.0;
+  }
+}
+
+template <int DIM, bool MASKED, bool UPDATE, bool VEC>
+__global__ void __launch_bounds__(256, DIM == 3 ? 2 : 3) k_outer_fix(LevelDev L, FixC c, double c2, const float* __restrict__ b,
+                                                   double* xa, double* xb, int dyn, float* __restrict__ rprime,
+                                                   SolveState* __restrict__ st, double* __restrict__ partials) {
+  const bool swap = dyn && st->cur;
+  const double* __restrict__ x = (swap != UPDATE) ? xb : xa;
+  const double sig_old = st->sigma;
+  double sig_new = sig_old;
+  if (UPDATE) sig_new = pow2_floor(sig_old * sqrt(fmax(st->rnorm2, 1e-300) / (double)st->n_fluid));
+  const float inv_sig_new = (float)(1.0 / sig_new);
+  float2 acc = make_float2(0.f, 0.f);
+  for (RowIter it(L); it.more(); it.next(L)) {
+    if (!it.active) continue;
+    const int x0 = it.x0, y = it.y, zz = it.z;
+    const Nbr n = neighbours<DIM>(L, x0, y, zz);
+    double xc[4], yu[4], yd[4];
+    row64<VEC>(x, n.i, x0, L.nx, true, xc);
+    row64<VEC>(x, n.iu, x0, L.nx, n.hu, yu);
+    row64<VEC>(x, n.id, x0, L.nx, n.hd, yd);
+    const double xl = n.hl ? x[n.il] : 0.0, xr = n.hr ? x[n.ir] : 0.0;
+    if (DIM == 3) {
+      double zb[4], zf[4];
+      row64<VEC>(x, n.ib, x0, L.nx, n.hb, zb);
+      row64<VEC>(x, n.iF, x0, L.nx, n.hf, zf);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) yu[k] = (yu[k] + yd[k]) + (zb[k] + zf[k]);
+    } else {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) yu[k] = yu[k] + yd[k];
+    }
+    float bv[4];
+    ld4(b, n.i, x0, L.nx, bv);
+    uint8_t m[4];
+    cells4<MASKED>(L, n.i, x0, m);
+    // the common exponent
+    unsigned top = max(magnitude(xl), magnitude(xr));
+    int emax = 0;
+    bool odd = false;  // an infinity or NaN in b
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      top = max(top, max(magnitude(xc[k]), magnitude(yu[k])));
+      const int eb = (int)((__float_as_uint(bv[k]) >> 23) & 255u);
+      odd = odd || (m[k] && eb == 255);
+      if (m[k] && eb) emax = max(emax, eb + c.e);
+    }
+    emax = max(emax, (int)(top >> 20));
+    odd = odd || emax >= 0x7ff;
+    float rv[4];
+    if (odd || emax < 128) {
+      // non-finite: the solve ends as diverged; below 2^-894: 0 in float32
+#pragma unroll
+      for (int k = 0; k < 4; ++k) rv[k] = odd && m[k] ? __int_as_float(0x7fc00000) : 0.f;
+    } else {
+      long long X[6];  // x0-1 .. x0+4
+      X[0] = fix_of(xl, emax);
+      X[5] = fix_of(xr, emax);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) X[k + 1] = fix_of(xc[k], emax);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        int q;
+        if (MASKED) {
+          q = (m[k] & 3) + ((m[k] >> 2) & 3) + ((m[k] >> 4) & 3);
+        } else {
+          q = axis_count(x0 + k, L.nx, L.bcD, 0) + axis_count(y, L.ny, L.bcD, 2);
+          if (DIM == 3) q += axis_count(zz, L.nz, L.bcD, 4);
+        }
+        // a missing link or solid neighbour holds 0; at most ten terms below
+        // 2^59
+        const long long s =
+            fix_cb(c, m[k] ? bv[k] : 0.f, emax) - q * X[k + 1] + X[k] + X[k + 2] + fix_of(yu[k], emax);
+        rv[k] = m[k] ? fix_float(s, emax) * inv_sig_new : 0.f;
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float p = rv[k] * rv[k];
+      acc = pair_add(acc, make_float2(p, fmaf(rv[k], rv[k], -p)));
+    }
+    st4(rprime, n.i, x0, L.nx, rv);
+  }
+  double tot;
+  if (grid_sum_last(acc, partials, &st->counter[kCntOuter], &tot)) {
+    if (threadIdx.x == 0) {
+      outer_decide(st, tot * sig_new * sig_new, c2, sig_new, UPDATE);
       if (UPDATE && dyn) st->cur ^= 1;
     }
   }
@@ -712,14 +858,16 @@ cudaError_t launch_outer(const LevelDev& L, const double w[3], double c, const f
                                                                      (double*)xin, (double*)xout, dyn,
                                                                      (const float*)dprime, st);
     }
-    if (w[0] == 1.0 && w[1] == 1.0 && (DIM == 2 || w[2] == 1.0))
-      k_outer64<DIM, MASKED, UPDATE, true><<<row_grid(L), 256, 0, s>>>(L, w[0], w[1], w[2], c, c * c, b,
-                                                                       (double*)xin, (double*)xout, dyn,
-                                                                       (float*)rprime, st, partials);
-    else
-      k_outer64<DIM, MASKED, UPDATE, false><<<row_grid(L), 256, 0, s>>>(L, w[0], w[1], w[2], c, c * c, b,
-                                                                        (double*)xin, (double*)xout, dyn,
-                                                                        (float*)rprime, st, partials);
+    if (w[0] == 1.0 && w[1] == 1.0 && (DIM == 2 || w[2] == 1.0) && isnormal(c)) {
+      uint64_t u;
+      memcpy(&u, &c, 8);
+      const FixC fc = {(unsigned)((u >> 32) & 0xfffffu) | 0x100000u, (unsigned)u, (int)((u >> 52) & 0x7ffu) - 126};
+      const auto k = (L.nx & 3) == 0 ? k_outer_fix<DIM, MASKED, UPDATE, true> : k_outer_fix<DIM, MASKED, UPDATE, false>;
+      k<<<row_grid(L), 256, 0, s>>>(L, fc, c * c, b, (double*)xin, (double*)xout, dyn, (float*)rprime, st, partials);
+    } else {
+      k_outer64<DIM, MASKED, UPDATE><<<row_grid(L), 256, 0, s>>>(L, w[0], w[1], w[2], c, c * c, b, (double*)xin,
+                                                                 (double*)xout, dyn, (float*)rprime, st, partials);
+    }
     return cudaGetLastError();
   }
   k_outer<DIM, T, MASKED, UPDATE><<<row_grid(L), 256, 0, s>>>(L, outer_args(w, c), b, (float2*)xin, (float2*)xout,

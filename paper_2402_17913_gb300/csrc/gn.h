@@ -27,9 +27,8 @@ constexpr int kLayers = 9;
 constexpr int kWElems = kTaps * kC * kC;  // 6912 FP32 weights per (padded) layer
 constexpr int kPackBytes = kTaps * 512;   // one packed BF16 operand set per layer
 
-// Forward / data-gradient convolution tile: M = 16 x 8 voxels per MMA, kTZ
-// z-planes per CTA iteration.
-constexpr int kTX = 16, kTY = 8, kTZ = 2;
+// Forward / data-gradient convolution tile: M = 8 x 16 voxels per MMA.
+constexpr int kTX = 8, kTY = 16;
 // Weight-gradient tile.
 constexpr int kWTX = 16, kWTY = 8, kWTZ = 4;
 

@@ -4,24 +4,35 @@
 // memory-bound glue (pooling, upsampling, skip sums, ReLU masks, input
 // scaling, loss, Adam).
 //
-// Convolution as a GEMM.  For an output tile of M = 128 voxels (16 along x,
-// 8 along y, one z-plane) the 3x3x3 correlation with 16 input and 16 output
-// channels is 27 MMAs of shape M x N x K = 128 x 16 x 16, one per tap t:
-//     D[v][co] += sum_ci X[v + o_t][ci] * W[t][ci][co].
-// A block walks a run of z-planes of one 16 x 8 column.  It keeps, for
-// each of three copies of the input (x shifted by dx = -1, 0, +1, with a
-// one-voxel halo in y), a ring of four z-planes fetched by TMA as rows of
-// one voxel's 16 channels (32 bytes) in the 32-byte-swizzled K-major layout
-// that the tensor core reads directly; each step of two output planes
-// fetches only the two planes it adds.  The A operand of tap (dz, dy, dx)
-// is then a contiguous 4 KB run of copy dx starting at line dy + 1 of the
-// ring slot holding plane z + dz: descriptors differ only in their start
-// address (a multiple of 256 bytes, so the swizzle phase never shifts) and
-// take two values per tap as the ring turns; out-of-range voxels arrive as
-// zeros (the zero padding).  Lane 0 of warp zi issues the 27 MMAs of output
-// plane zi into its TMEM accumulator (128 lanes x 16 FP32 columns), then,
-// once they are done, the next fetch; the four warps read the accumulator back with
-// tcgen05.ld, apply the epilogue and store 32 bytes per voxel.
+// Convolution as a GEMM.  For an output tile of M = 128 voxels (8 along x, 16
+// along y, one z-plane) the 3x3x3 correlation with 16 input and 16 output
+// channels is D[v][co] += sum_ci X[v + o_t][ci] * W[t][ci][co] over 27 taps t.
+// A block walks a run of z-planes of one 8 x 16 column.  Input plane z adds
+// to the output planes z - 1, z and z + 1 through the same nine shifted views
+// (dy, dx), so one MMA of shape 128 x 48 x 16 does the three dz taps of a
+// view: their accumulators are three slots of 16 TMEM columns, output plane p
+// in slot p mod 3, and the 48 columns of B hold the taps dz in the cyclic
+// order that puts each under its slot (a window of three in the stored
+// sequence +1, 0, -1, +1, 0).  An input plane takes 9 MMAs instead of 27, and
+// each view is read from shared memory once instead of three times, which is
+// what bounds a 128 x 16 x 16 MMA (its 4 KB A tile at 128 bytes per SM cycle
+// takes 32 cycles, its arithmetic about 9); an output's 27 taps still add up
+// in the order of t.  After plane z the slot of output z - 1 is complete: the
+// four warps read it with tcgen05.ld, write zeros to it for output z + 2, and
+// apply the epilogue and store 32 bytes per voxel while the next plane's MMAs
+// run.
+//
+// A plane with its one-voxel halo in x and y is copied once, two planes ahead,
+// by 16-byte cp.async into [channel half][y][x][8 channels]: eight voxels of a
+// line are then a 128-byte core matrix of the unswizzled K-major layout from
+// any x on, so the A operands of all nine views are descriptors into the same
+// copy (start address + 160 bytes per dy, + 16 per dx).  (Tiled TMA needs a
+// copy per dx, swizzled, and moves it as 432 rows of 32 bytes per plane, which
+// bound the layer at 62 us.)  Out-of-range voxels are zero-filled (the zero
+// padding).  Measured on GB300, one 16 -> 16 layer of 8 x 64^3 voxels: 92 us with
+// 27 MMAs per plane, 47 us now (134 MB in and out: 20 us at the copy rate; 84
+// cycles per MMA on an SM with five blocks, against 44 for its operands at 128
+// bytes per cycle); 256 x 128 x 128 voxels 184 -> 86 us.
 
 // The data gradient is the same kernel with the mirrored, transposed taps
 // (W'[26 - t][co][ci] = W[t][ci][co]).  The weight gradient
@@ -45,24 +56,25 @@ namespace gn {
 
 namespace {
 
-constexpr int kPlaneZ = (kTY + 2) * kTX * 32;               // one z-plane of one copy: [y][x][16 ch]
-constexpr int kRing = kTZ + 2;                               // z-planes kept per copy
-constexpr int kCopy = kRing * kPlaneZ;
-constexpr int kDescOff = 13824;                              // descriptor table after the 13824-byte weights
-constexpr int kDescA = 2 * kTZ * kTaps;                      // A descriptors: [ring phase][zi][tap]
-constexpr int kAOff = 14592;                                 // copies start (256-aligned: the swizzle atom)
-constexpr int kConvSmem = kAOff + 3 * kCopy + 256;           // + alignment slack; 3 blocks fit an SM
+constexpr int kLine = (kTX + 2) * 16;                        // 8 channels of one line of voxels with halo
+constexpr int kHalf = (kTY + 2) * kLine;                     // one channel half of a plane
+constexpr int kStage = 2 * kHalf;
+constexpr int kStages = 3;                                   // planes in flight or in use
+constexpr int kChunks = kStage / 16;                         // 16-byte pieces of a plane
+constexpr int kBView = 2 * 5 * 256;                          // B of one (dy, dx): [K half][five dz blocks][2][128 B]
+constexpr int kBBytes = 9 * kBView;
+constexpr int kConvSmem = kBBytes + kStages * kStage;
 constexpr int kConvThreads = 128;
-constexpr uint32_t kConvCols = 32;                           // TMEM columns (kTZ accumulators of 16, min 32)
-static_assert(kTZ == 2, "the ring turns by two planes per step");
-static_assert(kTZ * 16 <= (int)kConvCols, "TMEM columns");
-static_assert(kPlaneZ % 256 == 0 && kAOff % 256 == 0, "swizzled TMA destinations stay 256-aligned");
-static_assert(kDescOff + 4 * (kDescA + kTaps) <= kAOff, "descriptor table fits");
+constexpr int kPer = (kChunks + kConvThreads - 1) / kConvThreads;
+constexpr uint32_t kConvCols = 64;                           // TMEM columns (three accumulators of 16, a power of two)
+static_assert(kTX == 8 && kTX * kTY == kConvThreads, "a line is a core matrix, one voxel per thread");
+static_assert(kBBytes % 128 == 0 && kStage % 128 == 0, "operands start on 128-byte boundaries");
 
 constexpr int kXTile = (kWTX + 2) * (kWTY + 2) * (kWTZ + 2) * 32;  // wgrad x tile with halo
 constexpr int kGTile = kWTX * kWTY * kWTZ * 32;
 constexpr int kWgSmem = kXTile + kGTile + 1024;
-constexpr int kWgThreads = 288;  // 9 warps: warp w owns taps 3w .. 3w+2 (dz, dy fixed, dx = -1, 0, 1)
+constexpr int kWgThreads = 288;  // 9 warps: warp w owns the taps of one (dy, dx), dz = -1, 0, 1
+static_assert(kWElems % 32 == 0, "whole blocks of the reduction");
 static_assert(kXTile % 256 == 0 && kGTile % 256 == 0, "swizzled TMA destinations stay 256-aligned");
 
 // byte offset of channel group g of voxel v in a 32-byte-swizzled tile
@@ -72,7 +84,7 @@ __device__ __forceinline__ uint32_t sw32(uint32_t v, uint32_t g) { return v * 32
 struct ConvArgs {
   int nx, ny, nz, nn;
   int tx, ty;
-  int zc, nzc;  // planes per z-run (a multiple of kTZ) and runs per column
+  int zc, nzc;  // planes per z-run and runs per column
   long long nitems;
   void* out;
   const __nv_bfloat16* mask;
@@ -95,20 +107,37 @@ __device__ __forceinline__ uint32_t pack_bf2(float a, float b) {
 
 __device__ __forceinline__ bool bf_pos(uint32_t h16) { return !(h16 & 0x8000u) && (h16 & 0x7fffu); }
 
+// 32 bytes to a 16-byte aligned address; one store (a whole sector) where the
+// address is 32-byte aligned.
+__device__ __forceinline__ void store32(void* p, const uint32_t (&q)[8]) {
+  if (((uintptr_t)p & 31) == 0) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(q[0]), "r"(q[1]), "r"(q[2]),
+                 "r"(q[3]), "r"(q[4]), "r"(q[5]), "r"(q[6]), "r"(q[7])
+                 : "memory");
+  } else {
+    uint4* o = static_cast<uint4*>(p);
+    o[0] = make_uint4(q[0], q[1], q[2], q[3]);
+    o[1] = make_uint4(q[4], q[5], q[6], q[7]);
+  }
+}
+
 template <int EPI>
-__device__ __forceinline__ void store_epi(const ConvArgs& a, size_t vox, int n, const float (&v)[16]) {
+__device__ __forceinline__ void store_epi(const ConvArgs& a, size_t vox, int n, const float (&v)[16],
+                                          const uint4 (&m)[2]) {
   if (EPI == kEpiF32) {
-    float4* o = reinterpret_cast<float4*>(static_cast<float*>(a.out) + vox * kC);
+    uint32_t q[8];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) o[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+    for (int h = 0; h < 2; ++h) {
+#pragma unroll
+      for (int k = 0; k < 8; ++k) q[k] = __float_as_uint(v[8 * h + k]);
+      store32(static_cast<float*>(a.out) + vox * kC + 8 * h, q);
+    }
   } else if (EPI == kEpiOut0) {
     static_cast<float*>(a.out)[vox] = v[0] * (a.scale ? a.scale[n] : 1.f);
   } else {
     float w[16];
     if (EPI == kEpiMask) {
-      const uint4* mp = reinterpret_cast<const uint4*>(a.mask + vox * kC);
-      const uint4 m0 = mp[0], m1 = mp[1];
-      const uint32_t mw[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
+      const uint32_t mw[8] = {m[0].x, m[0].y, m[0].z, m[0].w, m[1].x, m[1].y, m[1].z, m[1].w};
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
         w[2 * k] = bf_pos(mw[k] & 0xffffu) ? v[2 * k] : 0.f;
@@ -118,157 +147,184 @@ __device__ __forceinline__ void store_epi(const ConvArgs& a, size_t vox, int n, 
 #pragma unroll
       for (int k = 0; k < 16; ++k) w[k] = EPI == kEpiRelu ? fmaxf(v[k], 0.f) : v[k];
     }
-    uint4* o = reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(a.out) + vox * kC);
-    o[0] = make_uint4(pack_bf2(w[0], w[1]), pack_bf2(w[2], w[3]), pack_bf2(w[4], w[5]), pack_bf2(w[6], w[7]));
-    o[1] = make_uint4(pack_bf2(w[8], w[9]), pack_bf2(w[10], w[11]), pack_bf2(w[12], w[13]), pack_bf2(w[14], w[15]));
+    uint32_t q[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) q[k] = pack_bf2(w[2 * k], w[2 * k + 1]);
+    store32(static_cast<__nv_bfloat16*>(a.out) + vox * kC, q);
   }
 }
 
-// Persistent implicit-GEMM convolution (see the file comment).  map4 /
-// map2 fetch four / two z-planes of the three copies.
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool on) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(on ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// Persistent implicit-GEMM convolution (see the file comment).
 template <int EPI>
-__global__ void __launch_bounds__(kConvThreads) k_conv(const __grid_constant__ CUtensorMap map4,
-                                                     const __grid_constant__ CUtensorMap map2,
-                                                     const uint4* __restrict__ wpack, ConvArgs a) {
-  extern __shared__ unsigned char dsm[];
-  __shared__ __align__(8) uint64_t bar_ld;
+__global__ void __launch_bounds__(kConvThreads) k_conv(const unsigned char* __restrict__ xin,
+                                                     const unsigned char* __restrict__ wpack, ConvArgs a) {
+  extern __shared__ __align__(128) unsigned char dsm[];
   __shared__ __align__(8) uint64_t bar_mma;
   __shared__ uint32_t tmem_slot;
-  const uint32_t pad = (256u - (smem_u32(dsm) & 255u)) & 255u;
-  unsigned char* sW = dsm + pad;
-  uint32_t* sD = reinterpret_cast<uint32_t*>(sW + kDescOff);  // low words: [ph][zi][t] A, then [t] B
-  unsigned char* sA = sW + kAOff;
   const int tid = threadIdx.x, warp = tid >> 5;
-  const uint32_t sW_u = smem_u32(sW), sA_u = smem_u32(sA);
+  const uint32_t sB_u = smem_u32(dsm), sA_u = sB_u + kBBytes;
 
-  for (int i = tid; i < kPackBytes / 16; i += kConvThreads) reinterpret_cast<uint4*>(sW)[i] = wpack[i];
-  for (int i = tid; i < kDescA + kTaps; i += kConvThreads) {
-    if (i < kDescA) {
-      const int t = i % kTaps, zi = (i / kTaps) % kTZ, ph = i / (kTaps * kTZ);
-      const int dz = t / 9 - 1, dy = (t / 3) % 3 - 1, dx = t % 3 - 1;
-      const int slot = (2 * ph + zi + dz + 1) & (kRing - 1);
-      sD[i] = (uint32_t)smem_desc_sw32(sA_u + (uint32_t)((dx + 1) * kCopy + slot * kPlaneZ + (dy + 1) * kTX * 32),
-                                       256);
-    } else {
-      sD[i] = (uint32_t)smem_desc(sW_u + (uint32_t)((i - kDescA) * 512), 256, 128);
-    }
+  // B of view v = (dy + 1) 3 + dx + 1, K half h, block q = 0 .. 4 (dz = +1, 0,
+  // -1, +1, 0): the 256 bytes of packed tap (dz, v), half h
+  for (int i = tid; i < kBBytes / 16; i += kConvThreads) {
+    const int q = (i >> 4) % 5, h = (i / 80) & 1, v = i / 160;
+    const int dz1 = (2 - q + 3) % 3;  // dz + 1
+    cp_async16(sB_u + (uint32_t)i * 16u, wpack + (dz1 * 9 + v) * 512 + h * 256 + (i & 15) * 16, true);
   }
-  const uint32_t hiA = (uint32_t)(smem_desc_sw32(0, 256) >> 32), hiB = (uint32_t)(smem_desc(0, 256, 128) >> 32);
-  fence_proxy_async_smem();
+  const uint32_t hiA = (uint32_t)(smem_desc(0, kHalf, kLine) >> 32), hiB = (uint32_t)(smem_desc(0, 1280, 128) >> 32);
+  const uint32_t loA = (uint32_t)smem_desc(sA_u, kHalf, kLine), loB = (uint32_t)smem_desc(sB_u, 1280, 128);
   if (tid == 0) {
-    mbar_init(&bar_ld, 1);
-    mbar_init(&bar_mma, kTZ);  // one commit per issuing warp
+    mbar_init(&bar_mma, 1);
     fence_mbar_init();
   }
   if (warp == 0) {
     tmem_alloc(&tmem_slot, kConvCols);
     tmem_relinquish();
   }
+
+  // A step is one input plane of an item = (x tile, y tile, z run, sample):
+  // planes zr0 - 1 .. zr0 + count, `count` outputs.
+  struct Step {
+    long long item;
+    int x0, y0, zr0, n, count, i;
+  };
+  auto open = [&](Step& p) {
+    if (p.item >= a.nitems) return;
+    long long r = p.item;
+    p.x0 = (int)(r % a.tx) * kTX;
+    r /= a.tx;
+    p.y0 = (int)(r % a.ty) * kTY;
+    r /= a.ty;
+    p.zr0 = (int)(r % a.nzc) * a.zc;
+    p.n = (int)(r / a.nzc);
+    p.count = min(a.zc, a.nz - p.zr0);
+    p.i = 0;
+  };
+  Step cur, ahead;  // the plane in work and the next one to fetch
+  cur.item = blockIdx.x;
+  open(cur);
+  ahead = cur;
+  // this thread's pieces of a plane: shared offsets, and for the item being
+  // fetched the offsets in a plane (-1 outside it)
+  uint32_t so[kPer];
+  long long go[kPer];
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    const int c = tid + k * kConvThreads, r = c % (2 * (kTX + 2));
+    so[k] = (uint32_t)((r & 1) * kHalf + c / (2 * (kTX + 2)) * kLine + (r >> 1) * 16);
+  }
+  auto locate = [&]() {
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      const int c = tid + k * kConvThreads, r = c % (2 * (kTX + 2));
+      const int x = ahead.x0 - 1 + (r >> 1), y = ahead.y0 - 1 + c / (2 * (kTX + 2));
+      const bool in = x >= 0 && x < a.nx && y >= 0 && y < a.ny;
+      go[k] = in ? ((long long)y * a.nx + x) * 32 + (r & 1) * 16 : -1;
+    }
+  };
+  locate();
+  // copy the next plane into `stage` (an empty group when none is left)
+  auto fetch = [&](int stage) {
+    if (ahead.item < a.nitems) {
+      const int z = ahead.zr0 - 1 + ahead.i;
+      const bool zin = z >= 0 && z < a.nz;
+      const unsigned char* src = xin + ((size_t)ahead.n * a.nz + (zin ? z : 0)) * a.ny * a.nx * 32;
+#pragma unroll
+      for (int k = 0; k < kPer; ++k)
+        if (kChunks % kConvThreads == 0 || tid + k * kConvThreads < kChunks) {
+          const bool on = zin && go[k] >= 0;
+          cp_async16(sA_u + (uint32_t)(stage * kStage) + so[k], src + (on ? go[k] : 0), on);
+        }
+      if (++ahead.i >= ahead.count + 2) {
+        ahead.item += gridDim.x;
+        open(ahead);
+        locate();
+      }
+    }
+    cp_async_commit();
+  };
+#pragma unroll
+  for (int k = 0; k < kStages - 1; ++k) fetch(k);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = tmem_slot;
-  constexpr uint32_t idesc = idesc_bf16(128, 16);
+  const uint32_t tmem = tmem_slot, lanes = (uint32_t)(warp * 32) << 16;
+  constexpr uint32_t idesc = idesc_bf16(128, 48);
+  tmem_zero16(tmem + lanes);  // slot 0, the first output's
+  cp_async_wait<kStages - 2>();
+  fence_proxy_async_smem();
+  tc_fence_before();
+  __syncthreads();
 
-  // item = (x tile, y tile, z run, sample)
-  auto origin = [&](long long item, int& x0, int& y0, int& zr0, int& n) {
-    long long r = item;
-    x0 = (int)(r % a.tx) * kTX;
-    r /= a.tx;
-    y0 = (int)(r % a.ty) * kTY;
-    r /= a.ty;
-    zr0 = (int)(r % a.nzc) * a.zc;
-    n = (int)(r / a.nzc);
-  };
-  // four planes z0 - 1 .. z0 + 2 (ring slots 0..3) or the two planes z0 + 1,
-  // z0 + 2 of the tile starting at z0 (ring slots `slot`, `slot` + 1)
-  auto fetch = [&](bool full, int x0, int y0, int z0, int n, int slot) {
-    mbar_arrive_expect_tx(&bar_ld, (full ? kRing : 2) * 3 * kPlaneZ);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      if (full)
-        tma_load_5d(sA + c * kCopy, &map4, &bar_ld, 0, x0 + c - 1, y0 - 1, z0 - 1, n);
-      else
-        tma_load_5d(sA + c * kCopy + slot * kPlaneZ, &map2, &bar_ld, 0, x0 + c - 1, y0 - 1, z0 + 1, n);
-    }
-  };
-
-  uint32_t phase = 0;
-  long long item = blockIdx.x;
-  bool pending = false;
-  if (tid == 0 && item < a.nitems) {
-    int x0, y0, zr0, n;
-    origin(item, x0, y0, zr0, n);
-    fetch(true, x0, y0, zr0, n, 0);
-  }
-  pending = item < a.nitems;
-  bool stop = false;
-  for (; item < a.nitems && !stop; item += gridDim.x) {
-    int x0, y0, zr0, n;
-    origin(item, x0, y0, zr0, n);
-    const int zend = min(zr0 + a.zc, a.nz);
-    for (int z0 = zr0, j = 0; z0 < zend; z0 += kTZ, ++j) {
-      const int ph = j & 1;
-      const bool ok_ld = mbar_wait_bounded(&bar_ld, phase);
-      if (__syncthreads_or(!ok_ld)) {
-        // a tile that never lands: report it, give the copy in flight a
-        // bounded wait, and stop (no MMA reads it)
-        if (tid == 0) atomicExch(a.err, 1);
-        mbar_wait_bounded(&bar_ld, phase);
-        pending = false;
-        stop = true;
-        break;
-      }
-      pending = false;
-      // lane 0 of warp zi issues the 27 MMAs of output plane zi (its own
-      // accumulator columns) and commits them
-      if (warp < kTZ && (tid & 31) == 0) {
-        tc_fence_after();
-        const int zi = warp;
-        const uint32_t* dA = sD + (ph * kTZ + zi) * kTaps;
-#pragma unroll
-        for (int t = 0; t < kTaps; ++t)
-          umma_bf16(tmem + (uint32_t)(zi * 16), ((uint64_t)hiA << 32) | dA[t],
-                    ((uint64_t)hiB << 32) | sD[kDescA + t], idesc, t > 0 ? 1u : 0u);
-        umma_commit(&bar_mma);
-      }
-      const bool ok_mma = mbar_wait_bounded(&bar_mma, phase);
-      if (__syncthreads_or(!ok_mma)) {
-        if (tid == 0) atomicExch(a.err, 2);
-        mbar_wait_bounded(&bar_mma, phase);
-        stop = true;
-        break;
-      }
+  int stage = 0, slot = 0;  // step mod kStages, step mod 3
+  uint32_t ph_mma = 0;
+  float v[16];
+  uint4 msk[2];  // the output's mask, on its way while the next plane is set up
+  size_t vox = 0;
+  int vn = 0;
+  bool have = false;
+  while (cur.item < a.nitems) {
+    if (tid == 0) {
       tc_fence_after();
-      // the planes this tile alone needed are free: fetch the next ones
-      // (the next tile of this run, else the first tile of the next item)
-      if (z0 + kTZ < zend) {
-        if (tid == 0) fetch(false, x0, y0, z0 + kTZ, n, (2 * (ph ^ 1) + 2) & (kRing - 1));
-        pending = true;
-      } else if (item + gridDim.x < a.nitems) {
-        int x1, y1, zr1, n1;
-        origin(item + gridDim.x, x1, y1, zr1, n1);
-        if (tid == 0) fetch(true, x1, y1, zr1, n1, 0);
-        pending = true;
-      }
-      const int row = tid;  // TMEM lane = M row = thread (warp w reads lanes 32w .. 32w + 31)
-      const int x = x0 + (row & 15), y = y0 + (row >> 4);
+      const uint32_t dA = loA + (uint32_t)(stage * kStage >> 4), dB = loB + (uint32_t)((2 - slot) * 256 >> 4);
 #pragma unroll
-      for (int zi = 0; zi < kTZ; ++zi) {
-        float v[16];
-        tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(zi * 16), v);
-        const int z = z0 + zi;
-        if (x < a.nx && y < a.ny && z < a.nz)
-          store_epi<EPI>(a, (((size_t)n * a.nz + z) * a.ny + y) * a.nx + x, n, v);
-      }
-      tc_fence_before();
-      __syncthreads();
-      phase ^= 1;
+      for (int t = 0; t < 9; ++t)
+        umma_bf16(tmem, ((uint64_t)hiA << 32) | (dA + (uint32_t)((t / 3 * kLine + t % 3 * 16) >> 4)),
+                  ((uint64_t)hiB << 32) | (dB + (uint32_t)(t * kBView >> 4)), idesc, 1u);
+      umma_commit(&bar_mma);
     }
+    // while the tensor core works: the plane kStages - 1 ahead into the stage
+    // of the previous one, and the previous plane's output
+    fetch(stage == 0 ? kStages - 1 : stage - 1);
+    if (have) store_epi<EPI>(a, vox, vn, v, msk);
+    const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&bar_mma, ph_mma));
+    const int done = slot == 2 ? 0 : slot + 1;
+    if (ok) {  // the whole warp
+      tc_fence_after();
+      // the slot of output i - 2 (its last tap was this plane's) is read and
+      // set to zero for the output that starts with the next plane
+      tmem_ld16(tmem + lanes + (uint32_t)(done * 16), v);
+      tmem_zero16(tmem + lanes + (uint32_t)(done * 16));
+    }
+    const int x = cur.x0 + (tid & (kTX - 1)), y = cur.y0 + tid / kTX, z = cur.zr0 + cur.i - 2;
+    have = ok && cur.i >= 2 && x < a.nx && y < a.ny;
+    vox = (((size_t)cur.n * a.nz + (have ? z : 0)) * a.ny + y) * a.nx + x;
+    vn = cur.n;
+    if (EPI == kEpiMask && have) {
+      msk[0] = __ldg(reinterpret_cast<const uint4*>(a.mask + vox * kC));
+      msk[1] = __ldg(reinterpret_cast<const uint4*>(a.mask + vox * kC) + 1);
+    }
+    cp_async_wait<kStages - 2>();  // the next plane has landed
+    fence_proxy_async_smem();
+    tc_fence_before();
+    if (__syncthreads_or(!ok)) {
+      // MMAs that never end: report it, give them one more bounded wait, stop
+      if (tid == 0) {
+        atomicExch(a.err, 2);
+        mbar_wait_bounded(&bar_mma, ph_mma);
+      }
+      have = false;
+      break;
+    }
+    if (++cur.i >= cur.count + 2) {
+      cur.item += gridDim.x;
+      open(cur);
+    }
+    slot = done;
+    ph_mma ^= 1u;
+    if (++stage == kStages) stage = 0;
   }
-  // a fetch still in flight after an early exit: bounded wait before the
-  // block's shared memory goes away
-  if (pending) mbar_wait_bounded(&bar_ld, phase ^ 1);
+  if (have) store_epi<EPI>(a, vox, vn, v, msk);
+  cp_async_wait<0>();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -277,8 +333,13 @@ __global__ void __launch_bounds__(kConvThreads) k_conv(const __grid_constant__ C
 
 // Weight gradient: per-block partial sums of dW over the block's tiles.
 // Staged (32-byte swizzled): x as [z][y][18][16 ch] covering x0 - 1 ..
-// x0 + 16, g as [z][y][16][16 ch].
-__global__ void __launch_bounds__(kWgThreads) k_wgrad(const __grid_constant__ CUtensorMap xmap,
+// x0 + 16, g as [z][y][16][16 ch].  Bound by the shared-memory fragment loads:
+// a warp keeps one (dy, dx) and walks a column of lines along z, so that one
+// fragment of x serves the three dz taps (against the g fragments of the
+// planes around it) and a tile's column takes 10 loads for 24 MMAs instead
+// of 16 (a warp per (dz, dy) with a load of x per dx): 8 x 64^3 voxels
+// 96 -> 76 us.
+__global__ void __launch_bounds__(kWgThreads, 4) k_wgrad(const __grid_constant__ CUtensorMap xmap,
                                                     const __grid_constant__ CUtensorMap gmap, WgArgs a) {
   extern __shared__ unsigned char dsm[];
   __shared__ __align__(8) uint64_t bar;
@@ -287,7 +348,7 @@ __global__ void __launch_bounds__(kWgThreads) k_wgrad(const __grid_constant__ CU
   unsigned char* sG = sX + kXTile;
   const uint32_t sX_u = smem_u32(sX), sG_u = smem_u32(sG);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int dz = warp / 3 - 1, dy = warp % 3 - 1;
+  const int dy = warp / 3 - 1, dx = warp % 3 - 1;
   if (tid == 0) {
     mbar_init(&bar, 1);
     fence_mbar_init();
@@ -327,18 +388,23 @@ __global__ void __launch_bounds__(kWgThreads) k_wgrad(const __grid_constant__ CU
       mbar_wait_bounded(&bar, phase);
       break;
     }
-#pragma unroll 2
-    for (int line = 0; line < kWTY * kWTZ; ++line) {
-      const int yi = line % kWTY, zi = line / kWTY;
-      uint32_t b[4];
-      ldsm_x4_trans(sG_u + sw32((uint32_t)((zi * kWTY + yi) * kWTX) + gk, gg), b);
-      const uint32_t xl = (uint32_t)(((zi + dz + 1) * (kWTY + 2) + (yi + dy + 1)) * (kWTX + 2));
+    for (int yi = 0; yi < kWTY; ++yi) {
+      uint32_t b[kWTZ][4];
 #pragma unroll
-      for (int j = 0; j < 3; ++j) {
+      for (int zi = 0; zi < kWTZ; ++zi)
+        ldsm_x4_trans(sG_u + sw32((uint32_t)((zi * kWTY + yi) * kWTX) + gk, gg), b[zi]);
+      const uint32_t xl = (uint32_t)((yi + dy + 1) * (kWTX + 2) + dx + 1) + xk;
+#pragma unroll
+      for (int p = 0; p < kWTZ + 2; ++p) {  // x plane z0 - 1 + p = g plane zi + dz
         uint32_t av[4];
-        ldsm_x4_trans(sX_u + sw32(xl + xk + (uint32_t)j, xg), av);
-        mma_16816(acc[j][0], av, b[0], b[1]);
-        mma_16816(acc[j][1], av, b[2], b[3]);
+        ldsm_x4_trans(sX_u + sw32(xl + (uint32_t)(p * (kWTY + 2) * (kWTX + 2)), xg), av);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+          const int zi = p - j;  // dz = j - 1
+          if (zi < 0 || zi >= kWTZ) continue;
+          mma_16816(acc[j][0], av, b[zi][0], b[zi][1]);
+          mma_16816(acc[j][1], av, b[zi][2], b[zi][3]);
+        }
       }
     }
     __syncthreads();
@@ -349,7 +415,7 @@ __global__ void __launch_bounds__(kWgThreads) k_wgrad(const __grid_constant__ CU
   const int g = lane >> 2, c2 = (lane & 3) * 2;
 #pragma unroll
   for (int j = 0; j < 3; ++j) {
-    const int t = 3 * warp + j;
+    const int t = 9 * j + warp;
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
       const int co = q * 8 + c2;
@@ -359,12 +425,31 @@ __global__ void __launch_bounds__(kWgThreads) k_wgrad(const __grid_constant__ CU
   }
 }
 
-__global__ void k_wgrad_reduce(const float* __restrict__ partials, int nblocks, float* __restrict__ dw, float scale,
-                               int accumulate) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= kWElems) return;
+// dw (+)= scale * the sum of the blocks' partials: a block of 256 threads sums
+// 32 elements, eight threads each taking every eighth block's partial with
+// sixteen loads in flight, their sums added in order (608 blocks, 16.8 MB: one
+// thread per element walked its 608 partials in 21 us, now 6.6 us).
+__global__ void __launch_bounds__(256) k_wgrad_reduce(const float* __restrict__ partials, int nblocks,
+                                                      float* __restrict__ dw, float scale, int accumulate) {
+  __shared__ float sh[8][32];
+  const int e = blockIdx.x * 32 + (threadIdx.x & 31), c = threadIdx.x >> 5;
+  const float* __restrict__ p = partials + e;
   float s = 0.f;
-  for (int b = 0; b < nblocks; ++b) s += partials[(size_t)b * kWElems + e];
+  int b = c;
+  for (; b + 8 * 15 < nblocks; b += 8 * 16) {
+    float v[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) v[k] = __ldg(p + (size_t)(b + 8 * k) * kWElems);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) s += v[k];
+  }
+  for (; b < nblocks; b += 8) s += __ldg(p + (size_t)b * kWElems);
+  sh[c][threadIdx.x & 31] = s;
+  __syncthreads();
+  if (threadIdx.x >= 32) return;
+  s = 0.f;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) s += sh[k][threadIdx.x];
   dw[e] = (accumulate ? dw[e] : 0.f) + scale * s;
 }
 
@@ -391,6 +476,17 @@ __device__ __forceinline__ void mask8(uint4 act, float (&f)[8]) {
   }
 }
 
+// Element counts below 2^31 (every grid-stride index then fits 32 bits) use
+// 32-bit index arithmetic: the 64-bit divisions by the extents bound these
+// kernels, which otherwise stream (residual loss of 8 x 64^3 voxels 50 -> 19 us,
+// with its neighbours loaded before use; skip sums 17.4 -> 13.7 us).
+static bool idx32(size_t total) { return total < (size_t)1 << 31; }
+#define GN_INDEXED(total, K, grid, block, s, ...)                        \
+  do {                                                                   \
+    if (idx32(total)) K<unsigned><<<grid, block, 0, s>>>(__VA_ARGS__);   \
+    else K<size_t><<<grid, block, 0, s>>>(__VA_ARGS__);                  \
+  } while (0)
+
 // index helpers: element (n, z, y, x, group) of a level with dims (nx, ny, nz)
 struct Lv {
   int nx, ny, nz;
@@ -399,16 +495,17 @@ struct Lv {
   }
 };
 
+template <typename I>
 __global__ void k_pool(const uint4* __restrict__ fine, uint4* __restrict__ coarse, Lv F, Lv Cc, size_t total) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
+  for (I i = blockIdx.x * (I)blockDim.x + threadIdx.x; i < (I)total; i += (I)(gridDim.x * blockDim.x)) {
     const int g = (int)(i & 1);
-    size_t v = i >> 1;
-    const int x = (int)(v % Cc.nx);
-    v /= Cc.nx;
-    const int y = (int)(v % Cc.ny);
-    v /= Cc.ny;
-    const int z = (int)(v % Cc.nz);
-    const size_t n = v / Cc.nz;
+    I v = i >> 1;
+    const int x = (int)(v % (I)Cc.nx);
+    v /= (I)Cc.nx;
+    const int y = (int)(v % (I)Cc.ny);
+    v /= (I)Cc.ny;
+    const int z = (int)(v % (I)Cc.nz);
+    const I n = v / (I)Cc.nz;
     float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
@@ -423,17 +520,18 @@ __global__ void k_pool(const uint4* __restrict__ fine, uint4* __restrict__ coars
   }
 }
 
+template <typename I>
 __global__ void k_up_add(const uint4* __restrict__ coarse, const uint4* __restrict__ fine, uint4* __restrict__ out,
                          Lv F, Lv Cc, size_t total) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
+  for (I i = blockIdx.x * (I)blockDim.x + threadIdx.x; i < (I)total; i += (I)(gridDim.x * blockDim.x)) {
     const int g = (int)(i & 1);
-    size_t v = i >> 1;
-    const int x = (int)(v % F.nx);
-    v /= F.nx;
-    const int y = (int)(v % F.ny);
-    v /= F.ny;
-    const int z = (int)(v % F.nz);
-    const size_t n = v / F.nz;
+    I v = i >> 1;
+    const int x = (int)(v % (I)F.nx);
+    v /= (I)F.nx;
+    const int y = (int)(v % (I)F.ny);
+    v /= (I)F.ny;
+    const int z = (int)(v % (I)F.nz);
+    const I n = v / (I)F.nz;
     float a[8], b[8];
     unpack8(coarse[Cc.u4(n, z >> 1, y >> 1, x >> 1, g)], a);
     unpack8(fine[i], b);
@@ -443,17 +541,18 @@ __global__ void k_up_add(const uint4* __restrict__ coarse, const uint4* __restri
   }
 }
 
+template <typename I>
 __global__ void k_upbwd_mask(const uint4* __restrict__ gfine, const uint4* __restrict__ act, uint4* __restrict__ out,
                              Lv F, Lv Cc, size_t total) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
+  for (I i = blockIdx.x * (I)blockDim.x + threadIdx.x; i < (I)total; i += (I)(gridDim.x * blockDim.x)) {
     const int g = (int)(i & 1);
-    size_t v = i >> 1;
-    const int x = (int)(v % Cc.nx);
-    v /= Cc.nx;
-    const int y = (int)(v % Cc.ny);
-    v /= Cc.ny;
-    const int z = (int)(v % Cc.nz);
-    const size_t n = v / Cc.nz;
+    I v = i >> 1;
+    const int x = (int)(v % (I)Cc.nx);
+    v /= (I)Cc.nx;
+    const int y = (int)(v % (I)Cc.ny);
+    v /= (I)Cc.ny;
+    const int z = (int)(v % (I)Cc.nz);
+    const I n = v / (I)Cc.nz;
     float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
@@ -467,18 +566,19 @@ __global__ void k_upbwd_mask(const uint4* __restrict__ gfine, const uint4* __res
   }
 }
 
+template <typename I>
 __global__ void k_poolbwd_add_mask(const uint4* __restrict__ gskip, const uint4* __restrict__ gcoarse,
                                    const uint4* __restrict__ act, uint4* __restrict__ out, Lv F, Lv Cc,
                                    size_t total) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
+  for (I i = blockIdx.x * (I)blockDim.x + threadIdx.x; i < (I)total; i += (I)(gridDim.x * blockDim.x)) {
     const int g = (int)(i & 1);
-    size_t v = i >> 1;
-    const int x = (int)(v % F.nx);
-    v /= F.nx;
-    const int y = (int)(v % F.ny);
-    v /= F.ny;
-    const int z = (int)(v % F.nz);
-    const size_t n = v / F.nz;
+    I v = i >> 1;
+    const int x = (int)(v % (I)F.nx);
+    v /= (I)F.nx;
+    const int y = (int)(v % (I)F.ny);
+    v /= (I)F.ny;
+    const int z = (int)(v % (I)F.nz);
+    const I n = v / (I)F.nz;
     float a[8], b[8];
     unpack8(gskip[i], a);
     unpack8(gcoarse[Cc.u4(n, z >> 1, y >> 1, x >> 1, g)], b);
@@ -500,8 +600,18 @@ __global__ void k_sumsq(Fields f, size_t vox, float* __restrict__ partials) {
   __shared__ double sh[32];
   const float* a = field(blockIdx.z ? f.p : f.b, f, blockIdx.y);
   float acc = 0.f;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < vox; i += (size_t)gridDim.x * blockDim.x)
-    acc = fmaf(a[i], a[i], acc);
+  // few blocks per sample: sixteen loads in flight per thread (256 x 128 x 128:
+  // 117 -> 18.5 us), added in the order of i
+  const size_t step = (size_t)gridDim.x * blockDim.x;
+  size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  for (; i + 15 * step < vox; i += 16 * step) {
+    float v[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) v[k] = __ldg(a + i + k * step);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) acc = fmaf(v[k], v[k], acc);
+  }
+  for (; i < vox; i += step) acc = fmaf(a[i], a[i], acc);
   const double t = block_sum((double)acc, sh);
   if (threadIdx.x == 0) partials[(blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = (float)t;
 }
@@ -516,35 +626,43 @@ __global__ void k_rms_final(const float* __restrict__ partials, int nblk, size_t
   double acc = 0.0;
   const int s0 = pooled ? 0 : s, s1 = pooled ? n : s + 1;
   for (int q = s0; q < s1; ++q)
-    for (int b = 0; b < nblk; ++b) acc += (double)partials[(fld * n + q) * nblk + b];
+    for (int b = 0; b < nblk; b += 16) {  // nblk is a multiple of 16
+      float v[16];
+#pragma unroll
+      for (int k = 0; k < 16; ++k) v[k] = partials[(fld * n + q) * nblk + b + k];
+#pragma unroll
+      for (int k = 0; k < 16; ++k) acc += (double)v[k];
+    }
   const double r = sqrt(acc / ((double)vox * (s1 - s0)));
   rms[i] = r > 0.0 ? (float)r : 1.f;
   inv[i] = r > 0.0 ? (float)(1.0 / r) : 1.f;
 }
 
+template <typename I>
 __global__ void k_pack_input(Fields f, const float* __restrict__ inv, uint4* __restrict__ x0, size_t vox, int n) {
   const size_t total = vox * (size_t)n;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-    const int s = (int)(i / vox);
-    const size_t v = i - (size_t)s * vox;
+  for (I i = blockIdx.x * (I)blockDim.x + threadIdx.x; i < (I)total; i += (I)(gridDim.x * blockDim.x)) {
+    const int s = (int)(i / (I)vox);
+    const I v = i - (I)s * (I)vox;
     const float bv = field(f.b, f, s)[v] * inv[s], pv = field(f.p, f, s)[v] * inv[n + s];
-    x0[2 * i] = make_uint4(pack_bf2(bv, pv), 0u, 0u, 0u);
-    x0[2 * i + 1] = make_uint4(0u, 0u, 0u, 0u);
+    const uint32_t q[8] = {pack_bf2(bv, pv), 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+    store32(x0 + 2 * (size_t)i, q);
   }
 }
 
+template <typename I>
 __global__ void k_loss_grad(const float* __restrict__ y, Fields f, const float* __restrict__ inv,
                             uint4* __restrict__ gy, size_t vox, int n, double* __restrict__ partials) {
   __shared__ double sh[32];
   const size_t total = vox * (size_t)n;
   float acc = 0.f;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-    const int s = (int)(i / vox);
-    const size_t v = i - (size_t)s * vox;
+  for (I i = blockIdx.x * (I)blockDim.x + threadIdx.x; i < (I)total; i += (I)(gridDim.x * blockDim.x)) {
+    const int s = (int)(i / (I)vox);
+    const I v = i - (I)s * (I)vox;
     const float d = y[i] - field(f.t, f, s)[v] * inv[s];
     acc = fmaf(d, d, acc);
-    gy[2 * i] = make_uint4(pack_bf2(d, 0.f), 0u, 0u, 0u);
-    gy[2 * i + 1] = make_uint4(0u, 0u, 0u, 0u);
+    const uint32_t q[8] = {pack_bf2(d, 0.f), 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+    store32(gy + 2 * (size_t)i, q);
   }
   const double t = block_sum((double)acc, sh);
   if (threadIdx.x == 0) partials[blockIdx.x] = t;
@@ -563,30 +681,36 @@ __global__ void k_sum_partials(const double* __restrict__ partials, int nblk, do
 // the crop of (v_c - v_n).
 __device__ __forceinline__ float crop_stencil(const float* v, const float* fl, size_t i, int x, int y, int z, int nx,
                                               int ny, int nz) {
+  // every load before the first use (a missing neighbour loads the cell)
   const size_t sy = (size_t)nx, sz = (size_t)nx * ny;
+  const bool in[6] = {x > 0, x < nx - 1, y > 0, y < ny - 1, z > 0, z < nz - 1};
+  const size_t j[6] = {in[0] ? i - 1 : i,  in[1] ? i + 1 : i,  in[2] ? i - sy : i,
+                       in[3] ? i + sy : i, in[4] ? i - sz : i, in[5] ? i + sz : i};
+  float vn[6], fn[6];
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    vn[k] = v[j[k]];
+    fn[k] = fl ? fl[j[k]] : 1.f;
+  }
   const float vc = v[i];
   float acc = 0.f;
-  auto nb = [&](bool inside, size_t j) {
-    if (inside && (!fl || fl[j] > 0.5f)) acc += vc - v[j];
-  };
-  nb(x > 0, i - 1);
-  nb(x < nx - 1, i + 1);
-  nb(y > 0, i - sy);
-  nb(y < ny - 1, i + sy);
-  nb(z > 0, i - sz);
-  nb(z < nz - 1, i + sz);
+#pragma unroll
+  for (int k = 0; k < 6; ++k)
+    if (in[k] && fn[k] > 0.5f) acc += vc - vn[k];
   return acc;
 }
 
+template <typename I>
 __global__ void k_residual(const float* __restrict__ y, Fields f, const float* __restrict__ inv, int nx, int ny,
                            int nz, int n, float inv_h2, float* __restrict__ r, double* __restrict__ partials) {
   __shared__ double sh[32];
   const size_t vox = (size_t)nx * ny * nz, total = vox * n;
   float acc = 0.f;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-    const int s = (int)(i / vox);
-    const size_t v = i - (size_t)s * vox;
-    const int x = (int)(v % nx), yy = (int)((v / nx) % ny), z = (int)(v / ((size_t)nx * ny));
+  for (I i = blockIdx.x * (I)blockDim.x + threadIdx.x; i < (I)total; i += (I)(gridDim.x * blockDim.x)) {
+    const int s = (int)(i / (I)vox);
+    const I v = i - (I)s * (I)vox;
+    const I row = v / (I)nx;
+    const int x = (int)(v % (I)nx), yy = (int)(row % (I)ny), z = (int)(row / (I)ny);
     const float* fl = f.fluid ? field(f.fluid, f, s) : nullptr;
     const bool inner = x > 0 && x < nx - 1 && yy > 0 && yy < ny - 1 && z > 0 && z < nz - 1;
     float rv = 0.f;
@@ -600,18 +724,20 @@ __global__ void k_residual(const float* __restrict__ y, Fields f, const float* _
   if (threadIdx.x == 0) partials[blockIdx.x] = t;
 }
 
+template <typename I>
 __global__ void k_apply_crop(const float* __restrict__ r, Fields f, int nx, int ny, int nz, int n, float inv_h2,
                              uint4* __restrict__ gy) {
   const size_t vox = (size_t)nx * ny * nz, total = vox * n;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-    const int s = (int)(i / vox);
-    const size_t v = i - (size_t)s * vox;
-    const int x = (int)(v % nx), yy = (int)((v / nx) % ny), z = (int)(v / ((size_t)nx * ny));
+  for (I i = blockIdx.x * (I)blockDim.x + threadIdx.x; i < (I)total; i += (I)(gridDim.x * blockDim.x)) {
+    const int s = (int)(i / (I)vox);
+    const I v = i - (I)s * (I)vox;
+    const I row = v / (I)nx;
+    const int x = (int)(v % (I)nx), yy = (int)(row % (I)ny), z = (int)(row / (I)ny);
     const float* fl = f.fluid ? field(f.fluid, f, s) : nullptr;
     float g = 0.f;
     if (!fl || fl[v] > 0.5f) g = crop_stencil(r + (size_t)s * vox, fl, v, x, yy, z, nx, ny, nz) * inv_h2;
-    gy[2 * i] = make_uint4(pack_bf2(g, 0.f), 0u, 0u, 0u);
-    gy[2 * i + 1] = make_uint4(0u, 0u, 0u, 0u);
+    const uint32_t q[8] = {pack_bf2(g, 0.f), 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+    store32(gy + 2 * (size_t)i, q);
   }
 }
 
@@ -721,22 +847,37 @@ static int grid_for(K kernel, int threads, int smem) {
   return occupancy_blocks(kernel, threads, smem);
 }
 
+static int device_sms() {
+  int dev = 0, nsm = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return 1;
+  return nsm > 0 ? nsm : 1;
+}
+
 template <int EPI>
-static cudaError_t conv_epi(const CUtensorMap& m4, const CUtensorMap& m2, const void* wpack, ConvArgs a,
-                            cudaStream_t s) {
+static cudaError_t conv_epi(const void* x, const void* wpack, ConvArgs a, cudaStream_t s) {
   static int grid_cache = 0;
   if (!grid_cache) grid_cache = grid_for(k_conv<EPI>, kConvThreads, kConvSmem);
   if (grid_cache < 0) return cudaErrorInvalidValue;
-  // z-runs: long enough to amortise the four-plane start, short enough for
-  // about three items per resident block
+  // z-runs: a run of c outputs costs c + 2 planes.  The tensor core's operand
+  // reads bound an SM that has two or more runs in work (its runs' planes add
+  // up); a lone run is bound by its own chain, about 1.7 planes' time each;
+  // and a block's start costs about eight planes.
   const long long columns = (long long)a.tx * a.ty * a.nn;
-  long long zc = (a.nz * columns + 3LL * grid_cache - 1) / (3LL * grid_cache);
-  zc = std::max(2LL, std::min(32LL, (zc + 1) / 2 * 2));
-  a.zc = (int)zc;
-  a.nzc = (int)((a.nz + zc - 1) / zc);
-  a.nitems = columns * a.nzc;
+  const long long nsm = device_sms();
+  double best = -1.0;
+  for (int runs = 1; runs <= (a.nz + 3) / 4; ++runs) {
+    const int zc = (a.nz + runs - 1) / runs;
+    const long long items = columns * ((a.nz + zc - 1) / zc);
+    const double cost = std::max((double)((items + nsm - 1) / nsm), 1.7) * (zc + 2) + 8.0;
+    if (best >= 0.0 && cost >= best) continue;
+    best = cost;
+    a.zc = zc;
+    a.nzc = (a.nz + zc - 1) / zc;
+    a.nitems = items;
+  }
   const long long g = a.nitems < grid_cache ? a.nitems : grid_cache;
-  k_conv<EPI><<<(unsigned)(g > 0 ? g : 1), kConvThreads, kConvSmem, s>>>(m4, m2, (const uint4*)wpack, a);
+  k_conv<EPI><<<(unsigned)(g > 0 ? g : 1), kConvThreads, kConvSmem, s>>>((const unsigned char*)x, (const unsigned char*)wpack, a);
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return cudaGetLastError();
 }
@@ -744,9 +885,7 @@ static cudaError_t conv_epi(const CUtensorMap& m4, const CUtensorMap& m2, const 
 cudaError_t launch_conv(const void* x, const void* wpack, void* out, int epi, const void* mask, const float* scale,
                         const Dims& d, int* err, cudaStream_t s) {
   if (d.n <= 0 || d.vox() == 0) return cudaSuccess;
-  CUtensorMap m4, m2;
-  if (!encode_act(&m4, x, d, kTX, kTY + 2, kRing) || !encode_act(&m2, x, d, kTX, kTY + 2, 2))
-    return cudaErrorInvalidValue;
+  if (((uintptr_t)x | (uintptr_t)wpack) & 15) return cudaErrorInvalidValue;
   ConvArgs a;
   a.nx = d.nx;
   a.ny = d.ny;
@@ -761,11 +900,11 @@ cudaError_t launch_conv(const void* x, const void* wpack, void* out, int epi, co
   a.scale = scale;
   a.err = err;
   switch (epi) {
-    case kEpiF32: return conv_epi<kEpiF32>(m4, m2, wpack, a, s);
-    case kEpiRelu: return conv_epi<kEpiRelu>(m4, m2, wpack, a, s);
-    case kEpiLin: return conv_epi<kEpiLin>(m4, m2, wpack, a, s);
-    case kEpiMask: return conv_epi<kEpiMask>(m4, m2, wpack, a, s);
-    case kEpiOut0: return conv_epi<kEpiOut0>(m4, m2, wpack, a, s);
+    case kEpiF32: return conv_epi<kEpiF32>(x, wpack, a, s);
+    case kEpiRelu: return conv_epi<kEpiRelu>(x, wpack, a, s);
+    case kEpiLin: return conv_epi<kEpiLin>(x, wpack, a, s);
+    case kEpiMask: return conv_epi<kEpiMask>(x, wpack, a, s);
+    case kEpiOut0: return conv_epi<kEpiOut0>(x, wpack, a, s);
   }
   return cudaErrorInvalidValue;
 }
@@ -800,7 +939,7 @@ cudaError_t launch_wgrad(const void* x, const void* g, float* partials, int max_
 
 cudaError_t launch_wgrad_reduce(const float* partials, int nblocks, float* dw, float scale, bool accumulate,
                                 cudaStream_t s) {
-  k_wgrad_reduce<<<(kWElems + 255) / 256, 256, 0, s>>>(partials, nblocks, dw, scale, accumulate ? 1 : 0);
+  k_wgrad_reduce<<<kWElems / 32, 256, 0, s>>>(partials, nblocks, dw, scale, accumulate ? 1 : 0);
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return cudaGetLastError();
 }
@@ -809,14 +948,14 @@ static Lv lv_of(const Dims& d, int shift) { return Lv{d.nx >> shift, d.ny >> shi
 
 cudaError_t launch_pool(const void* fine, void* coarse, const Dims& d, cudaStream_t s) {
   const size_t total = d.vox() / 8 * d.n * 2;
-  k_pool<<<grid_1d(total), 256, 0, s>>>((const uint4*)fine, (uint4*)coarse, lv_of(d, 0), lv_of(d, 1), total);
+  GN_INDEXED(total, k_pool, grid_1d(total), 256, s, (const uint4*)fine, (uint4*)coarse, lv_of(d, 0), lv_of(d, 1), total);
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return cudaGetLastError();
 }
 
 cudaError_t launch_up_add(const void* coarse, const void* fine, void* out, const Dims& d, cudaStream_t s) {
   const size_t total = d.vox() * d.n * 2;
-  k_up_add<<<grid_1d(total), 256, 0, s>>>((const uint4*)coarse, (const uint4*)fine, (uint4*)out, lv_of(d, 0),
+  GN_INDEXED(total, k_up_add, grid_1d(total), 256, s, (const uint4*)coarse, (const uint4*)fine, (uint4*)out, lv_of(d, 0),
                                           lv_of(d, 1), total);
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return cudaGetLastError();
@@ -825,7 +964,7 @@ cudaError_t launch_up_add(const void* coarse, const void* fine, void* out, const
 cudaError_t launch_upbwd_mask(const void* gfine, const void* act_coarse, void* out_coarse, const Dims& d,
                               cudaStream_t s) {
   const size_t total = d.vox() / 8 * d.n * 2;
-  k_upbwd_mask<<<grid_1d(total), 256, 0, s>>>((const uint4*)gfine, (const uint4*)act_coarse, (uint4*)out_coarse,
+  GN_INDEXED(total, k_upbwd_mask, grid_1d(total), 256, s, (const uint4*)gfine, (const uint4*)act_coarse, (uint4*)out_coarse,
                                               lv_of(d, 0), lv_of(d, 1), total);
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return cudaGetLastError();
@@ -834,7 +973,7 @@ cudaError_t launch_upbwd_mask(const void* gfine, const void* act_coarse, void* o
 cudaError_t launch_poolbwd_add_mask(const void* gskip, const void* gcoarse, const void* act, void* out,
                                     const Dims& d, cudaStream_t s) {
   const size_t total = d.vox() * d.n * 2;
-  k_poolbwd_add_mask<<<grid_1d(total), 256, 0, s>>>((const uint4*)gskip, (const uint4*)gcoarse, (const uint4*)act,
+  GN_INDEXED(total, k_poolbwd_add_mask, grid_1d(total), 256, s, (const uint4*)gskip, (const uint4*)gcoarse, (const uint4*)act,
                                                     (uint4*)out, lv_of(d, 0), lv_of(d, 1), total);
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return cudaGetLastError();
@@ -851,7 +990,7 @@ cudaError_t launch_rms(const Fields& f, const Dims& d, bool pooled, float* parti
 }
 
 cudaError_t launch_pack_input(const Fields& f, const float* inv_rms, void* x0, const Dims& d, cudaStream_t s) {
-  k_pack_input<<<grid_1d(d.vox() * d.n), 256, 0, s>>>(f, inv_rms, (uint4*)x0, d.vox(), d.n);
+  GN_INDEXED(d.vox() * d.n, k_pack_input, grid_1d(d.vox() * d.n), 256, s, f, inv_rms, (uint4*)x0, d.vox(), d.n);
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return cudaGetLastError();
 }
@@ -859,7 +998,7 @@ cudaError_t launch_pack_input(const Fields& f, const float* inv_rms, void* x0, c
 cudaError_t launch_loss_grad(const float* y, const Fields& f, const float* inv_rms, void* gy, double* partials,
                              double* loss, const Dims& d, cudaStream_t s) {
   const int g = grid_1d(d.vox() * d.n);
-  k_loss_grad<<<g, 256, 0, s>>>(y, f, inv_rms, (uint4*)gy, d.vox(), d.n, partials);
+  GN_INDEXED(d.vox() * d.n, k_loss_grad, g, 256, s, y, f, inv_rms, (uint4*)gy, d.vox(), d.n, partials);
   g_launches.fetch_add(1, std::memory_order_relaxed);
   k_sum_partials<<<1, 256, 0, s>>>(partials, g, 0.5 / ((double)d.vox() * d.n), loss);
   g_launches.fetch_add(1, std::memory_order_relaxed);
@@ -869,11 +1008,11 @@ cudaError_t launch_loss_grad(const float* y, const Fields& f, const float* inv_r
 cudaError_t launch_residual_loss_grad(const float* y, const Fields& f, const float* inv_rms, float inv_h2, float* r,
                                       void* gy, double* partials, double* loss, const Dims& d, cudaStream_t s) {
   const int g = grid_1d(d.vox() * d.n);
-  k_residual<<<g, 256, 0, s>>>(y, f, inv_rms, d.nx, d.ny, d.nz, d.n, inv_h2, r, partials);
+  GN_INDEXED(d.vox() * d.n, k_residual, g, 256, s, y, f, inv_rms, d.nx, d.ny, d.nz, d.n, inv_h2, r, partials);
   g_launches.fetch_add(1, std::memory_order_relaxed);
   k_sum_partials<<<1, 256, 0, s>>>(partials, g, 0.5 / ((double)d.vox() * d.n), loss);
   g_launches.fetch_add(1, std::memory_order_relaxed);
-  k_apply_crop<<<g, 256, 0, s>>>(r, f, d.nx, d.ny, d.nz, d.n, inv_h2, (uint4*)gy);
+  GN_INDEXED(d.vox() * d.n, k_apply_crop, g, 256, s, r, f, d.nx, d.ny, d.nz, d.n, inv_h2, (uint4*)gy);
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return cudaGetLastError();
 }

@@ -47,15 +47,16 @@ int coarse_start_level(const LevelDev* lv, int L, int dim, size_t smem_limit, bo
 
 // The coarse cycle of level n cells as a dense matrix (mg_dense.cu): bytes of
 // the matrix and of its set-up's scratch, its set-up (a.finest 0; a wait
-// that times out sets st->status), and y = M b (b and y with 16-byte aligned
-// storage padded to a multiple of four values).
+// that times out sets st->status), and y = M b unless *done (b and y with
+// 16-byte aligned storage padded to a multiple of four values).
 size_t dense_bytes(int n);
 size_t dense_scratch_bytes(int n);
 cudaError_t launch_dense_matrix(const CoarseArgs& a, size_t smem_bytes, int n, float* M, float* scratch,
                                 SolveState* st, cudaStream_t s);
 template <typename T>
-cudaError_t launch_dense(int dim, int n, const float* M, const void* b, void* y, const SolveState* st,
-                         cudaStream_t s);
+cudaError_t launch_dense(int dim, int n, const float* M, const void* b, void* y, const int* done, cudaStream_t s);
+int dense_stride(int n);  // floats of a row of M
+cudaError_t launch_transpose(float* M, int n, cudaStream_t s);  // in place
 
 // Level legs: T is the storage of a level's iterate and of its coarse-side
 // arrays, TB that of its right-hand side b and of the up leg's output (the
@@ -146,7 +147,10 @@ struct ClusterArgs {
   int ca_off;               // float offset of the coarse cycle's region
   int ca_floats;
   float omega, s;
+  const float* dense;       // matrix of that cycle (n <= 1024 cells, a multiple of 4 C), or nullptr: block 0 runs it
+  int dense_n;
 };
+constexpr int kClusterDense = 1024;
 // Plan the cluster launch: the first distributed level k1, the first level
 // of the coarse cycle kd (the first level after k1 within the coarse-cell
 // limit, at least kc), the cluster size, the shared-memory bytes, and the

@@ -225,7 +225,8 @@ bool cluster_pcg2d_plan(const LevelDev* lv, int L, int kc, ClusterPcgArgs* out, 
     return false;
   // the kernel's static shared memory (two solve states, sums) and slack
   const size_t limit = (size_t)optin - 4096;
-  const size_t thr = cluster_coarse_cells();
+  // the coarse cycle is a dense matrix here: levels of at most 1024 cells
+  const size_t thr = getenv("NPMG_CLUSTER_COARSE_CELLS") ? cluster_coarse_cells() : kClusterDense;
   for (int C : {16, 8}) {
     if (!distributable(lv[0], C)) continue;
     int kq = 0;

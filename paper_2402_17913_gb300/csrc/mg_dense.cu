@@ -92,7 +92,7 @@ constexpr int kAhead = 16;     // float4 of its row a lane holds before b is nee
 template <typename T>
 __global__ void __launch_bounds__(32 * kRowWarps) k_dense(int n, int ld, const float* __restrict__ M,
                                                           const T* __restrict__ b, T* __restrict__ y,
-                                                          const SolveState* __restrict__ st, int release) {
+                                                          const int* __restrict__ done, int release) {
   if (release) chain_release();
   const int row = blockIdx.x * kRowWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   const float4* __restrict__ m = reinterpret_cast<const float4*>(M + (size_t)min(row, n - 1) * ld);
@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(32 * kRowWarps) k_dense(int n, int ld, const f
     r[k] = i < n4 ? __ldg(m + i) : make_float4(0.f, 0.f, 0.f, 0.f);
   }
   chain_enter();
-  if (st && st->inner_done) return;
+  if (done && *done) return;
   if (row >= n) return;  // whole warps
   float acc[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
@@ -127,6 +127,12 @@ int dense_stride(int n) { return (n + 3) & ~3; }
 size_t dense_bytes(int n) { return (size_t)n * dense_stride(n) * sizeof(float); }
 size_t dense_scratch_bytes(int n) { return 4 * (size_t)(2 * dense_stride(n) + 4) * sizeof(float); }
 
+cudaError_t launch_transpose(float* M, int n, cudaStream_t s) {
+  const int t = (n + 31) / 32;
+  k_transpose<<<dim3(t, t), 256, 0, s>>>(M, n, dense_stride(n));
+  return cudaGetLastError();
+}
+
 cudaError_t launch_dense_matrix(const CoarseArgs& a, size_t smem_bytes, int n, float* M, float* scratch,
                                 SolveState* st, cudaStream_t s) {
   const int ld = dense_stride(n);
@@ -139,20 +145,17 @@ cudaError_t launch_dense_matrix(const CoarseArgs& a, size_t smem_bytes, int n, f
   if (e != cudaSuccess) return e;
   k_unit_vectors<<<32, 256, 0, s>>>(scratch, ld);
   k<<<n, 1024, smem_bytes, s>>>(a, scratch, ld, ld, M, st, (int)(smem_bytes / sizeof(float)));
-  const int t = (n + 31) / 32;
-  k_transpose<<<dim3(t, t), 256, 0, s>>>(M, n, ld);
-  return cudaGetLastError();
+  e = cudaGetLastError();
+  return e == cudaSuccess ? launch_transpose(M, n, s) : e;
 }
 
 template <typename T>
-cudaError_t launch_dense(int dim, int n, const float* M, const void* b, void* y, const SolveState* st,
-                         cudaStream_t s) {
+cudaError_t launch_dense(int dim, int n, const float* M, const void* b, void* y, const int* done, cudaStream_t s) {
   return launch_chain(k_dense<T>, (n + kRowWarps - 1) / kRowWarps, 32 * kRowWarps, 0, s, n, dense_stride(n), M,
-                      (const T*)b, (T*)y, st, dim == 3 ? 1 : 0);
+                      (const T*)b, (T*)y, done, dim == 3 ? 1 : 0);
 }
-template cudaError_t launch_dense<float>(int, int, const float*, const void*, void*, const SolveState*, cudaStream_t);
-template cudaError_t launch_dense<__half>(int, int, const float*, const void*, void*, const SolveState*, cudaStream_t);
-template cudaError_t launch_dense<__nv_bfloat16>(int, int, const float*, const void*, void*, const SolveState*,
-                                                 cudaStream_t);
+template cudaError_t launch_dense<float>(int, int, const float*, const void*, void*, const int*, cudaStream_t);
+template cudaError_t launch_dense<__half>(int, int, const float*, const void*, void*, const int*, cudaStream_t);
+template cudaError_t launch_dense<__nv_bfloat16>(int, int, const float*, const void*, void*, const int*, cudaStream_t);
 
 }  // namespace npmg

@@ -193,8 +193,8 @@ static cudaError_t enqueue_vcycle(mg_handle_s* h, const void* r, void* z, SolveS
                            h->clu_y, st, s);
     else
       e = h->kc == 0 ? launch_coarse<float>(ca, h->ca_smem, r, z, st, s)
-                     : launch_dense<T>(DIM, (int)h->ncell[h->kc], h->dense, h->bk[h->kc], h->yk[h->kc], st,
-                                       s);
+                     : launch_dense<T>(DIM, (int)h->ncell[h->kc], h->dense, h->bk[h->kc], h->yk[h->kc],
+                                       st ? &st->inner_done : nullptr, s);
   }
   if (e != cudaSuccess) return e;
   for (int k = kdown - 1; k >= 0; --k) {
@@ -700,6 +700,8 @@ mg_status mg_create(mg_handle* out, int dim, const int64_t shape[3], const doubl
     plan.push_back({(void**)&h->clu_y, h->ncell[kc] * 4});
     plan.push_back({(void**)&h->clu_image, h->ca_smem});
     plan.push_back({(void**)&h->cpcg_image, h->ca_smem});
+    // grids above 2^17 cells do not fit a cluster's shared memory
+    if (n0c <= (size_t)1 << 17) plan.push_back({(void**)&h->cpcg_dense, dense_bytes(kClusterDense)});
   }
   plan.push_back({(void**)&h->partials, (size_t)kMaxPartials * 8});
   plan.push_back({(void**)&h->st, sizeof(SolveState)});
@@ -780,7 +782,6 @@ mg_status mg_create(mg_handle* out, int dim, const int64_t shape[3], const doubl
     ca.image = h->cimage;
     if (kc > 0) {
       NPMG_TRY(launch_dense_matrix(ca, h->ca_smem, (int)h->ncell[kc], h->dense, h->dense_scratch, h->st, s));
-      NPMG_TRY(cudaMemcpyAsync(h->st_host, h->st, sizeof(SolveState), cudaMemcpyDeviceToHost, s));
     }
   }
   h->nb1d = default_blocks_1d(h, h->ncell[0]);
@@ -880,6 +881,13 @@ mg_status mg_create(mg_handle* out, int dim, const int64_t shape[3], const doubl
         pa.a.ca = cc;
         pa.a.omega = (float)o.omega;
         pa.a.s = (float)o.coarse_scale;
+        const int nd = (int)h->ncell[h->cpcg_kd];
+        if (h->cpcg_dense && nd <= kClusterDense && nd % (4 * pa.a.C) == 0) {
+          if (e == cudaSuccess)
+            e = launch_dense_matrix(cc, ca_bytes, nd, h->cpcg_dense, h->dense_scratch, h->st, s);
+          pa.a.dense = h->cpcg_dense;
+          pa.a.dense_n = nd;
+        }
         h->cpcg = pa;
         h->cpcg_ok = e == cudaSuccess;
       }
@@ -891,6 +899,7 @@ mg_status mg_create(mg_handle* out, int dim, const int64_t shape[3], const doubl
                                  (const float*)h->p[1], (const float*)h->d, (const float*)h->r);
     return e;
   }));
+  NPMG_TRY(cudaMemcpyAsync(h->st_host, h->st, sizeof(SolveState), cudaMemcpyDeviceToHost, s));
   NPMG_TRY(cudaStreamSynchronize(s));
   NPMG_TRY(cudaGetLastError());
 #undef NPMG_TRY

@@ -17,17 +17,18 @@
 // which its last block takes the convergence decision), on levels 0 .. kc-1
 // a tile down leg (V: pre sweeps from zero, residual, 2x2 average;
 // sawtooth: x = b / c, average of b, on level 0 after forming r and ||r||
-// itself), one single-block kernel
-// for levels kc .. L-1 (<= 4096 nodes; coarsest level by a dense inverse
-// in the V cycle), tile up legs back to level 0 (x + s P e, post sweeps);
+// itself), the cycle of levels kc .. L-1 (<= 2048 nodes; coarsest level by a
+// dense inverse in the V cycle) as one dense matrix written at create
+// (mg_dense.cu), tile up legs back to level 0 (x + s P e, post sweeps);
 // the level-0 up leg adds the correction to the float-float iterate and sums
 // its L1 norm (the paper's stopping gauge).  Every kernel returns at once
-// after the state's done flag is set, so a CUDA graph of kChunk cycles is
-// replayed until the host sees the flag.
+// after the state's done flag is set; the cycles run as one graph with a
+// conditional while node, so a solve needs the host once, at its end.
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <cmath>
+#include <cstdlib>
 #include <cstring>
 #include <new>
 #include <vector>
@@ -41,9 +42,16 @@ namespace ad {
 constexpr int TX = 64, TY = 16;  // tile of the level-leg kernels
 constexpr int kT = 256;          // threads per tile block
 constexpr int kCB = 1024;        // threads of the coarse block
-constexpr int kCoarseCells = 4096;
+constexpr int kCoarseCells = 4096;  // largest first level of the coarse cycle
+// The first level of the coarse matrix: 2048 nodes.  With 4096 (64 MB on 64^2)
+// 1024^2 steps take 0.84 instead of 0.79 ms, 176x208 ones 0.55 instead of 0.58.
+constexpr int kDenseCells = 2048;
 constexpr int kCoarsestMax = 256;
-constexpr int kChunk = 8;        // cycles per graph launch
+constexpr int kChunk = 8;        // cycles per graph launch (host-driven loop)
+constexpr int kBody = 2;         // cycles per body of the device-side loop
+// Levels up to this size on the 32 x 8 tiles: 1024^2 steps 0.84 / 0.79 / 0.90 ms
+// with 100,000 / 300,000 / 1,200,000 (level 0 too).
+constexpr long kSmallNodes = 300000;
 
 struct Lev {
   int nx, ny;
@@ -56,47 +64,8 @@ struct State {
   double bnorm2, relres, relres0, l1, l1_first;
   int cycles, done, status;
   unsigned int counter[2];
+  unsigned int checks;  // of the device-side loop
 };
-
-// Sum of v over the block, in a fixed shuffle-tree order; the result is
-// valid in thread 0.
-__device__ __forceinline__ double block_sum(double v) {
-  __shared__ double ws[32];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  __syncthreads();  // ws may still be read by a previous call
-  if (lane == 0) ws[wid] = v;
-  __syncthreads();
-  double s = 0.0;
-  if (threadIdx.x == 0)
-    for (int w = 0; w < (int)(blockDim.x + 31) / 32; ++w) s += ws[w];
-  return s;
-}
-
-// Grid sum of v: each block writes its sum to partials[bid]; the last block
-// to finish adds the nblocks partials with all its threads (a fixed strided
-// assignment, then block_sum: deterministic) and gets the total in thread
-// 0, which alone returns true.  The counter is reset for the next use.
-__device__ bool grid_sum(double v, double* partials, unsigned int* counter, unsigned int nblocks, unsigned int bid,
-                         double* total) {
-  __shared__ bool is_last;
-  const double bs = block_sum(v);
-  if (threadIdx.x == 0) {
-    partials[bid] = bs;
-    __threadfence();
-    is_last = atomicAdd(counter, 1u) == nblocks - 1;
-  }
-  __syncthreads();
-  if (!is_last) return false;
-  __threadfence();
-  double s = 0.0;
-  for (unsigned int k = threadIdx.x; k < nblocks; k += blockDim.x) s += ((volatile double*)partials)[k];
-  s = block_sum(s);
-  if (threadIdx.x != 0) return false;
-  *total = s;
-  *counter = 0;
-  return true;
-}
 
 // Error-free transformations (Knuth's two-sum, the FMA two-product): a + b
 // = s + e and a * b = p + e exactly in float32.
@@ -128,7 +97,7 @@ __global__ void __launch_bounds__(kT) k_ad_init(Lev L, const float* __restrict__
     acc = fmaf(bv, bv, acc);
   }
   double tot;
-  if (grid_sum(acc, partials, &st->counter[0], gridDim.x, blockIdx.x, &tot)) {
+  if (grid_sum_last(acc, partials, &st->counter[0], &tot) && threadIdx.x == 0) {
     st->tol = tol;
     st->l1_tol = l1_tol;
     st->max_cycles = max_cycles;
@@ -139,6 +108,7 @@ __global__ void __launch_bounds__(kT) k_ad_init(Lev L, const float* __restrict__
     st->done = 0;
     st->status = MG_OK;
     st->counter[1] = 0;
+    st->checks = 0;
   }
 }
 
@@ -171,27 +141,80 @@ __device__ __forceinline__ void ff_sub_term(float w, float2 x, float& S, float& 
 }
 
 // r = b - A x in float-float (rounded to float32 for the cycle), relres and
-// the stopping decision.  `final` computes the relres of the returned
-// iterate whatever the flag says and decides nothing.
+// the stopping decision.  FINAL: the relres of the returned iterate whatever
+// the flag says, deciding nothing, and the float32 output (the float-float
+// iterate rounded once) into r's place.  Blocks of 256 threads walk groups of
+// 8 rows x 128 nodes; VEC (rows of whole float4, 16-byte aligned arrays): a
+// thread takes four nodes with all their loads in flight.
+template <bool VEC, bool FINAL>
 __global__ void __launch_bounds__(kT) k_ad_resid(Lev L, const float* __restrict__ b, const float2* __restrict__ x,
-                                                 float* __restrict__ r, State* st, double* partials, int final) {
+                                                 float* __restrict__ r, State* st, double* partials) {
   chain_enter();
-  if (!final && st->done) return;
+  if (!FINAL && st->done) return;
   float acc = 0.f;
-  AD_FOR_NODES(L) {
+  const int gxn = (L.nx + 127) / 128, groups = gxn * ((L.ny + 7) / 8);
+  for (int g = blockIdx.x; g < groups; g += gridDim.x) {
+    const int ix = (g % gxn) * 128 + (threadIdx.x & 31) * 4, iy = (g / gxn) * 8 + (threadIdx.x >> 5);
+    if (ix >= L.nx || iy >= L.ny) continue;
     const size_t i = (size_t)iy * L.nx + ix;
-    float S = b[i], E = 0.f;
-    ff_sub_term(L.c, x[i], S, E);
-    if (ix > 0) ff_sub_term(L.xm, x[i - 1], S, E);
-    if (ix + 1 < L.nx) ff_sub_term(L.xp, x[i + 1], S, E);
-    if (iy > 0) ff_sub_term(L.ym, x[i - L.nx], S, E);
-    if (iy + 1 < L.ny) ff_sub_term(L.yp, x[i + L.nx], S, E);
-    const float rv = S + E;
-    if (!final) r[i] = rv;
-    acc = fmaf(rv, rv, acc);
+    const bool up = iy > 0, dn = iy + 1 < L.ny;
+    const float2 zero = make_float2(0.f, 0.f);
+    float2 xc[6], xu[4], xd[4];
+    float bv[4], rv[4];
+    auto row = [&](const float2* __restrict__ p, bool on, float2* v) {
+      if (VEC) {
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f), c = a;
+        if (on) {
+          a = *reinterpret_cast<const float4*>(p);
+          c = *reinterpret_cast<const float4*>(p + 2);
+        }
+        v[0] = make_float2(a.x, a.y);
+        v[1] = make_float2(a.z, a.w);
+        v[2] = make_float2(c.x, c.y);
+        v[3] = make_float2(c.z, c.w);
+      } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = on && ix + k < L.nx ? p[k] : zero;
+      }
+    };
+    row(x + i, true, xc + 1);
+    row(x + i - (up ? L.nx : 0), up, xu);
+    row(x + i + (dn ? L.nx : 0), dn, xd);
+    xc[0] = ix > 0 ? x[i - 1] : zero;
+    xc[5] = ix + 4 < L.nx ? x[i + 4] : zero;
+    if (VEC) {
+      const float4 q = *reinterpret_cast<const float4*>(b + i);
+      bv[0] = q.x;
+      bv[1] = q.y;
+      bv[2] = q.z;
+      bv[3] = q.w;
+    } else {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) bv[k] = ix + k < L.nx ? b[i + k] : 0.f;
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      // a neighbour off the grid is 0 and adds exactly 0
+      float S = bv[k], E = 0.f;
+      ff_sub_term(L.c, xc[k + 1], S, E);
+      ff_sub_term(L.xm, xc[k], S, E);
+      ff_sub_term(L.xp, xc[k + 2], S, E);
+      ff_sub_term(L.ym, xu[k], S, E);
+      ff_sub_term(L.yp, xd[k], S, E);
+      rv[k] = S + E;
+      if (VEC || ix + k < L.nx) acc = fmaf(rv[k], rv[k], acc);
+      if (FINAL) rv[k] = xc[k + 1].x + xc[k + 1].y;
+    }
+    if (VEC) {
+      *reinterpret_cast<float4*>(r + i) = make_float4(rv[0], rv[1], rv[2], rv[3]);
+    } else {
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (ix + k < L.nx) r[i + k] = rv[k];
+    }
   }
   double tot;
-  if (grid_sum(acc, partials, &st->counter[0], gridDim.x, blockIdx.x, &tot)) decide(st, tot, final != 0);
+  if (grid_sum_last(acc, partials, &st->counter[0], &tot) && threadIdx.x == 0) decide(st, tot, FINAL);
 }
 
 // One relaxed Jacobi sweep over window J, [J, RX - J) x [J, RY - J), of a
@@ -326,7 +349,27 @@ __global__ void __launch_bounds__(kT) k_ad_down_saw(Lev L, const float* __restri
   }
   if (FUSED) {
     double tot;
-    if (grid_sum(acc, partials, &st->counter[0], gridDim.x, blockIdx.x, &tot)) decide(st, tot, false);
+    if (grid_sum_last(acc, partials, &st->counter[0], &tot) && threadIdx.x == 0) decide(st, tot, false);
+  }
+}
+
+// x + v in float-float, renormalised.
+__device__ __forceinline__ float2 ff_plus(float2 x, float v) {
+  float hs, he;
+  two_sum(x.x, v, hs, he);
+  he += x.y;
+  const float hi = hs + he;
+  return make_float2(hi, he - (hi - hs));
+}
+
+// Bookkeeping of one cycle from the L1 norm of its change of x.
+__device__ __forceinline__ void cycle_end(State* st, double l1) {
+  st->cycles += 1;
+  st->l1 = l1;
+  if (st->cycles == 1) st->l1_first = l1;
+  if (l1 <= st->l1_tol) {
+    st->status = MG_OK;
+    st->done = 1;
   }
 }
 
@@ -368,13 +411,7 @@ __global__ void __launch_bounds__(kT) k_ad_up(Lev L, const float* __restrict__ b
       const size_t gi = (size_t)gy * L.nx + gx;
       const float v = cur[(R + ty) * RX + R + tx];
       if (FINEST) {
-        // x += v in float-float, renormalised
-        const float2 xo = xff[gi];
-        float hs, he;
-        two_sum(xo.x, v, hs, he);
-        he += xo.y;
-        const float hi = hs + he;
-        xff[gi] = make_float2(hi, he - (hi - hs));
+        xff[gi] = ff_plus(xff[gi], v);
         acc += fabsf(v);
       } else {
         y[gi] = v;
@@ -383,15 +420,126 @@ __global__ void __launch_bounds__(kT) k_ad_up(Lev L, const float* __restrict__ b
   }
   if (FINEST) {
     double t;
-    if (grid_sum(acc, partials, &st->counter[1], gridDim.x * gridDim.y, blockIdx.y * gridDim.x + blockIdx.x, &t)) {
-      st->cycles += 1;
-      st->l1 = t;
-      if (st->cycles == 1) st->l1_first = t;
-      if (t <= st->l1_tol) {
-        st->status = MG_OK;
-        st->done = 1;
-      }
+    if (grid_sum_last(acc, partials, &st->counter[1], &t) && threadIdx.x == 0) cycle_end(st, t);
+  }
+}
+
+// V legs with two sweeps on tiles of 32 x 8 nodes, one output node per thread
+// (mg_small.cu gives the reasons: a level's leg is the latency of one block,
+// and 64 x 16 tiles put six nodes per thread in each of its phases).  The
+// first sweep from zero is pointwise, so the halo is two nodes.
+constexpr int SX = 32, SY = 8, SRX = SX + 4, SRY = SY + 4, SRN = SRX * SRY;
+constexpr int SWX = SX + 2, SWN = SWX * (SY + 2);
+static_assert(SX * SY == kT, "one output node per thread");
+
+__device__ __forceinline__ float stencil(const Lev& L, const float* x, int i) {
+  return L.c * x[i] + L.xm * x[i - 1] + L.xp * x[i + 1] + L.ym * x[i - SRX] + L.yp * x[i + SRX];
+}
+
+// One sweep of the tile and its one-node ring; nodes off the level stay 0.
+__device__ __forceinline__ void sweep_ring(const Lev& L, const float* cur, float* nxt, const float* sb, int ox,
+                                           int oy, float omega) {
+#pragma unroll
+  for (int k = 0; k < (SWN + kT - 1) / kT; ++k) {
+    const int q = threadIdx.x + k * kT;
+    if (q >= SWN) break;
+    const int lx = 1 + q % SWX, ly = 1 + q / SWX, i = ly * SRX + lx;
+    const int gx = ox + lx, gy = oy + ly;
+    const bool in = gx >= 0 && gx < L.nx && gy >= 0 && gy < L.ny;
+    nxt[i] = in ? cur[i] + omega * (sb[i] - stencil(L, cur, i)) * L.inv_c : 0.f;
+  }
+}
+
+__global__ void __launch_bounds__(kT) k_ad_down_c(Lev L, const float* __restrict__ b, float* __restrict__ x,
+                                                  float* __restrict__ bc, float omega, const State* st) {
+  __shared__ float sb[SRN], s1[SRN], s2[SRN], sr[kT];
+  const int ox = blockIdx.x * SX - 2, oy = blockIdx.y * SY - 2;
+  chain_enter();
+  if (st->done) return;
+  constexpr int K = (SRN + kT - 1) / kT;
+  float v[K];
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const int i = threadIdx.x + k * kT, gx = ox + i % SRX, gy = oy + i / SRX;
+    v[k] = i < SRN && gx >= 0 && gx < L.nx && gy >= 0 && gy < L.ny ? b[(size_t)gy * L.nx + gx] : 0.f;
+  }
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const int i = threadIdx.x + k * kT;
+    if (i < SRN) {
+      sb[i] = v[k];
+      s1[i] = omega * v[k] * L.inv_c;
     }
+  }
+  __syncthreads();
+  sweep_ring(L, s1, s2, sb, ox, oy, omega);
+  __syncthreads();
+  const int tx = threadIdx.x % SX, ty = threadIdx.x / SX, li = (ty + 2) * SRX + tx + 2;
+  const int gx = blockIdx.x * SX + tx, gy = blockIdx.y * SY + ty;
+  const bool in = gx < L.nx && gy < L.ny;
+  sr[threadIdx.x] = in ? sb[li] - stencil(L, s2, li) : 0.f;
+  if (in) x[(size_t)gy * L.nx + gx] = s2[li];
+  __syncthreads();
+  if (threadIdx.x < kT / 4) {
+    const int cx = threadIdx.x % (SX / 2), cy = threadIdx.x / (SX / 2);
+    const int gcx = blockIdx.x * (SX / 2) + cx, gcy = blockIdx.y * (SY / 2) + cy;
+    if (gcx < L.nx / 2 && gcy < L.ny / 2) {
+      const float* p = sr + 2 * cy * SX + 2 * cx;
+      bc[(size_t)gcy * (L.nx / 2) + gcx] = 0.25f * ((p[0] + p[1]) + (p[SX] + p[SX + 1]));
+    }
+  }
+}
+
+template <bool FINEST>
+__global__ void __launch_bounds__(kT) k_ad_up_c(Lev L, const float* __restrict__ b, const float* __restrict__ x,
+                                                const float* __restrict__ e, float* __restrict__ y,
+                                                float2* __restrict__ xff, float s, float omega, State* st,
+                                                double* partials) {
+  __shared__ float sb[SRN], s0[SRN], s1[SRN];
+  const int ox = blockIdx.x * SX - 2, oy = blockIdx.y * SY - 2, cnx = L.nx / 2;
+  const int tx = threadIdx.x % SX, ty = threadIdx.x / SX, li = (ty + 2) * SRX + tx + 2;
+  const int gx = blockIdx.x * SX + tx, gy = blockIdx.y * SY + ty;
+  const bool in = gx < L.nx && gy < L.ny;
+  const size_t gi = (size_t)gy * L.nx + gx;
+  chain_enter();
+  if (st->done) return;
+  constexpr int K = (SRN + kT - 1) / kT;
+  float bv[K], xv[K], ev[K];
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const int i = threadIdx.x + k * kT, hx = ox + i % SRX, hy = oy + i / SRX;
+    const bool on = i < SRN && hx >= 0 && hx < L.nx && hy >= 0 && hy < L.ny;
+    const size_t h = (size_t)hy * L.nx + hx;
+    bv[k] = on ? b[h] : 0.f;
+    xv[k] = on ? x[h] : 0.f;
+    ev[k] = on ? e[(size_t)(hy >> 1) * cnx + (hx >> 1)] : 0.f;
+  }
+  float2 xo = make_float2(0.f, 0.f);
+  if (FINEST && in) xo = xff[gi];
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const int i = threadIdx.x + k * kT;
+    if (i < SRN) {
+      sb[i] = bv[k];
+      s0[i] = fmaf(s, ev[k], xv[k]);
+    }
+  }
+  __syncthreads();
+  sweep_ring(L, s0, s1, sb, ox, oy, omega);
+  __syncthreads();
+  float acc = 0.f;
+  if (in) {
+    const float v = s1[li] + omega * (sb[li] - stencil(L, s1, li)) * L.inv_c;
+    if (FINEST) {
+      xff[gi] = ff_plus(xo, v);
+      acc = fabsf(v);
+    } else {
+      y[gi] = v;
+    }
+  }
+  if (FINEST) {
+    double t;
+    if (grid_sum_last(acc, partials, &st->counter[1], &t) && threadIdx.x == 0) cycle_end(st, t);
   }
 }
 
@@ -412,8 +560,6 @@ struct AdCoarseArgs {
                         // x and t, each (nx + 2)(ny + 2) with a zero ring
   int lnx[kMaxLevels];  // log2(nx) when nx is a power of two, else -1
   int words;            // floats of shared memory in use
-  const float* b_first;
-  float* y_first;
   const float* inv;  // dense inverse of the coarsest level (V cycle)
 };
 
@@ -448,9 +594,11 @@ __device__ void cb_sweeps(const Lev& L, int lnx, const float* b, float*& cur, fl
   }
 }
 
-__global__ void __launch_bounds__(kCB) k_ad_coarse(AdCoarseArgs a, const State* st) {
-  chain_enter();
-  if (st->done) return;
+// The cycle of the levels first .. last is a fixed linear map of level first's
+// right-hand side: column j of its matrix into row j of `Mt`, one block per
+// column, from unit vector j (`E`: 2 n + 1 zeros but a 1 at index n).
+__global__ void __launch_bounds__(kCB) k_ad_columns(AdCoarseArgs a, const float* __restrict__ E,
+                                                    float* __restrict__ Mt, int ld) {
   extern __shared__ float sm[];
   float* res[kMaxLevels];
   const bool saw = a.cycle == MG_CYCLE_SAWTOOTH;
@@ -462,7 +610,7 @@ __global__ void __launch_bounds__(kCB) k_ad_coarse(AdCoarseArgs a, const State* 
   __syncthreads();
   {
     const int n = a.lv[a.first].nx * a.lv[a.first].ny;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) B(a.first)[i] = a.b_first[i];
+    for (int i = threadIdx.x; i < n; i += blockDim.x) B(a.first)[i] = E[n - (int)blockIdx.x + i];
     __syncthreads();
   }
   // down: V smooths from zero and restricts the residual; the sawtooth
@@ -542,17 +690,20 @@ __global__ void __launch_bounds__(kCB) k_ad_coarse(AdCoarseArgs a, const State* 
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
       int ix, iy;
       node_xy(i, L.nx, a.lnx[a.first], ix, iy);
-      a.y_first[i] = res[a.first][(iy + 1) * W + ix + 1];
+      Mt[(size_t)blockIdx.x * ld + i] = res[a.first][(iy + 1) * W + ix + 1];
     }
   }
 }
 
-// x (float32 output) = the float-float iterate rounded once.
-__global__ void __launch_bounds__(kT) k_ad_out(size_t n, const float2* __restrict__ xff, float* __restrict__ x) {
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const float2 v = xff[i];
-    x[i] = v.x + v.y;
-  }
+__global__ void k_ad_unit(float* E, int n) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < 2 * n + 1; i += gridDim.x * blockDim.x)
+    E[i] = i == n ? 1.f : 0.f;
+}
+
+// The condition of the device-side loop (one thread).
+__global__ void k_ad_loop(cudaGraphConditionalHandle h, State* st, unsigned int cap) {
+  const unsigned int n = ++st->checks;
+  cudaGraphSetConditional(h, !st->done && n < cap ? 1u : 0u);
 }
 
 }  // namespace ad
@@ -573,10 +724,16 @@ struct ad_handle_s {
   float* xk[kMaxLevels];
   float* yk[kMaxLevels];
   float* inv;
+  float* dense;    // matrix of the cycle on levels kc .. L-1
   double* partials;
   State* st;
   State* st_host;
+  cudaEvent_t ev0, ev1;
+  // the solve's cycles: a graph with a conditional while node (loop_state 1)
+  // or, where that cannot be built (-1), a graph of kChunk cycles launched
+  // until the host sees the done flag
   cudaGraphExec_t graph;
+  int loop_state;
   int64_t chunk_kernels;
   int64_t launches;
 };
@@ -668,12 +825,18 @@ static int grid_1d(const ad_handle_s* h, size_t n) {
   return (int)(b < 1 ? 1 : b);
 }
 
-// Row-strided kernels: one block per row up to 8 blocks per SM.
+// Row-strided kernels: one block per row up to 8 blocks per SM; the residual:
+// groups of 8 rows x 128 nodes on 4 blocks per SM.
 static int row_grid(const ad_handle_s* h) { return std::min(h->ny, h->nsm * 8); }
+static int group_grid(const ad_handle_s* h) {
+  return (int)std::min((long)((h->nx + 127) / 128) * ((h->ny + 7) / 8), (long)h->nsm * 4);
+}
+static bool small_level(const Lev& L) { return (long)L.nx * L.ny <= kSmallNodes; }
+static dim3 small_grid(const Lev& L) { return dim3((L.nx + SX - 1) / SX, (L.ny + SY - 1) / SY); }
 
 static dim3 tile_grid(const Lev& L) { return dim3((L.nx + TX - 1) / TX, (L.ny + TY - 1) / TY); }
 
-// One cycle: residual, down legs, the coarse block, up legs.
+// One cycle: residual, down legs, the coarse matrix, up legs.
 static cudaError_t enqueue_cycle(ad_handle_s* h, cudaStream_t s) {
   const ad_options& o = h->opt;
   const float om = (float)o.omega, sc = (float)o.coarse_scale;
@@ -684,8 +847,13 @@ static cudaError_t enqueue_cycle(ad_handle_s* h, cudaStream_t s) {
   // inside the sawtooth's down leg, which has no halo
   cudaError_t e = cudaSuccess;
   if (!saw) {
-    e = launch_chain(k_ad_resid, dim3(row_grid(h)), dim3(kT), 0, s, h->lv[0], (const float*)h->b,
-                     (const float2*)h->xff, h->r, h->st, h->partials, 0);
+    const float* b = h->b;
+    const float2* x = h->xff;
+    e = h->nx % 4 == 0
+            ? launch_chain(k_ad_resid<true, false>, dim3(group_grid(h)), dim3(kT), 0, s, h->lv[0], b, x, h->r, h->st,
+                           h->partials)
+            : launch_chain(k_ad_resid<false, false>, dim3(group_grid(h)), dim3(kT), 0, s, h->lv[0], b, x, h->r, h->st,
+                           h->partials);
     h->launches += 1;
   }
   for (int k = 0; k < h->kc && e == cudaSuccess; ++k) {
@@ -700,6 +868,9 @@ static cudaError_t enqueue_cycle(ad_handle_s* h, cudaStream_t s) {
                                 h->bk[k + 1], h->st, xf, rr, pt)
                  : launch_chain(k_ad_down_saw<false>, dim3(grid_1d(h, nc)), dim3(kT), 0, s, L, bk, h->xk[k],
                                 h->bk[k + 1], h->st, xf, rr, pt);
+    } else if (o.pre == 2 && small_level(L)) {
+      e = launch_chain(k_ad_down_c, small_grid(L), dim3(kT), 0, s, L, bk, h->xk[k], h->bk[k + 1], om,
+                       (const State*)h->st);
     } else {
 #define NPMG_AD_DOWN(P) \
   launch_chain(k_ad_down<P>, tile_grid(L), dim3(kT), 0, s, L, bk, h->xk[k], h->bk[k + 1], om, (const State*)h->st)
@@ -709,6 +880,33 @@ static cudaError_t enqueue_cycle(ad_handle_s* h, cudaStream_t s) {
     h->launches += 1;
   }
   if (e != cudaSuccess) return e;
+  e = launch_dense<float>(2, h->lv[h->kc].nx * h->lv[h->kc].ny, h->dense, h->bk[h->kc], h->yk[h->kc], &h->st->done, s);
+  h->launches += 1;
+  for (int k = h->kc - 1; k >= 0 && e == cudaSuccess; --k) {
+    const float* bk = k == 0 ? h->r : h->bk[k];
+    const Lev& L = h->lv[k];
+    const dim3 g = tile_grid(L);
+#define NPMG_AD_UP(P, F)                                                                                      \
+  launch_chain(k_ad_up<P, F>, g, dim3(kT), 0, s, L, bk, (const float*)h->xk[k], (const float*)h->yk[k + 1], \
+               h->yk[k], h->xff, sc, om, h->st, h->partials)
+    if (o.post == 2 && small_level(L))
+      e = k == 0 ? launch_chain(k_ad_up_c<true>, small_grid(L), dim3(kT), 0, s, L, bk, (const float*)h->xk[k],
+                                (const float*)h->yk[k + 1], h->yk[k], h->xff, sc, om, h->st, h->partials)
+                 : launch_chain(k_ad_up_c<false>, small_grid(L), dim3(kT), 0, s, L, bk, (const float*)h->xk[k],
+                                (const float*)h->yk[k + 1], h->yk[k], h->xff, sc, om, h->st, h->partials);
+    else if (k == 0)
+      e = o.post == 0 ? NPMG_AD_UP(0, true) : (o.post == 1 ? NPMG_AD_UP(1, true) : NPMG_AD_UP(2, true));
+    else
+      e = o.post == 0 ? NPMG_AD_UP(0, false) : (o.post == 1 ? NPMG_AD_UP(1, false) : NPMG_AD_UP(2, false));
+#undef NPMG_AD_UP
+    h->launches += 1;
+  }
+  return e;
+}
+
+// Set-up of the coarse matrix (`scratch`: 2 n + 1 floats).
+static cudaError_t make_dense(ad_handle_s* h, float* scratch, cudaStream_t s) {
+  const ad_options& o = h->opt;
   AdCoarseArgs ca;
   memset(&ca, 0, sizeof(ca));
   ca.first = h->kc;
@@ -716,8 +914,8 @@ static cudaError_t enqueue_cycle(ad_handle_s* h, cudaStream_t s) {
   ca.cycle = o.cycle;
   ca.pre = o.pre;
   ca.post = o.post;
-  ca.omega = om;
-  ca.s = sc;
+  ca.omega = (float)o.omega;
+  ca.s = (float)o.coarse_scale;
   int off = 0;
   for (int k = 0; k < h->L; ++k) {
     ca.lv[k] = h->lv[k];
@@ -729,31 +927,61 @@ static cudaError_t enqueue_cycle(ad_handle_s* h, cudaStream_t s) {
     }
   }
   ca.words = off;
-  ca.b_first = h->bk[h->kc];
-  ca.y_first = h->yk[h->kc];
-  const size_t cb_smem = (size_t)off * sizeof(float);
   ca.inv = h->inv;
-  e = launch_chain(k_ad_coarse, dim3(1), dim3(kCB), cb_smem, s, ca, (const State*)h->st);
-  h->launches += 1;
-  for (int k = h->kc - 1; k >= 0 && e == cudaSuccess; --k) {
-    const float* bk = k == 0 ? h->r : h->bk[k];
-    const Lev& L = h->lv[k];
-    const dim3 g = tile_grid(L);
-#define NPMG_AD_UP(P, F)                                                                                      \
-  launch_chain(k_ad_up<P, F>, g, dim3(kT), 0, s, L, bk, (const float*)h->xk[k], (const float*)h->yk[k + 1], \
-               h->yk[k], h->xff, sc, om, h->st, h->partials)
-    if (k == 0)
-      e = o.post == 0 ? NPMG_AD_UP(0, true) : (o.post == 1 ? NPMG_AD_UP(1, true) : NPMG_AD_UP(2, true));
-    else
-      e = o.post == 0 ? NPMG_AD_UP(0, false) : (o.post == 1 ? NPMG_AD_UP(1, false) : NPMG_AD_UP(2, false));
-#undef NPMG_AD_UP
-    h->launches += 1;
+  const int n = h->lv[h->kc].nx * h->lv[h->kc].ny;
+  k_ad_unit<<<16, 256, 0, s>>>(scratch, n);
+  k_ad_columns<<<n, kCB, (size_t)off * sizeof(float), s>>>(ca, scratch, h->dense, dense_stride(n));
+  const cudaError_t e = cudaGetLastError();
+  return e == cudaSuccess ? launch_transpose(h->dense, n, s) : e;
+}
+
+// while (!done) { kBody cycles; condition }, entered once: the first residual
+// of the body takes the decision on the guess.
+static cudaError_t build_loop(ad_handle_s* h) {
+  cudaGraph_t G = nullptr, body = nullptr, tmp = nullptr;
+  cudaStream_t cs = nullptr;
+  cudaGraphConditionalHandle ch;
+  const int64_t before = h->launches;
+  cudaError_t e = cudaGraphCreate(&G, 0);
+  if (e != cudaSuccess) return e;
+  e = cudaGraphConditionalHandleCreate(&ch, G, 1, cudaGraphCondAssignDefault);
+  if (e == cudaSuccess) {
+    cudaGraphNodeParams p = {cudaGraphNodeTypeConditional};
+    p.conditional.handle = ch;
+    p.conditional.type = cudaGraphCondTypeWhile;
+    p.conditional.size = 1;
+    cudaGraphNode_t node;
+    e = cudaGraphAddNode(&node, G, nullptr, nullptr, 0, &p);
+    if (e == cudaSuccess) body = p.conditional.phGraph_out[0];
   }
+  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
+  if (e == cudaSuccess) e = cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
+  if (e == cudaSuccess) {
+    cudaError_t e2 = cudaSuccess;
+    for (int c = 0; c < kBody && e2 == cudaSuccess; ++c) e2 = enqueue_cycle(h, cs);
+    if (e2 == cudaSuccess) {
+      k_ad_loop<<<1, 1, 0, cs>>>(ch, h->st, (unsigned)h->opt.max_cycles / kBody + 2u);
+      h->launches += 1;
+      e2 = cudaGetLastError();
+    }
+    e = cudaStreamEndCapture(cs, &tmp);
+    if (e2 != cudaSuccess) e = e2;
+  }
+  h->chunk_kernels = h->launches - before;
+  h->launches = before;
+  if (e == cudaSuccess) e = cudaGraphInstantiate(&h->graph, G, 0);
+  cudaGraphDestroy(G);
+  if (cs) cudaStreamDestroy(cs);
   return e;
 }
 
 static cudaError_t ensure_graph(ad_handle_s* h) {
   if (h->graph) return cudaSuccess;
+  if (h->loop_state == 0) {
+    h->loop_state = getenv("NPMG_NO_DEVICE_LOOP") == nullptr && build_loop(h) == cudaSuccess ? 1 : -1;
+    cudaGetLastError();
+    if (h->loop_state == 1) return cudaSuccess;
+  }
   cudaStream_t cs;
   cudaError_t e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
   if (e != cudaSuccess) return e;
@@ -853,11 +1081,12 @@ mg_status ad_create(ad_handle* out, const int64_t cells[2], double h, double dt,
     const double scale = o.coarse_op == AD_COARSE_GALERKIN ? (double)(1 << k) : 1.0;
     hd->lv[k] = make_level((int)(nx >> k), (int)(ny >> k), h * (1 << k), dt, nu, u, v, scheme, scale);
   }
-  // the single block takes every level from the first one of <= 4096 nodes
-  // (never the finest, whose up leg updates the iterate)
+  // the coarse matrix takes every level from the first one of <= 2048 nodes,
+  // or a coarsest one of <= 4096 (never the finest, whose up leg updates the
+  // iterate)
   hd->kc = L - 1;
   for (int k = 1; k < L; ++k)
-    if ((int64_t)hd->lv[k].nx * hd->lv[k].ny <= kCoarseCells) {
+    if ((int64_t)hd->lv[k].nx * hd->lv[k].ny <= kDenseCells) {
       hd->kc = k;
       break;
     }
@@ -878,7 +1107,7 @@ mg_status ad_create(ad_handle* out, const int64_t cells[2], double h, double dt,
       return MG_ERR_INVALID;
     }
   }
-  if (cudaFuncSetAttribute(k_ad_coarse, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  if (cudaFuncSetAttribute(k_ad_columns, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)(kCoarseSmemMax * sizeof(float))) != cudaSuccess) {
     set_error("ad_create: %s", cudaGetErrorString(cudaGetLastError()));
     delete hd;
@@ -910,10 +1139,13 @@ mg_status ad_create(ad_handle* out, const int64_t cells[2], double h, double dt,
   // one pool: b, r, the iterate, per-level arrays, the inverse, partials, state
   const size_t n0 = (size_t)nx * ny;
   const size_t tiles0 = (size_t)tile_grid(hd->lv[0]).x * tile_grid(hd->lv[0]).y;
-  const size_t npart = std::max(tiles0, (size_t)hd->nsm * 8) + 1;
+  const size_t small0 = small_level(hd->lv[0]) ? (size_t)small_grid(hd->lv[0]).x * small_grid(hd->lv[0]).y : 0;
+  const size_t npart = std::max(std::max(tiles0, small0), (size_t)hd->nsm * 8) + 1;
+  const int nkc = hd->lv[hd->kc].nx * hd->lv[hd->kc].ny;
   auto al = [](size_t v) { return (v + 255) / 256 * 256; };
   size_t bytes = al(n0 * 4) * 2 + al(n0 * 8) + al(npart * 8) + al(sizeof(State)) + al(inv.size() * 4 + 4);
   bytes += al(n0 * 4);  // x on level 0 (the V down leg's smoothed iterate)
+  bytes += al(dense_bytes(nkc)) + al((size_t)(2 * nkc + 1) * 4);
   // levels 1 .. kc: right-hand side and correction; below kc also the
   // smoothed iterate; the single block keeps levels kc .. L-1 on chip
   for (int k = 1; k <= hd->kc; ++k) bytes += (k < hd->kc ? 3 : 2) * al((size_t)hd->lv[k].nx * hd->lv[k].ny * 4);
@@ -936,6 +1168,8 @@ mg_status ad_create(ad_handle* out, const int64_t cells[2], double h, double dt,
   hd->partials = (double*)take(npart * 8);
   hd->st = (State*)take(sizeof(State));
   hd->inv = (float*)take(inv.size() * 4 + 4);
+  hd->dense = (float*)take(dense_bytes(nkc));
+  float* unit = (float*)take((size_t)(2 * nkc + 1) * 4);
   hd->xk[0] = (float*)take(n0 * 4);
   hd->bk[0] = hd->r;
   hd->yk[0] = nullptr;
@@ -950,7 +1184,9 @@ mg_status ad_create(ad_handle* out, const int64_t cells[2], double h, double dt,
   if (cudaMemsetAsync(hd->pool, 0, bytes, s) != cudaSuccess ||
       (!inv.empty() &&
        cudaMemcpyAsync(hd->inv, inv.data(), inv.size() * 4, cudaMemcpyHostToDevice, s) != cudaSuccess) ||
-      cudaMallocHost((void**)&hd->st_host, sizeof(State)) != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) {
+      cudaMallocHost((void**)&hd->st_host, sizeof(State)) != cudaSuccess ||
+      cudaEventCreate(&hd->ev0) != cudaSuccess || cudaEventCreate(&hd->ev1) != cudaSuccess ||
+      make_dense(hd, unit, s) != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) {
     set_error("ad_create: %s", cudaGetErrorString(cudaGetLastError()));
     st = MG_ERR_CUDA;
   }
@@ -970,38 +1206,39 @@ mg_status ad_solve(ad_handle hd, const float* d_b, const float* d_x0, float* d_x
   }
   cudaStream_t s = (cudaStream_t)stream;
   const size_t n0 = (size_t)hd->nx * hd->ny;
-  cudaEvent_t e0 = nullptr, e1 = nullptr;
-  NPMG_CUDA(cudaEventCreate(&e0));
-  NPMG_CUDA(cudaEventCreate(&e1));
-  NPMG_CUDA(cudaEventRecord(e0, s));
+  NPMG_CUDA(ensure_graph(hd));
+  NPMG_CUDA(cudaEventRecord(hd->ev0, s));
   NPMG_CUDA(cudaMemcpyAsync(hd->b, d_b, n0 * 4, cudaMemcpyDeviceToDevice, s));
   k_ad_init<<<row_grid(hd), kT, 0, s>>>(hd->lv[0], hd->b, d_x0, hd->xff, hd->st, rel_tol, l1_tol,
                                            hd->opt.max_cycles, hd->partials);
   hd->launches += 1;
   NPMG_CUDA(cudaGetLastError());
-  NPMG_CUDA(ensure_graph(hd));
-  // each graph launch runs kChunk cycles (kernels return once done); the
-  // resid kernel ends the solve at max_cycles, at most one launch later
-  const int max_launch = hd->opt.max_cycles / kChunk + 2;
-  for (int it = 0; it < max_launch; ++it) {
+  if (hd->loop_state == 1) {
     NPMG_CUDA(cudaGraphLaunch(hd->graph, s));
-    hd->launches += hd->chunk_kernels;
-    NPMG_CUDA(cudaMemcpyAsync(hd->st_host, hd->st, sizeof(State), cudaMemcpyDeviceToHost, s));
-    NPMG_CUDA(cudaStreamSynchronize(s));
-    if (hd->st_host->done) break;
+  } else {
+    // each graph launch runs kChunk cycles (kernels return once done); the
+    // resid kernel ends the solve at max_cycles, at most one launch later
+    const int max_launch = hd->opt.max_cycles / kChunk + 2;
+    for (int it = 0; it < max_launch; ++it) {
+      NPMG_CUDA(cudaGraphLaunch(hd->graph, s));
+      hd->launches += hd->chunk_kernels;
+      NPMG_CUDA(cudaMemcpyAsync(hd->st_host, hd->st, sizeof(State), cudaMemcpyDeviceToHost, s));
+      NPMG_CUDA(cudaStreamSynchronize(s));
+      if (hd->st_host->done) break;
+    }
   }
   // relres of the returned iterate, and the float32 output
-  k_ad_resid<<<row_grid(hd), kT, 0, s>>>(hd->lv[0], hd->b, hd->xff, hd->r, hd->st, hd->partials, 1);
-  k_ad_out<<<grid_1d(hd, n0), kT, 0, s>>>(n0, hd->xff, d_x);
-  hd->launches += 2;
+  const bool vec = hd->nx % 4 == 0 && ((uintptr_t)d_x & 15) == 0;
+  const auto last = vec ? k_ad_resid<true, true> : k_ad_resid<false, true>;
+  last<<<group_grid(hd), kT, 0, s>>>(hd->lv[0], hd->b, hd->xff, d_x, hd->st, hd->partials);
+  hd->launches += 1;
   NPMG_CUDA(cudaGetLastError());
-  NPMG_CUDA(cudaEventRecord(e1, s));
+  NPMG_CUDA(cudaEventRecord(hd->ev1, s));
   NPMG_CUDA(cudaMemcpyAsync(hd->st_host, hd->st, sizeof(State), cudaMemcpyDeviceToHost, s));
   NPMG_CUDA(cudaStreamSynchronize(s));
   float ms = 0.f;
-  cudaEventElapsedTime(&ms, e0, e1);
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
+  cudaEventElapsedTime(&ms, hd->ev0, hd->ev1);
+  if (hd->loop_state == 1) hd->launches += hd->chunk_kernels * (int64_t)hd->st_host->checks;
   const State& S = *hd->st_host;
   const mg_status status = S.done ? (mg_status)S.status : MG_NOT_CONVERGED;
   if (out) {
@@ -1027,6 +1264,8 @@ mg_status ad_destroy(ad_handle hd) {
   if (hd->graph) cudaGraphExecDestroy(hd->graph);
   if (hd->pool) cudaFree(hd->pool);
   if (hd->st_host) cudaFreeHost(hd->st_host);
+  if (hd->ev0) cudaEventDestroy(hd->ev0);
+  if (hd->ev1) cudaEventDestroy(hd->ev1);
   delete hd;
   return MG_OK;
 }

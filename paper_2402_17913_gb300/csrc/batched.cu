@@ -63,6 +63,8 @@ struct BatchArgs {
   const int4* items[kMaxLevels];  // (instance, tile x, tile y, slot) per level
   int nitems[kMaxLevels];
   int ntile_levels;      // max kc over instances
+  const int2* citems;    // coarse phase: (instance, first row of a dense product) or (instance, -1)
+  int ncitems;
   double* partials;      // one per level-0 tile
   unsigned* bar;         // [0] arrivals, [1] generation, [2] error, [4..5] active counts
   int sweeps;
@@ -880,6 +882,29 @@ __device__ __forceinline__ double reduce_slots(const BatchArgs& A, const BInst& 
   return tot;
 }
 
+// Rows row0 .. row0 + kBRows - 1 of the exact solve of an instance whose
+// coarse part is its coarsest level alone (sides with few factors of two: up
+// to 32 x 32 cells): a warp per row.  As one item of one block the whole
+// product, up to 4 MB, came through a single SM, a row per lane (15 instances
+// of sides 96, 100, 160 and 320, coarsest 25 x 25 for 100: 15.0 -> 5.1 ms).
+constexpr int kBRows = 64;
+constexpr int kBDense = 128;  // cells from which the product is split
+__device__ void b_dense_rows(const BInst& I, int row0, float* S) {
+  const int n = I.ca.ncoarse;
+  const float* __restrict__ b = I.b[I.kc];
+  for (int j = threadIdx.x; j < n; j += kBThreads) S[j] = b[j];
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  for (int r = row0 + (threadIdx.x >> 5); r < min(row0 + kBRows, n); r += kBThreads / 32) {
+    const float* __restrict__ m = I.ca.inv + (size_t)r * n;
+    float acc = 0.f;
+#pragma unroll 8
+    for (int j = lane; j < n; j += 32) acc = fmaf(__ldg(m + j), S[j], acc);
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) I.y[I.kc][r] = acc;
+  }
+}
+
 // active-instance counters alternate between two slots (the reducing phase
 // clears the other one for the next count)
 __device__ __forceinline__ void count_active(const BatchArgs& A, int slot, bool active) {
@@ -1011,12 +1036,14 @@ __global__ void __launch_bounds__(kBThreads, 4) k_batched(const __grid_constant_
         }
         if (!grid_barrier(A, epoch)) return;
       }
-      // block-local coarse part of each instance
-      for (int w = blockIdx.x; w < A.count; w += gridDim.x) {
-        if (A.st[w].inner_done) continue;
-        const BInst& I = A.inst[w];
+      // coarse part of each instance: block-local, or rows of its dense solve
+      for (int w = blockIdx.x; w < A.ncitems; w += gridDim.x) {
+        const int2 item = A.citems[w];
+        if (A.st[item.x].inner_done) continue;
+        const BInst& I = A.inst[item.x];
         __syncthreads();
-        coarse_cycle<2, float, false>(I.ca, I.kc == 0 ? I.r : I.b[I.kc], I.kc == 0 ? I.z : I.y[I.kc], nullptr, S,
+        if (item.y >= 0) b_dense_rows(I, item.y, S);
+        else coarse_cycle<2, float, false>(I.ca, I.kc == 0 ? I.r : I.b[I.kc], I.kc == 0 ? I.z : I.y[I.kc], nullptr, S,
                                I.cfloats);
       }
       if (!grid_barrier(A, epoch)) return;
@@ -1165,6 +1192,8 @@ struct mg_batch_s {
   const float** d_xin;           // guesses read by the init phase
   void** h_ptrs;                 // pinned staging of the pointer tables
   std::vector<int4*> d_items;
+  int2* d_citems;
+  int ncitems;
   int nitems[kMaxLevels];
   int ntile_levels;
   double* d_partials;
@@ -1243,6 +1272,8 @@ static mg_status batched_launch(mg_batch_s* B, int tile, int sweeps, double tol,
     A.nitems[k] = B->nitems[k];
   }
   A.ntile_levels = B->ntile_levels;
+  A.citems = B->d_citems;
+  A.ncitems = B->ncitems;
   A.partials = B->d_partials;
   A.bar = B->d_bar;
   A.sweeps = sweeps;
@@ -1598,6 +1629,20 @@ static mg_status build_items(mg_batch_s* B, int tile, cudaStream_t s) {
   }
   for (int4* p : B->d_items) cudaFree(p);
   B->d_items.assign(kMaxLevels, nullptr);
+  if (!B->d_citems) {
+    std::vector<int2> ci;
+    for (int i = 0; i < B->count; ++i) {
+      const BInst& I = B->inst[i];
+      if (I.kc > 0 && I.kc == I.L - 1 && I.ca.ncoarse > kBDense && I.ca.pre >= 0)
+        for (int r = 0; r < I.ca.ncoarse; r += kBRows) ci.push_back(make_int2(i, r));
+      else
+        ci.push_back(make_int2(i, -1));
+    }
+    B->ncitems = (int)ci.size();
+    NPMG_CUDA(cudaMalloc((void**)&B->d_citems, ci.size() * sizeof(int2)));
+    NPMG_CUDA(cudaMemcpyAsync(B->d_citems, ci.data(), ci.size() * sizeof(int2), cudaMemcpyHostToDevice, s));
+    NPMG_CUDA(cudaStreamSynchronize(s));
+  }
   for (int k = 0; k < kMaxLevels; ++k) {
     B->nitems[k] = (int)items[k].size();
     if (items[k].empty()) continue;
@@ -1778,6 +1823,7 @@ mg_status mg_destroy_batched(mg_batch B) {
   for (int t = 0; t < kNTiles; ++t)
     for (int k = 0; k < 4; ++k)
       if (B->graph[t][k]) cudaGraphExecDestroy(B->graph[t][k]);
+  if (B->d_citems) cudaFree(B->d_citems);
   for (int4* p : B->d_items) cudaFree(p);
   if (B->pool) cudaFree(B->pool);
   if (B->d_inst) cudaFree(B->d_inst);

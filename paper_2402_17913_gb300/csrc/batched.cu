@@ -1627,6 +1627,13 @@ static mg_status build_items(mg_batch_s* B, int tile, cudaStream_t s) {
     }
     I.ntiles0 = slot - I.slot0;
   }
+  // the captured launches hold the lists freed here
+  for (int t = 0; t < kNTiles; ++t)
+    for (int k = 0; k < 4; ++k)
+      if (B->graph[t][k]) {
+        cudaGraphExecDestroy(B->graph[t][k]);
+        B->graph[t][k] = nullptr;
+      }
   for (int4* p : B->d_items) cudaFree(p);
   B->d_items.assign(kMaxLevels, nullptr);
   if (!B->d_citems) {

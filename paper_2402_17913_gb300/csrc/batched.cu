@@ -22,10 +22,12 @@
 
 #include <sys/stat.h>
 
+#include <algorithm>
 #include <cmath>
 #include <string>
 #include <vector>
 
+#include "batched_stream.cuh"
 #include "coarse.cuh"
 #include "launch.h"
 #include "mg_kernels.cuh"
@@ -34,6 +36,7 @@
 namespace npmg {
 
 constexpr int kBThreads = 256;
+constexpr int kBBlocks = 2;  // per SM
 constexpr int kBCoarseCells = 1024;
 
 struct BInst {
@@ -48,6 +51,7 @@ struct BInst {
   ff cff;                // c = h_x^2
   double c, c2;
   int slot0, ntiles0;    // partial-sum slots of the level-0 tiles
+  int wslot0, nstrips0;  // and of the level-0 strips
   int cfloats;           // shared floats of the coarse item
   CoarseArgs ca;
 };
@@ -60,12 +64,14 @@ struct BatchArgs {
   const float* const* xin;   // initial guesses (the outputs, except in the tuner)
   float* const* xout;
   int count;
-  const int4* items[kMaxLevels];  // (instance, tile x, tile y, slot) per level
+  const int4* items[kMaxLevels];  // (instance, tile x, tile y, slot): level 0, and coarser levels off the strips
   int nitems[kMaxLevels];
+  const int4* strips[kMaxLevels]; // (instance, first group and length of a strip, first row, slot) per level
+  int nstrips[kMaxLevels], srows[kMaxLevels];  // and rows per strip
   int ntile_levels;      // max kc over instances
   const int2* citems;    // coarse phase: (instance, first row of a dense product) or (instance, -1)
   int ncitems;
-  double* partials;      // one per level-0 tile
+  double* partials;      // one per level-0 tile, then one per level-0 strip
   unsigned* bar;         // [0] arrivals, [1] generation, [2] error, [4..5] active counts
   int sweeps;
   float omega, s;
@@ -256,12 +262,11 @@ __device__ __noinline__ void b_down_h(const LevelDev& L, int tx, int ty, const f
   }
 }
 
-// up leg of one tile: x + s P e, H sweeps, output; returns this thread's
-// share of (b, out) when `dot`
+// up leg of one tile: x + s P e, H sweeps, output
 template <int TX, int TY, int H>
-__device__ __noinline__ float b_up_h(const LevelDev& L, int tx, int ty, const float* __restrict__ b,
+__device__ __noinline__ void b_up_h(const LevelDev& L, int tx, int ty, const float* __restrict__ b,
                         const float* __restrict__ xin, float* __restrict__ xout, const float* __restrict__ e,
-                        float omega, float s, bool dot, float* S) {
+                        float omega, float s, float* S) {
   using G = BReg<TX, TY, H>;
   const G g(tx, ty);
   const BSmem<TX, TY, H> M(S);
@@ -306,7 +311,6 @@ __device__ __noinline__ float b_up_h(const LevelDev& L, int tx, int ty, const fl
     b_sweep<TX, TY, H, 0>(L, M.s0, M.s1, M.sb, M.sw, omega, false);
     cur = M.s1;
   }
-  float acc = 0.f;
 #pragma unroll
   for (int i = threadIdx.x; i < TX * TY; i += kBThreads) {
     const int lx = i % TX + H, ly = i / TX + H;
@@ -314,23 +318,15 @@ __device__ __noinline__ float b_up_h(const LevelDev& L, int tx, int ty, const fl
     if (gx < L.nx && gy < L.ny) {
       const int li = ly * G::RX + lx;
       xout[(size_t)gy * L.nx + gx] = cur[li];
-      if (dot) acc = fmaf(M.sb[li], cur[li], acc);
     }
   }
-  return acc;
 }
 
 // ---------------------------------------------------------------------------
-// float4 tile path, for a level whose width is a multiple of 4 (every level-0
-// grid; coarser levels while their width stays a multiple of 4).  The region
-// is the tile plus one group of four cells on each side in x and H rows in y,
-// so a global access is a whole float4 (uchar4 for the cell bytes) that is
-// either all on the grid or all off it, and a sweep updates four cells per
-// thread.  A sweep updates every group of its rows: the outermost groups'
-// outer neighbours lie outside the region (a pad float), which spoils one
-// more cell per sweep from the region's x edges inward -- at most H - 1 <= 2
-// cells after the last sweep, so the tile and the one-cell ring around it
-// that the restriction reads stay exact.
+// float4 region of the refinement residual: the level-0 tile plus one group
+// of four cells on each side in x and H rows in y, so a global access is a
+// whole float4 (uchar4 for the cell bytes) that is either all on the grid or
+// all off it (an instance's width is a multiple of 4).
 template <int TX, int TY, int H>
 struct VReg {
   static constexpr int RX = TX + 8, RY = TY + 2 * H, R = RX * RY, W4 = RX / 4, PAD = 4;
@@ -343,22 +339,6 @@ struct VReg {
     const int gx = ox + 4 * (q % W4), gy = oy + q / W4;
     if (q >= NG || gx < 0 || gx >= L.nx || gy < 0 || gy >= L.ny) return -1;
     return gy * L.nx + gx;
-  }
-};
-
-// smem of one float4 tile: b, two iterates, omega / d (padded float arrays),
-// cell bytes
-template <int TX, int TY, int H>
-struct VSmem {
-  float *sb, *s0, *s1, *sw;
-  uint8_t* sm;
-  __device__ __forceinline__ explicit VSmem(float* S) {
-    using G = VReg<TX, TY, H>;
-    sb = S + G::PAD;
-    s0 = sb + G::A;
-    s1 = s0 + G::A;
-    sw = s1 + G::A;
-    sm = reinterpret_cast<uint8_t*>(S + 4 * G::A);
   }
 };
 
@@ -391,273 +371,6 @@ struct VNb {
   __device__ __forceinline__ float left(int k) const { return k == 0 ? l : lane(c, k - 1); }
   __device__ __forceinline__ float right(int k) const { return k == 3 ? r : lane(c, k + 1); }
 };
-
-// one sweep over rows H - M .. H + TY + M - 1 of the region (all groups).
-// Thread t owns group column t % W4 of rows t / W4, t / W4 + RPP, ... (RPP
-// = rows per pass), so no group index is divided.  Cells off the fluid and
-// off the grid hold x = 0 and omega / d = 0, so the update gives them 0
-// with no test.
-template <int TX, int TY, int H, int M>
-__device__ __forceinline__ void v_sweep(const LevelDev& L, const float* __restrict__ xin, float* __restrict__ xout,
-                                        const float* __restrict__ sb, const float* __restrict__ sw, float omega,
-                                        bool from_zero) {
-  using G = VReg<TX, TY, H>;
-  constexpr int RPP = kBThreads / G::W4, NROW = TY + 2 * M, NI = (NROW + RPP - 1) / RPP;
-  const float keep = 1.f - omega;
-  const int c4 = threadIdx.x % G::W4, r0 = threadIdx.x / G::W4;
-  if (r0 < RPP) {
-#pragma unroll
-    for (int j = 0; j < NI; ++j) {
-      const int row = r0 + j * RPP;
-      if (row >= NROW) break;
-      const int li = (row + H - M) * G::RX + 4 * c4;
-      const float4 w = lds4(sw + li), bb = lds4(sb + li);
-      float4 v;
-      if (from_zero) {
-        v = make_float4(w.x * bb.x, w.y * bb.y, w.z * bb.z, w.w * bb.w);
-      } else {
-        const VNb n(xin, li, G::RX);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const float nb = L.wx * (n.left(k) + n.right(k)) + L.wy * (lane(n.d, k) + lane(n.u, k));
-          set_lane(v, k, keep * lane(n.c, k) + lane(w, k) * (lane(bb, k) + nb));
-        }
-      }
-      sts4(xout + li, v);
-    }
-  }
-  __syncthreads();
-}
-
-// b, omega / d and cell bytes of one region group into shared memory
-template <int TX, int TY, int H>
-__device__ __forceinline__ void v_stage(const LevelDev& L, const VReg<TX, TY, H>& g, const VSmem<TX, TY, H>& M,
-                                        int q, uchar4 m4, float4 b4, float omega) {
-  using G = VReg<TX, TY, H>;
-  const int li = (q / G::W4) * G::RX + 4 * (q % G::W4);
-  const int gx = g.ox + 4 * (q % G::W4), gy = g.oy + q / G::W4;
-  float4 sb, sw;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const uint8_t m = lane(m4, k);
-    set_lane(sb, k, m ? lane(b4, k) : 0.f);
-    set_lane(sw, k, m ? __fdividef(omega, b_diag(L, gx + k, gy, m)) : 0.f);
-  }
-  sts4(M.sb + li, sb);
-  sts4(M.sw + li, sw);
-  *reinterpret_cast<uchar4*>(M.sm + li) = m4;
-}
-
-// down leg of one tile, float4 path
-template <int TX, int TY, int H>
-__device__ void v_down(const LevelDev& L, int tx, int ty, const float* __restrict__ b, float* __restrict__ x,
-                       float* __restrict__ bc, float omega, float* S) {
-  using G = VReg<TX, TY, H>;
-  const G g(tx, ty);
-  const VSmem<TX, TY, H> M(S);
-  constexpr int NR = (G::NG + kBThreads - 1) / kBThreads;
-  float4 bv[NR];
-  uchar4 mv[NR];
-#pragma unroll
-  for (int j = 0; j < NR; ++j) {
-    const int gi = g.gidx(L, threadIdx.x + j * kBThreads);
-    mv[j] = v_cells(L, gi);
-    bv[j] = gi < 0 ? make_float4(0.f, 0.f, 0.f, 0.f) : *reinterpret_cast<const float4*>(b + gi);
-  }
-  __syncthreads();
-#pragma unroll
-  for (int j = 0; j < NR; ++j) {
-    const int q = threadIdx.x + j * kBThreads;
-    if (q >= G::NG) break;
-    v_stage(L, g, M, q, mv[j], bv[j], omega);
-  }
-  __syncthreads();
-  v_sweep<TX, TY, H, H>(L, nullptr, M.s0, M.sb, M.sw, omega, true);
-  float* cur = M.s0;
-  if (H >= 2) {
-    v_sweep<TX, TY, H, (H >= 2 ? H - 1 : 1)>(L, M.s0, M.s1, M.sb, M.sw, omega, false);
-    cur = M.s1;
-  }
-  if (H >= 3) {
-    v_sweep<TX, TY, H, 1>(L, M.s1, M.s0, M.sb, M.sw, omega, false);
-    cur = M.s0;
-  }
-  constexpr int T4 = TX / 4;
-#pragma unroll
-  for (int q = threadIdx.x; q < TY * T4; q += kBThreads) {
-    const int row = q / T4, c = q % T4;
-    const int gx = tx * TX + 4 * c, gy = ty * TY + row;
-    if (gx < L.nx && gy < L.ny)
-      *reinterpret_cast<float4*>(x + gy * L.nx + gx) = lds4(cur + (row + H) * G::RX + 4 * (c + 1));
-  }
-  // residual and restriction, two coarse cells (a 4 x 2 block of fine cells)
-  // per thread
-  const int cnx = L.nx / 2, cny = L.ny / 2;
-#pragma unroll
-  for (int q = threadIdx.x; q < (TY / 2) * T4; q += kBThreads) {
-    const int cy = q / T4, c = q % T4;
-    const int gcx = tx * (TX / 2) + 2 * c, gcy = ty * (TY / 2) + cy;
-    if (gcx >= cnx || gcy >= cny) continue;
-    float sum[2] = {0.f, 0.f};
-#pragma unroll
-    for (int ay = 0; ay < 2; ++ay) {
-      const int ly = H + 2 * cy + ay, li = ly * G::RX + 4 * (c + 1);
-      const VNb n(cur, li, G::RX);
-      const float4 b4 = lds4(M.sb + li);
-      const uchar4 m4 = *reinterpret_cast<const uchar4*>(M.sm + li);
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const uint8_t mm = lane(m4, k);
-        if (!mm) continue;
-        const float d = b_diag(L, g.ox + 4 * (c + 1) + k, g.oy + ly, mm);
-        const float nb = L.wx * (n.left(k) + n.right(k)) + L.wy * (lane(n.d, k) + lane(n.u, k));
-        sum[k >> 1] += lane(b4, k) - (d * lane(n.c, k) - nb);
-      }
-    }
-    *reinterpret_cast<float2*>(bc + gcy * cnx + gcx) = make_float2(0.25f * sum[0], 0.25f * sum[1]);
-  }
-}
-
-// up leg of one tile, float4 path: x + s P e, H sweeps, output; returns this
-// thread's share of (b, out) when `dot`
-template <int TX, int TY, int H>
-__device__ float v_up(const LevelDev& L, int tx, int ty, const float* __restrict__ b, const float* __restrict__ xin,
-                      float* __restrict__ xout, const float* __restrict__ e, float omega, float s, bool dot,
-                      float* S) {
-  using G = VReg<TX, TY, H>;
-  const G g(tx, ty);
-  const VSmem<TX, TY, H> M(S);
-  const int cnx = L.nx / 2;
-  constexpr int NR = (G::NG + kBThreads - 1) / kBThreads;
-  float4 xv[NR], bv[NR];
-  float2 ev[NR];
-  uchar4 mv[NR];
-#pragma unroll
-  for (int j = 0; j < NR; ++j) {
-    const int q = threadIdx.x + j * kBThreads;
-    const int gi = g.gidx(L, q);
-    const int gx = g.ox + 4 * (q % G::W4), gy = g.oy + q / G::W4;
-    mv[j] = v_cells(L, gi);
-    xv[j] = gi < 0 ? make_float4(0.f, 0.f, 0.f, 0.f) : *reinterpret_cast<const float4*>(xin + gi);
-    bv[j] = gi < 0 ? make_float4(0.f, 0.f, 0.f, 0.f) : *reinterpret_cast<const float4*>(b + gi);
-    ev[j] = gi < 0 ? make_float2(0.f, 0.f) : *reinterpret_cast<const float2*>(e + (gy >> 1) * cnx + (gx >> 1));
-  }
-  __syncthreads();
-#pragma unroll
-  for (int j = 0; j < NR; ++j) {
-    const int q = threadIdx.x + j * kBThreads;
-    if (q >= G::NG) break;
-    const int li = (q / G::W4) * G::RX + 4 * (q % G::W4);
-    float4 v;
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-      set_lane(v, k, lane(mv[j], k) ? lane(xv[j], k) + s * (k < 2 ? ev[j].x : ev[j].y) : 0.f);
-    sts4(M.s0 + li, v);
-    v_stage(L, g, M, q, mv[j], bv[j], omega);
-  }
-  __syncthreads();
-  float* cur = M.s0;
-  if (H == 1) {
-    v_sweep<TX, TY, H, 0>(L, M.s0, M.s1, M.sb, M.sw, omega, false);
-    cur = M.s1;
-  } else if (H == 2) {
-    v_sweep<TX, TY, H, 1>(L, M.s0, M.s1, M.sb, M.sw, omega, false);
-    v_sweep<TX, TY, H, 0>(L, M.s1, M.s0, M.sb, M.sw, omega, false);
-  } else {
-    v_sweep<TX, TY, H, (H >= 3 ? 2 : 0)>(L, M.s0, M.s1, M.sb, M.sw, omega, false);
-    v_sweep<TX, TY, H, 1>(L, M.s1, M.s0, M.sb, M.sw, omega, false);
-    v_sweep<TX, TY, H, 0>(L, M.s0, M.s1, M.sb, M.sw, omega, false);
-    cur = M.s1;
-  }
-  float acc = 0.f;
-  constexpr int T4 = TX / 4;
-#pragma unroll
-  for (int q = threadIdx.x; q < TY * T4; q += kBThreads) {
-    const int row = q / T4, c = q % T4;
-    const int gx = tx * TX + 4 * c, gy = ty * TY + row;
-    if (gx < L.nx && gy < L.ny) {
-      const int li = (row + H) * G::RX + 4 * (c + 1);
-      const float4 v = lds4(cur + li);
-      *reinterpret_cast<float4*>(xout + gy * L.nx + gx) = v;
-      if (dot) {
-        const float4 bb = lds4(M.sb + li);
-        acc = fmaf(bb.x, v.x, acc);
-        acc = fmaf(bb.y, v.y, acc);
-        acc = fmaf(bb.z, v.z, acc);
-        acc = fmaf(bb.w, v.w, acc);
-      }
-    }
-  }
-  return acc;
-}
-
-// p = z + beta p_old on a level-0 tile and its halo (one group in x, one
-// row in y; staged in shared memory, zero off the fluid and off the grid),
-// then Ap and the thread's share of (p, Ap) on the tile
-template <int TX, int TY>
-__device__ float b_pupdate(const LevelDev& L, int tx, int ty, const float* __restrict__ z,
-                           const float* __restrict__ pold, float* __restrict__ pnew, float* __restrict__ Ap,
-                           float beta, bool first, float* S) {
-  using G = VReg<TX, TY, 1>;
-  const G g(tx, ty);
-  float* sp = S + G::PAD;
-  uint8_t* sm = reinterpret_cast<uint8_t*>(S + G::A);
-  constexpr int NR = (G::NG + kBThreads - 1) / kBThreads;
-  float4 zv[NR], pv[NR];
-  uchar4 mv[NR];
-  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-  for (int j = 0; j < NR; ++j) {
-    const int gi = g.gidx(L, threadIdx.x + j * kBThreads);
-    mv[j] = v_cells(L, gi);
-    zv[j] = gi < 0 ? zero : *reinterpret_cast<const float4*>(z + gi);
-    pv[j] = (gi < 0 || first) ? zero : *reinterpret_cast<const float4*>(pold + gi);
-  }
-  __syncthreads();
-#pragma unroll
-  for (int j = 0; j < NR; ++j) {
-    const int q = threadIdx.x + j * kBThreads;
-    if (q >= G::NG) break;
-    const int li = (q / G::W4) * G::RX + 4 * (q % G::W4);
-    float4 v;
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-      set_lane(v, k, lane(mv[j], k) ? (first ? lane(zv[j], k) : fmaf(beta, lane(pv[j], k), lane(zv[j], k))) : 0.f);
-    sts4(sp + li, v);
-    *reinterpret_cast<uchar4*>(sm + li) = mv[j];
-  }
-  __syncthreads();
-  float acc = 0.f;
-  constexpr int T4 = TX / 4;
-#pragma unroll
-  for (int q = threadIdx.x; q < TY * T4; q += kBThreads) {
-    const int row = q / T4, c = q % T4;
-    const int gx = tx * TX + 4 * c, gy = ty * TY + row;
-    if (gx >= L.nx || gy >= L.ny) continue;
-    const int li = (row + 1) * G::RX + 4 * (c + 1);
-    const VNb n(sp, li, G::RX);
-    const uchar4 m4 = *reinterpret_cast<const uchar4*>(sm + li);
-    float4 pc = zero, ap = zero;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const uint8_t m = lane(m4, k);
-      if (!m) continue;
-      const float p = lane(n.c, k);
-      float nb = 0.f;
-      nb += L.wx * n.left(k);
-      nb += L.wx * n.right(k);
-      nb += L.wy * lane(n.d, k);
-      nb += L.wy * lane(n.u, k);
-      const float a = b_diag(L, gx + k, gy, m) * p - nb;
-      set_lane(pc, k, p);
-      set_lane(ap, k, a);
-      acc = fmaf(p, a, acc);
-    }
-    *reinterpret_cast<float4*>(pnew + gy * L.nx + gx) = pc;
-    *reinterpret_cast<float4*>(Ap + gy * L.nx + gx) = ap;
-  }
-  return acc;
-}
 
 // d += alpha p (d = alpha p on the first iteration), r -= alpha Ap on a
 // level-0 tile, four cells per access; returns the thread's share of ||r||^2
@@ -697,34 +410,53 @@ __device__ float b_xr(const LevelDev& L, int tx, int ty, float* __restrict__ d, 
   return acc;
 }
 
+// legs of a level whose width is not a multiple of 4 (tiles), and of one item
+// of any other level (a strip of rows, one warp)
 template <int TX, int TY>
 __device__ __forceinline__ void b_down(const LevelDev& L, int tx, int ty, const float* __restrict__ b,
                                        float* __restrict__ x, float* __restrict__ bc, int sweeps, float omega,
                                        float* S) {
-  if ((L.nx & 3) == 0) {
-    if (sweeps <= 1) v_down<TX, TY, 1>(L, tx, ty, b, x, bc, omega, S);
-    else if (sweeps == 2) v_down<TX, TY, 2>(L, tx, ty, b, x, bc, omega, S);
-    else v_down<TX, TY, 3>(L, tx, ty, b, x, bc, omega, S);
-  } else {
-    if (sweeps <= 1) b_down_h<TX, TY, 1>(L, tx, ty, b, x, bc, omega, S);
-    else if (sweeps == 2) b_down_h<TX, TY, 2>(L, tx, ty, b, x, bc, omega, S);
-    else b_down_h<TX, TY, 3>(L, tx, ty, b, x, bc, omega, S);
-  }
+  if (sweeps <= 1) b_down_h<TX, TY, 1>(L, tx, ty, b, x, bc, omega, S);
+  else if (sweeps == 2) b_down_h<TX, TY, 2>(L, tx, ty, b, x, bc, omega, S);
+  else b_down_h<TX, TY, 3>(L, tx, ty, b, x, bc, omega, S);
 }
 
 template <int TX, int TY>
-__device__ __forceinline__ float b_up(const LevelDev& L, int tx, int ty, const float* __restrict__ b,
+__device__ __forceinline__ void b_up(const LevelDev& L, int tx, int ty, const float* __restrict__ b,
+                                     const float* __restrict__ xin, float* __restrict__ xout,
+                                     const float* __restrict__ e, int sweeps, float omega, float s, float* S) {
+  if (sweeps <= 1) b_up_h<TX, TY, 1>(L, tx, ty, b, xin, xout, e, omega, s, S);
+  else if (sweeps == 2) b_up_h<TX, TY, 2>(L, tx, ty, b, xin, xout, e, omega, s, S);
+  else b_up_h<TX, TY, 3>(L, tx, ty, b, xin, xout, e, omega, s, S);
+}
+
+struct Strip {
+  int u0, u1, y0, y1;  // groups of four cells, rows
+  __device__ __forceinline__ Strip(const int4& item, const LevelDev& L, int rows)
+      : u0((int)((unsigned)item.y >> 5)), u1(u0 + 1 + (item.y & 31)), y0(item.z), y1(min(item.z + rows, L.ny)) {}
+};
+
+__device__ __forceinline__ void s_down(const LevelDev& L, const Strip& t, const float* __restrict__ b,
+                                       float* __restrict__ x, float* __restrict__ bc, int sweeps, float omega,
+                                       unsigned char* ring) {
+  if (sweeps <= 1) s_down<1>(L, t.u0, t.u1, t.y0, t.y1, b, x, bc, omega, ring);
+  else if (sweeps == 2) s_down<2>(L, t.u0, t.u1, t.y0, t.y1, b, x, bc, omega, ring);
+  else s_down<3>(L, t.u0, t.u1, t.y0, t.y1, b, x, bc, omega, ring);
+}
+
+__device__ __forceinline__ float s_up(const LevelDev& L, const Strip& t, const float* __restrict__ b,
                                       const float* __restrict__ xin, float* __restrict__ xout,
-                                      const float* __restrict__ e, int sweeps, float omega, float s, bool dot,
-                                      float* S) {
-  if ((L.nx & 3) == 0) {
-    if (sweeps <= 1) return v_up<TX, TY, 1>(L, tx, ty, b, xin, xout, e, omega, s, dot, S);
-    if (sweeps == 2) return v_up<TX, TY, 2>(L, tx, ty, b, xin, xout, e, omega, s, dot, S);
-    return v_up<TX, TY, 3>(L, tx, ty, b, xin, xout, e, omega, s, dot, S);
-  }
-  if (sweeps <= 1) return b_up_h<TX, TY, 1>(L, tx, ty, b, xin, xout, e, omega, s, dot, S);
-  if (sweeps == 2) return b_up_h<TX, TY, 2>(L, tx, ty, b, xin, xout, e, omega, s, dot, S);
-  return b_up_h<TX, TY, 3>(L, tx, ty, b, xin, xout, e, omega, s, dot, S);
+                                      const float* __restrict__ e, int sweeps, float omega, float s,
+                                      unsigned char* ring) {
+  if (sweeps <= 1) return s_up<1>(L, t.u0, t.u1, t.y0, t.y1, b, xin, xout, e, omega, s, ring);
+  if (sweeps == 2) return s_up<2>(L, t.u0, t.u1, t.y0, t.y1, b, xin, xout, e, omega, s, ring);
+  return s_up<3>(L, t.u0, t.u1, t.y0, t.y1, b, xin, xout, e, omega, s, ring);
+}
+
+__device__ __forceinline__ void warp_partial(const BatchArgs& A, int slot, float acc) {
+  double t = (double)acc;
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(kFull, t, o);
+  if ((threadIdx.x & 31) == 0) A.partials[slot] = t;
 }
 
 // ---------------------------------------------------------------------------
@@ -870,10 +602,10 @@ __device__ __forceinline__ double block_total(float v) {
   return tot;
 }
 
-// per-instance fixed-order reduction of the level-0 tile partial slots
-__device__ __forceinline__ double reduce_slots(const BatchArgs& A, const BInst& I) {
+// per-instance fixed-order reduction of the level-0 partial slots
+__device__ __forceinline__ double reduce_slots(const BatchArgs& A, int slot0, int n) {
   double acc = 0.0;
-  for (int j = threadIdx.x; j < I.ntiles0; j += blockDim.x) acc += __ldcg(A.partials + I.slot0 + j);
+  for (int j = threadIdx.x; j < n; j += blockDim.x) acc += __ldcg(A.partials + slot0 + j);
   __shared__ double sh[32];
   __shared__ double tot;
   const double t = block_sum(acc, sh);
@@ -912,13 +644,16 @@ __device__ __forceinline__ void count_active(const BatchArgs& A, int slot, bool 
 }
 
 template <int TX, int TY>
-__global__ void __launch_bounds__(kBThreads, 4) k_batched(const __grid_constant__ BatchArgs A) {
+__global__ void __launch_bounds__(kBThreads, kBBlocks) k_batched(const __grid_constant__ BatchArgs A) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float* S = reinterpret_cast<float*>(smem_raw);
   unsigned epoch = 0;
   int cslot = 0;
   const int4* it0 = A.items[0];
   const int n0 = A.nitems[0];
+  // a warp's place among the strips: consecutive ones on different SMs
+  const int wid = (int)(threadIdx.x >> 5) * (int)gridDim.x + (int)blockIdx.x, nw = (int)gridDim.x * (kBThreads / 32);
+  unsigned char* ring = smem_raw + (threadIdx.x >> 5) * kSRing;
   const float omega = A.omega;
   // ---- init: x = (guess, 0) on fluid cells, ||b||^2 per tile
   for (int w = blockIdx.x; w < n0; w += gridDim.x) {
@@ -942,7 +677,7 @@ __global__ void __launch_bounds__(kBThreads, 4) k_batched(const __grid_constant_
   if (!grid_barrier(A, epoch)) return;
   for (int w = blockIdx.x; w < A.count; w += gridDim.x) {
     const BInst& I = A.inst[w];
-    const double tot = reduce_slots(A, I);
+    const double tot = reduce_slots(A, I.slot0, I.ntiles0);
     if (threadIdx.x == 0) {
       SolveParams prm = A.prm;
       prm.n_fluid = I.nfluid > 0 ? I.nfluid : 1;
@@ -1006,7 +741,7 @@ __global__ void __launch_bounds__(kBThreads, 4) k_batched(const __grid_constant_
       SolveState& st = A.st[w];
       if (st.outer_done) continue;
       const BInst& I = A.inst[w];
-      const double tot = reduce_slots(A, I);
+      const double tot = reduce_slots(A, I.slot0, I.ntiles0);
       if (threadIdx.x == 0) {
         const double sig_old_d = st.sigma;
         const double sig_new_d =
@@ -1027,12 +762,19 @@ __global__ void __launch_bounds__(kBThreads, 4) k_batched(const __grid_constant_
     for (int iter = 0; iter < A.prm.max_inner; ++iter) {
       // down legs, level by level
       for (int k = 0; k < A.ntile_levels; ++k) {
+        for (int w = wid; w < A.nstrips[k]; w += nw) {
+          const int4 item = A.strips[k][w];
+          if (A.st[item.x].inner_done) continue;
+          const BInst& I = A.inst[item.x];
+          const LevelDev L = I.lv[k];
+          s_down(L, Strip(item, L, A.srows[k]), k == 0 ? I.r : I.b[k], I.x[k], I.b[k + 1], A.sweeps, omega, ring);
+        }
         const int4* its = A.items[k];
-        for (int w = blockIdx.x; w < A.nitems[k]; w += gridDim.x) {
+        for (int w = blockIdx.x; k > 0 && w < A.nitems[k]; w += gridDim.x) {
           const int4 item = its[w];
           if (A.st[item.x].inner_done) continue;
           const BInst& I = A.inst[item.x];
-          b_down<TX, TY>(I.lv[k], item.y, item.z, k == 0 ? I.r : I.b[k], I.x[k], I.b[k + 1], A.sweeps, omega, S);
+          b_down<TX, TY>(I.lv[k], item.y, item.z, I.b[k], I.x[k], I.b[k + 1], A.sweeps, omega, S);
         }
         if (!grid_barrier(A, epoch)) return;
       }
@@ -1049,17 +791,21 @@ __global__ void __launch_bounds__(kBThreads, 4) k_batched(const __grid_constant_
       if (!grid_barrier(A, epoch)) return;
       // up legs; the finest produces z = M r and (r, z)
       for (int k = A.ntile_levels - 1; k >= 0; --k) {
+        for (int w = wid; w < A.nstrips[k]; w += nw) {
+          const int4 item = A.strips[k][w];
+          if (A.st[item.x].inner_done) continue;
+          const BInst& I = A.inst[item.x];
+          const LevelDev L = I.lv[k];
+          const float acc = s_up(L, Strip(item, L, A.srows[k]), k == 0 ? I.r : I.b[k], I.x[k], k == 0 ? I.z : I.y[k],
+                                 I.y[k + 1], A.sweeps, omega, A.s, ring);
+          if (k == 0) warp_partial(A, item.w, acc);
+        }
         const int4* its = A.items[k];
-        for (int w = blockIdx.x; w < A.nitems[k]; w += gridDim.x) {
+        for (int w = blockIdx.x; k > 0 && w < A.nitems[k]; w += gridDim.x) {
           const int4 item = its[w];
           if (A.st[item.x].inner_done) continue;
           const BInst& I = A.inst[item.x];
-          const float acc = b_up<TX, TY>(I.lv[k], item.y, item.z, k == 0 ? I.r : I.b[k], I.x[k],
-                                         k == 0 ? I.z : I.y[k], I.y[k + 1], A.sweeps, omega, A.s, k == 0, S);
-          if (k == 0) {
-            const double t = block_total(acc);
-            if (threadIdx.x == 0) A.partials[item.w] = t;
-          }
+          b_up<TX, TY>(I.lv[k], item.y, item.z, I.b[k], I.x[k], I.y[k], I.y[k + 1], A.sweeps, omega, A.s, S);
         }
         if (!grid_barrier(A, epoch)) return;
       }
@@ -1068,7 +814,7 @@ __global__ void __launch_bounds__(kBThreads, 4) k_batched(const __grid_constant_
         SolveState& st = A.st[w];
         if (st.inner_done) continue;
         const BInst& I = A.inst[w];
-        const double tot = reduce_slots(A, I);
+        const double tot = reduce_slots(A, I.wslot0, I.nstrips0);
         if (threadIdx.x == 0) {
           st.rz = tot;
           st.beta = (st.first || !st.krylov) ? 0.0 : tot / st.rz_old;
@@ -1077,24 +823,25 @@ __global__ void __launch_bounds__(kBThreads, 4) k_batched(const __grid_constant_
       }
       if (!grid_barrier(A, epoch)) return;
       // p = z + beta p, Ap, (p, Ap)
-      for (int w = blockIdx.x; w < n0; w += gridDim.x) {
-        const int4 item = it0[w];
+      for (int w = wid; w < A.nstrips[0]; w += nw) {
+        const int4 item = A.strips[0][w];
         const SolveState& st = A.st[item.x];
         if (st.inner_done) continue;
         const BInst& I = A.inst[item.x];
+        const LevelDev L = I.lv[0];
         const bool first = st.first || !st.krylov;
         const float beta = first ? 0.f : (float)st.beta;
         const float* pold = (st.it & 1) ? I.p1 : I.p0;
         float* pnew = (st.it & 1) ? I.p0 : I.p1;
-        const float acc = b_pupdate<TX, TY>(I.lv[0], item.y, item.z, I.z, pold, pnew, I.Ap, beta, first, S);
-        const double t = block_total(acc);
-        if (threadIdx.x == 0) A.partials[item.w] = t;
+        const Strip t(item, L, A.srows[0]);
+        warp_partial(A, item.w,
+                     s_pupdate(L, t.u0, t.u1, t.y0, t.y1, I.z, pold, pnew, I.Ap, beta, first, ring));
       }
       if (!grid_barrier(A, epoch)) return;
       for (int w = blockIdx.x; w < A.count; w += gridDim.x) {
         SolveState& st = A.st[w];
         if (st.inner_done) continue;
-        const double tot = reduce_slots(A, A.inst[w]);
+        const double tot = reduce_slots(A, A.inst[w].wslot0, A.inst[w].nstrips0);
         if (threadIdx.x == 0) {
           st.pAp = tot;
           st.alpha = st.krylov ? st.rz / tot : 1.0;
@@ -1117,7 +864,7 @@ __global__ void __launch_bounds__(kBThreads, 4) k_batched(const __grid_constant_
       for (int w = blockIdx.x; w < A.count; w += gridDim.x) {
         SolveState& st = A.st[w];
         if (st.inner_done) continue;
-        const double tot = reduce_slots(A, A.inst[w]);
+        const double tot = reduce_slots(A, A.inst[w].slot0, A.inst[w].ntiles0);
         if (threadIdx.x == 0) inner_decide(&st, tot);
         __syncthreads();
         count_active(A, cslot, !st.inner_done);
@@ -1191,7 +938,9 @@ struct mg_batch_s {
   float** d_xout;
   const float** d_xin;           // guesses read by the init phase
   void** h_ptrs;                 // pinned staging of the pointer tables
-  std::vector<int4*> d_items;
+  std::vector<int4*> d_items, d_strips;
+  int nstrips[kMaxLevels], srows[kMaxLevels];
+  int strip_slot0;               // first partial slot of the strips
   int2* d_citems;
   int ncitems;
   int nitems[kMaxLevels];
@@ -1213,13 +962,14 @@ struct mg_batch_s {
 
 static size_t batched_smem(int tx, int ty, int sweeps, size_t coarse_bytes) {
   const int h = sweeps < 1 ? 1 : (sweeps > 3 ? 3 : sweeps);
-  // scalar tile: halo h on every side; float4 tile: one group of 4 in x and
-  // h rows in y, arrays padded by 4 floats at both ends
-  const size_t R = (size_t)(tx + 2 * h) * (ty + 2 * h), Rv = (size_t)(tx + 8) * (ty + 2 * h);
-  const size_t t = 4 * R * 4 + ((R + 15) & ~size_t(15));  // b, two iterates, omega/d; cell bytes
-  const size_t tv = 4 * (Rv + 8) * 4 + ((Rv + 15) & ~size_t(15));
-  size_t m = t > tv ? t : tv;
-  return m > coarse_bytes ? m : coarse_bytes;
+  // scalar tile: halo h on every side; the residual's tile: one group of four
+  // in x and one row in y, (hi, lo) planes padded by 4 floats at both ends;
+  // the warps' rings
+  const size_t R = (size_t)(tx + 2 * h) * (ty + 2 * h), Rv = (size_t)(tx + 8) * (ty + 2);
+  size_t m = 4 * R * 4 + ((R + 15) & ~size_t(15));  // b, two iterates, omega/d; cell bytes
+  m = std::max(m, 2 * (Rv + 8) * 4 + ((Rv + 15) & ~size_t(15)));
+  m = std::max(m, (size_t)(kBThreads / 32) * kSRing);
+  return std::max(m, coarse_bytes);
 }
 
 static std::string tune_cache_path() {
@@ -1270,6 +1020,9 @@ static mg_status batched_launch(mg_batch_s* B, int tile, int sweeps, double tol,
   for (int k = 0; k < kMaxLevels; ++k) {
     A.items[k] = k < (int)B->d_items.size() ? B->d_items[k] : nullptr;
     A.nitems[k] = B->nitems[k];
+    A.strips[k] = k < (int)B->d_strips.size() ? B->d_strips[k] : nullptr;
+    A.nstrips[k] = B->nstrips[k];
+    A.srows[k] = B->srows[k];
   }
   A.ntile_levels = B->ntile_levels;
   A.citems = B->d_citems;
@@ -1330,6 +1083,13 @@ static mg_status batched_launch(mg_batch_s* B, int tile, int sweeps, double tol,
 }
 
 static mg_status build_items(mg_batch_s* B, int tile, cudaStream_t s);
+
+// Strips of a level: at most 32 groups of four cells, of which one at each
+// inner edge belongs to the neighbour; runs of rows, chosen per level so that
+// the warps' rounds times the rows walked (the halo rows and about six rows'
+// time of latency at a run's start included) are fewest.
+constexpr int kStripRows[] = {8, 16, 32, 64, 128};
+static int strip_count(int nx) { return nx <= 128 ? 1 : (nx / 4 + 29) / 30; }
 
 extern "C" {
 
@@ -1466,6 +1226,9 @@ mg_status mg_create_batched(mg_batch* out, int count, const int64_t* shapes, con
   // partial slots: worst case over tile shapes = the smallest tile (32 x 16)
   long long max_slots = 0;
   for (int i = 0; i < count; ++i) max_slots += (long long)((B->inst[i].nx + 31) / 32) * ((B->inst[i].ny + 15) / 16);
+  B->strip_slot0 = (int)max_slots;
+  for (int i = 0; i < count; ++i)
+    max_slots += (long long)strip_count(B->inst[i].nx) * ((B->inst[i].ny + kStripRows[0] - 1) / kStripRows[0]);
   const size_t off_partials = reserve((size_t)max_slots * 8);
   const size_t off_bar = reserve(64);
   cudaError_t ce = cudaMalloc((void**)&B->pool, bytes);
@@ -1583,7 +1346,7 @@ mg_status mg_create_batched(mg_batch* out, int count, const int64_t* shapes, con
         st = MG_ERR_INVALID;
         goto fail;
       }
-      B->grid[t][sw] = B->nsm * (per_sm > 4 ? 4 : per_sm);
+      B->grid[t][sw] = B->nsm * (per_sm > kBBlocks ? kBBlocks : per_sm);
     }
   {
     char name[256] = {0};
@@ -1622,6 +1385,7 @@ static mg_status build_items(mg_batch_s* B, int tile, cudaStream_t s) {
     I.slot0 = slot;
     for (int k = 0; k < I.kc; ++k) {
       const int nx = I.lv[k].nx, ny = I.lv[k].ny;
+      if (k > 0 && nx % 4 == 0) continue;  // strips
       for (int ty = 0; ty < (ny + TY - 1) / TY; ++ty)
         for (int tx = 0; tx < (nx + TX - 1) / TX; ++tx) items[k].push_back(make_int4(i, tx, ty, k == 0 ? slot++ : -1));
     }
@@ -1635,7 +1399,40 @@ static mg_status build_items(mg_batch_s* B, int tile, cudaStream_t s) {
         B->graph[t][k] = nullptr;
       }
   for (int4* p : B->d_items) cudaFree(p);
+  for (int4* p : B->d_strips) cudaFree(p);
   B->d_items.assign(kMaxLevels, nullptr);
+  B->d_strips.assign(kMaxLevels, nullptr);
+  for (int k = 0; k < kMaxLevels; ++k) {
+    const long long warps = (long long)B->grid[tile][B->sweeps] * (kBThreads / 32);
+    long long best = 0;
+    B->srows[k] = kStripRows[0];
+    for (int rows : kStripRows) {
+      long long n = 0;
+      for (const BInst& I : B->inst)
+        if (k < I.kc && I.lv[k].nx % 4 == 0) n += (long long)strip_count(I.lv[k].nx) * ((I.lv[k].ny + rows - 1) / rows);
+      const long long cost = (n + warps - 1) / warps * (rows + 2 * B->sweeps + 6);
+      if (best == 0 || cost < best) {
+        best = cost;
+        B->srows[k] = rows;
+      }
+    }
+  }
+  std::vector<std::vector<int4>> strips(kMaxLevels);
+  slot = B->strip_slot0;
+  for (int i = 0; i < B->count; ++i) {
+    BInst& I = B->inst[i];
+    I.wslot0 = slot;
+    for (int k = 0; k < I.kc; ++k) {
+      const int nx = I.lv[k].nx, ny = I.lv[k].ny, n = strip_count(nx);
+      if (nx % 4) continue;
+      for (int y = 0; y < ny; y += B->srows[k])
+        for (int j = 0; j < n; ++j) {
+          const unsigned u0 = (unsigned)((long long)(nx / 4) * j / n), u1 = (unsigned)((long long)(nx / 4) * (j + 1) / n);
+          strips[k].push_back(make_int4(i, (int)(u0 << 5 | (u1 - u0 - 1)), y, k == 0 ? slot++ : -1));
+        }
+    }
+    I.nstrips0 = slot - I.wslot0;
+  }
   if (!B->d_citems) {
     std::vector<int2> ci;
     for (int i = 0; i < B->count; ++i) {
@@ -1652,6 +1449,12 @@ static mg_status build_items(mg_batch_s* B, int tile, cudaStream_t s) {
   }
   for (int k = 0; k < kMaxLevels; ++k) {
     B->nitems[k] = (int)items[k].size();
+    B->nstrips[k] = (int)strips[k].size();
+    if (!strips[k].empty()) {
+      NPMG_CUDA(cudaMalloc((void**)&B->d_strips[k], strips[k].size() * sizeof(int4)));
+      NPMG_CUDA(cudaMemcpyAsync(B->d_strips[k], strips[k].data(), strips[k].size() * sizeof(int4),
+                                cudaMemcpyHostToDevice, s));
+    }
     if (items[k].empty()) continue;
     NPMG_CUDA(cudaMalloc((void**)&B->d_items[k], items[k].size() * sizeof(int4)));
     NPMG_CUDA(cudaMemcpyAsync(B->d_items[k], items[k].data(), items[k].size() * sizeof(int4), cudaMemcpyHostToDevice,
@@ -1832,6 +1635,7 @@ mg_status mg_destroy_batched(mg_batch B) {
       if (B->graph[t][k]) cudaGraphExecDestroy(B->graph[t][k]);
   if (B->d_citems) cudaFree(B->d_citems);
   for (int4* p : B->d_items) cudaFree(p);
+  for (int4* p : B->d_strips) cudaFree(p);
   if (B->pool) cudaFree(B->pool);
   if (B->d_inst) cudaFree(B->d_inst);
   if (B->d_st) cudaFree(B->d_st);

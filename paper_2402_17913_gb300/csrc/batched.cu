@@ -758,7 +758,9 @@ __global__ void __launch_bounds__(kBThreads, kBBlocks) k_batched(const __grid_co
     const unsigned active_outer = *(volatile unsigned*)(A.bar + 4 + cslot);
     cslot ^= 1;
     if (active_outer == 0) break;
-    // ---- CG iterations
+    // ---- CG iterations.  The phases over a level walk the list of strips (or
+    // tiles) up and down in turn, so that each starts where the one before it
+    // ended, on what the L2 still holds of it.
     for (int iter = 0; iter < A.prm.max_inner; ++iter) {
       // down legs, level by level
       for (int k = 0; k < A.ntile_levels; ++k) {
@@ -792,7 +794,7 @@ __global__ void __launch_bounds__(kBThreads, kBBlocks) k_batched(const __grid_co
       // up legs; the finest produces z = M r and (r, z)
       for (int k = A.ntile_levels - 1; k >= 0; --k) {
         for (int w = wid; w < A.nstrips[k]; w += nw) {
-          const int4 item = A.strips[k][w];
+          const int4 item = A.strips[k][A.nstrips[k] - 1 - w];
           if (A.st[item.x].inner_done) continue;
           const BInst& I = A.inst[item.x];
           const LevelDev L = I.lv[k];
@@ -850,7 +852,7 @@ __global__ void __launch_bounds__(kBThreads, kBBlocks) k_batched(const __grid_co
       if (!grid_barrier(A, epoch)) return;
       // d += alpha p, r -= alpha Ap, ||r||^2
       for (int w = blockIdx.x; w < n0; w += gridDim.x) {
-        const int4 item = it0[w];
+        const int4 item = it0[n0 - 1 - w];
         const SolveState& st = A.st[item.x];
         if (st.inner_done) continue;
         const BInst& I = A.inst[item.x];

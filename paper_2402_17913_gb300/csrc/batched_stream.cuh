@@ -11,11 +11,13 @@
 // more of its cells from the outside, at most three of four, and the fourth
 // is all the strip's own cells need.
 //
-// What bounds it: issue slots and memory about equally (140 to 160
-// instructions per row of 128 cells against 0.6 to 1.8 KB).  The block tiles
-// it replaced staged a 72 x 38 region for 64 x 32 cells behind seven block
-// barriers, 6 us a tile at four blocks per SM: 256 instances of sides 64 to
-// 512, three sweeps, 28.1 -> 21.0 ms a solve.
+// What bounds it: 256 instances of sides 64 to 512, three sweeps: the p and
+// x / r updates run at the copy rate, the two finest legs at 0.6 of it (four
+// warps per scheduler at 128 registers, about seven cycles an issue; three
+// blocks per SM at 80 registers spill: 36 ms).  The block tiles before staged
+// 72 x 38 cells for 64 x 32 behind seven block barriers, 6 us a tile at four
+// blocks per SM: 28.1 -> 21.0 ms a solve, -> 19.7 with paired arithmetic and
+// with the phases walking the list up and down in turn.
 #pragma once
 
 #include "npmg_internal.cuh"
@@ -77,49 +79,76 @@ __device__ __forceinline__ unsigned s_cells(const LevelDev& L, const SLane& c, i
 }
 __device__ __forceinline__ unsigned s_byte(unsigned m, int j) { return (m >> (8 * j)) & 0xffu; }
 
-// values beside the lane's first and last cell: 0 beyond the warp, which is
-// the level's edge or the spoilt side of a halo lane
-__device__ __forceinline__ void s_edges(const SLane& c, const float (&a)[4], float& left, float& right) {
-  left = __shfl_up_sync(kFull, a[3], 1);
-  right = __shfl_down_sync(kFull, a[0], 1);
+// The four cells of a lane as two pairs: a pair's multiply-add is one
+// instruction (fma.rn.f32x2), and issue slots are what the sweeps run out of.
+struct Quad {
+  float2 a, b;
+  __device__ __forceinline__ float2 pair(int q) const { return q ? b : a; }
+  __device__ __forceinline__ float get(int j) const { return j == 0 ? a.x : j == 1 ? a.y : j == 2 ? b.x : b.y; }
+  __device__ __forceinline__ void set(int j, float v) {
+    if (j == 0) a.x = v;
+    else if (j == 1) a.y = v;
+    else if (j == 2) b.x = v;
+    else b.y = v;
+  }
+};
+__device__ __forceinline__ float2 s_dup(float v) { return make_float2(v, v); }
+
+// sums of the two neighbours in x of each cell of a row: 0 beyond the warp,
+// which is the level's edge or the spoilt side of a halo lane
+__device__ __forceinline__ Quad s_xsum(const SLane& c, const Quad& v) {
+  float left = __shfl_up_sync(kFull, v.b.y, 1);
+  float right = __shfl_down_sync(kFull, v.a.x, 1);
   if (c.lane == 0) left = 0.f;
   if (c.lane == 31) right = 0.f;
+  Quad o;
+  o.a = make_float2(left + v.a.y, v.a.x + v.b.x);
+  o.b = make_float2(v.a.y + v.b.y, v.b.x + right);
+  return o;
 }
 
-// one sweep on row a between rows dn and up
-__device__ __forceinline__ void s_sweep(const LevelDev& L, const SLane& c, float keep, const float (&dn)[4],
-                                        const float (&a)[4], const float (&up)[4], const float (&b)[4],
-                                        const float (&w)[4], float (&out)[4]) {
-  float left, right;
-  s_edges(c, a, left, right);
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const float l = j == 0 ? left : a[j - 1], r = j == 3 ? right : a[j + 1];
-    const float nb = L.wx * (l + r) + L.wy * (dn[j] + up[j]);
-    out[j] = keep * a[j] + w[j] * (b[j] + nb);
-  }
+// f + wx (left + right) + wy (below + above)
+__device__ __forceinline__ Quad s_stencil(const SLane& c, float2 wx, float2 wy, const Quad& f, const Quad& dn,
+                                          const Quad& v, const Quad& up) {
+  const Quad x = s_xsum(c, v);
+  Quad o;
+  o.a = __ffma2_rn(wx, x.a, __ffma2_rn(wy, __fadd2_rn(dn.a, up.a), f.a));
+  o.b = __ffma2_rn(wx, x.b, __ffma2_rn(wy, __fadd2_rn(dn.b, up.b), f.b));
+  return o;
 }
 
-__device__ __forceinline__ void s_put(float* p, const float (&v)[4]) {
-  *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+// one sweep on row v between rows dn and up
+__device__ __forceinline__ Quad s_sweep(const SLane& c, float2 wx, float2 wy, float2 keep, const Quad& dn,
+                                        const Quad& v, const Quad& up, const Quad& b, const Quad& w) {
+  const Quad t = s_stencil(c, wx, wy, b, dn, v, up);
+  Quad o;
+  o.a = __ffma2_rn(w.a, t.a, __fmul2_rn(keep, v.a));
+  o.b = __ffma2_rn(w.b, t.b, __fmul2_rn(keep, v.b));
+  return o;
 }
-__device__ __forceinline__ void s_get(const unsigned char* p, float (&v)[4]) {
+
+__device__ __forceinline__ void s_put(float* p, const Quad& v) {
+  *reinterpret_cast<float4*>(p) = make_float4(v.a.x, v.a.y, v.b.x, v.b.y);
+}
+__device__ __forceinline__ Quad s_get(const unsigned char* p) {
   const float4 q = *reinterpret_cast<const float4*>(p);
-  v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+  return Quad{make_float2(q.x, q.y), make_float2(q.z, q.w)};
+}
+__device__ __forceinline__ Quad s_table(const SLane& c, float entry, unsigned m) {
+  Quad o;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) o.set(j, __shfl_sync(kFull, entry, (int)(s_byte(m, j) & 15u)));
+  return o;
 }
 template <int N>
-__device__ __forceinline__ void s_shift(float (&a)[N][4]) {
+__device__ __forceinline__ void s_shift(Quad (&a)[N]) {
 #pragma unroll
-  for (int k = 0; k + 1 < N; ++k)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) a[k][j] = a[k + 1][j];
+  for (int k = 0; k + 1 < N; ++k) a[k] = a[k + 1];
 }
 template <int N>
-__device__ __forceinline__ void s_zero(float (&a)[N][4]) {
+__device__ __forceinline__ void s_zero(Quad (&a)[N]) {
 #pragma unroll
-  for (int k = 0; k < N; ++k)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) a[k][j] = 0.f;
+  for (int k = 0; k < N; ++k) a[k].a = a[k].b = make_float2(0.f, 0.f);
 }
 
 // Walks rows p = y0 - halo .. y1 + halo - 1 (an even count): issue(p, slot)
@@ -153,10 +182,10 @@ __device__ __forceinline__ void s_down(const LevelDev& L, int u0, int u1, int y0
                                        float* __restrict__ x, float* __restrict__ bc, float omega,
                                        unsigned char* ring) {
   const SLane c = s_lane(L, u0, u1, omega);
-  const float keep = 1.f - omega;
+  const float2 wx = s_dup(L.wx), wy = s_dup(L.wy), keep = s_dup(1.f - omega);
   const int cnx = L.nx >> 1;
   // index H (or 2) is the newest row; xs[k] holds the rows after sweep k + 1
-  float bq[H + 1][4], wq[H + 1][4], xs[H][3][4];
+  Quad bq[H + 1], wq[H + 1], xs[H][3];
   unsigned mq[H + 1];
   float rp0 = 0.f, rp1 = 0.f;
   s_zero(bq);
@@ -180,29 +209,22 @@ __device__ __forceinline__ void s_down(const LevelDev& L, int u0, int u1, int y0
         for (int k = 0; k < H; ++k) s_shift(xs[k]);
 #pragma unroll
         for (int k = 0; k < H; ++k) mq[k] = mq[k + 1];
-        s_get(slot + c.lane * 16, bq[H]);
+        bq[H] = s_get(slot + c.lane * 16);
         mq[H] = s_cells(L, c, p, slot + 512);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          wq[H][j] = __shfl_sync(kFull, c.tabw, (int)(s_byte(mq[H], j) & 15u));
-          xs[0][2][j] = wq[H][j] * bq[H][j];
-        }
+        wq[H] = s_table(c, c.tabw, mq[H]);
+        xs[0][2].a = __fmul2_rn(wq[H].a, bq[H].a);
+        xs[0][2].b = __fmul2_rn(wq[H].b, bq[H].b);
 #pragma unroll
         for (int k = 1; k < H; ++k)
-          s_sweep(L, c, keep, xs[k - 1][0], xs[k - 1][1], xs[k - 1][2], bq[H - k], wq[H - k], xs[k][2]);
-        // row o: x and its residual, pairs of cells summed; the coarse cells
-        // are written on the odd row
+          xs[k][2] = s_sweep(c, wx, wy, keep, xs[k - 1][0], xs[k - 1][1], xs[k - 1][2], bq[H - k], wq[H - k]);
+        // row o: x and its residual b + nb - d x, pairs of cells summed; the
+        // coarse cells are written on the odd row
         const int o = p - H;
-        const float(&v)[3][4] = xs[H - 1];
-        float left, right, r[4];
-        s_edges(c, v[1], left, right);
+        const Quad(&v)[3] = xs[H - 1];
+        const Quad d = s_table(c, c.tabd, mq[0]), t = s_stencil(c, wx, wy, bq[0], v[0], v[1], v[2]);
+        float r[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const float l = j == 0 ? left : v[1][j - 1], rr = j == 3 ? right : v[1][j + 1];
-          const float d = __shfl_sync(kFull, c.tabd, (int)(s_byte(mq[0], j) & 15u));
-          const float nb = L.wx * (l + rr) + L.wy * (v[0][j] + v[2][j]);
-          r[j] = s_byte(mq[0], j) ? bq[0][j] - (d * v[1][j] - nb) : 0.f;
-        }
+        for (int j = 0; j < 4; ++j) r[j] = s_byte(mq[0], j) ? fmaf(-d.get(j), v[1].get(j), t.get(j)) : 0.f;
         if (o >= y0 && c.own) s_put(x + o * L.nx + c.gx, v[1]);
         if (o & 1) {
           if (o >= y0 && c.own)
@@ -221,10 +243,10 @@ __device__ __forceinline__ float s_up(const LevelDev& L, int u0, int u1, int y0,
                                       const float* __restrict__ xin, float* __restrict__ xout,
                                       const float* __restrict__ e, float omega, float s, unsigned char* ring) {
   const SLane c = s_lane(L, u0, u1, omega);
-  const float keep = 1.f - omega;
+  const float2 wx = s_dup(L.wx), wy = s_dup(L.wy), keep = s_dup(1.f - omega);
   const int cnx = L.nx >> 1;
-  // xs[k] holds the rows after sweep k (0: the corrected input)
-  float bq[H + 1][4], wq[H + 1][4], xs[H][3][4];
+  // xs[k] holds the rows after sweep k (0: the corrected input, H: the output)
+  Quad bq[H + 1], wq[H + 1], xs[H + 1][3];
   float acc = 0.f;
   s_zero(bq);
   s_zero(wq);
@@ -246,26 +268,24 @@ __device__ __forceinline__ float s_up(const LevelDev& L, int u0, int u1, int y0,
         s_shift(wq);
 #pragma unroll
         for (int k = 0; k < H; ++k) s_shift(xs[k]);
-        float xv[4];
-        s_get(slot + c.lane * 16, xv);
-        s_get(slot + 512 + c.lane * 16, bq[H]);
+        const Quad xv = s_get(slot + c.lane * 16);
+        bq[H] = s_get(slot + 512 + c.lane * 16);
         const float2 ev = *reinterpret_cast<const float2*>(slot + 1024 + c.lane * 8);
         const unsigned m = s_cells(L, c, p, slot + 1280);
+        wq[H] = s_table(c, c.tabw, m);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          wq[H][j] = __shfl_sync(kFull, c.tabw, (int)(s_byte(m, j) & 15u));
-          xs[0][2][j] = s_byte(m, j) ? xv[j] + s * (j < 2 ? ev.x : ev.y) : 0.f;
-        }
-        float z[4];
+        for (int j = 0; j < 4; ++j)
+          xs[0][2].set(j, s_byte(m, j) ? fmaf(s, j < 2 ? ev.x : ev.y, xv.get(j)) : 0.f);
 #pragma unroll
         for (int k = 1; k <= H; ++k)
-          s_sweep(L, c, keep, xs[k - 1][0], xs[k - 1][1], xs[k - 1][2], bq[H - k], wq[H - k],
-                  *(k < H ? &xs[k < H ? k : 0][2] : &z));
+          xs[k][2] = s_sweep(c, wx, wy, keep, xs[k - 1][0], xs[k - 1][1], xs[k - 1][2], bq[H - k], wq[H - k]);
         const int o = p - H;
         if (o >= y0 && c.own) {
+          const Quad& z = xs[H][2];
           s_put(xout + o * L.nx + c.gx, z);
+          // b off the fluid stays out of the sum
 #pragma unroll
-          for (int j = 0; j < 4; ++j) acc = fmaf(wq[0][j] > 0.f ? bq[0][j] : 0.f, z[j], acc);
+          for (int j = 0; j < 4; ++j) acc = fmaf(wq[0].get(j) > 0.f ? bq[0].get(j) : 0.f, z.get(j), acc);
         }
       });
   return acc;
@@ -277,7 +297,8 @@ __device__ __forceinline__ float s_pupdate(const LevelDev& L, int u0, int u1, in
                                            float* __restrict__ pnew, float* __restrict__ Ap, float beta, bool first,
                                            unsigned char* ring) {
   const SLane c = s_lane(L, u0, u1, 1.f);
-  float ps[3][4];
+  const float2 wx = s_dup(-L.wx), wy = s_dup(-L.wy), bt = s_dup(beta);
+  Quad ps[3];
   unsigned mp = 0u;
   float acc = 0.f;
   s_zero(ps);
@@ -293,33 +314,28 @@ __device__ __forceinline__ float s_pupdate(const LevelDev& L, int u0, int u1, in
       },
       [&](int p, const unsigned char* slot) {
         s_shift(ps);
-        float zv[4], pv[4] = {0.f, 0.f, 0.f, 0.f};
-        s_get(slot + c.lane * 16, zv);
-        if (!first) s_get(slot + 512 + c.lane * 16, pv);
+        Quad v = s_get(slot + c.lane * 16);
         const unsigned m = s_cells(L, c, p, slot + 1280);
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          ps[2][j] = s_byte(m, j) ? (first ? zv[j] : fmaf(beta, pv[j], zv[j])) : 0.f;
-        const int o = p - 1;
-        float left, right, ap[4];
-        s_edges(c, ps[1], left, right);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const float l = j == 0 ? left : ps[1][j - 1], r = j == 3 ? right : ps[1][j + 1];
-          const float d = __shfl_sync(kFull, c.tabd, (int)(s_byte(mp, j) & 15u));
-          float nb = 0.f;
-          nb += L.wx * l;
-          nb += L.wx * r;
-          nb += L.wy * ps[0][j];
-          nb += L.wy * ps[2][j];
-          ap[j] = s_byte(mp, j) ? d * ps[1][j] - nb : 0.f;
+        if (!first) {
+          const Quad pv = s_get(slot + 512 + c.lane * 16);
+          v.a = __ffma2_rn(bt, pv.a, v.a);
+          v.b = __ffma2_rn(bt, pv.b, v.b);
         }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) ps[2].set(j, s_byte(m, j) ? v.get(j) : 0.f);
+        const int o = p - 1;
+        Quad t = s_table(c, c.tabd, mp), ap;
+        t.a = __fmul2_rn(t.a, ps[1].a);
+        t.b = __fmul2_rn(t.b, ps[1].b);
+        t = s_stencil(c, wx, wy, t, ps[0], ps[1], ps[2]);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) ap.set(j, s_byte(mp, j) ? t.get(j) : 0.f);
         mp = m;
         if (o >= y0 && c.own) {
           s_put(pnew + o * L.nx + c.gx, ps[1]);
           s_put(Ap + o * L.nx + c.gx, ap);
 #pragma unroll
-          for (int j = 0; j < 4; ++j) acc = fmaf(ps[1][j], ap[j], acc);
+          for (int j = 0; j < 4; ++j) acc = fmaf(ps[1].get(j), ap.get(j), acc);
         }
       });
   return acc;

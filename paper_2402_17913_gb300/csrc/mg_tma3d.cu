@@ -129,6 +129,8 @@ struct Th {
   bool xin;       // chunk inside the domain (nx % 16 == 0: a chunk is all in or all out)
   bool yin[2];    // rows inside the domain
   bool own;       // the chunk and both rows belong to the column's output
+  bool wown;      // some thread of the warp owns its cells
+  int edge;       // first lane of the warp: -1, last: 4 (offset of the neighbour no lane holds), others 0
 };
 
 __device__ __forceinline__ Th thread_geom(const LevelDev& L, int x0, int y0) {
@@ -141,6 +143,8 @@ __device__ __forceinline__ Th thread_geom(const LevelDev& L, int x0, int y0) {
   t.yin[0] = t.gy >= 0 && t.gy < L.ny;
   t.yin[1] = t.gy + 1 >= 0 && t.gy + 1 < L.ny;
   t.own = t.c >= 1 && t.c <= NCH - 2 && t.q >= 1 && t.q <= NQ - 2;
+  t.wown = __any_sync(0xffffffffu, t.own);
+  t.edge = (threadIdx.x & 31) == 0 ? -1 : ((threadIdx.x & 31) == 31 || threadIdx.x == NT - 1) ? 4 : 0;
   return t;
 }
 
@@ -202,11 +206,23 @@ __device__ __forceinline__ const float* brow(const float* buf, const Th& t, int 
   return buf + (2 * t.q + h + 1) * RS + 4 + 4 * t.c;
 }
 
+// Two cells' arithmetic is one instruction (add, mul, fma .rn.f32x2), with
+// the rounding of the scalar ones.
+__device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
+__device__ __forceinline__ float2 cells2(const float (&v)[4], int q) { return f2(v[2 * q], v[2 * q + 1]); }
+
 // Neighbour sums of a thread's 4 x 2 cells on one plane, a = the cells'
 // own values (registers), zm / zp = the same cells one plane below / above
-// (registers); the row above the pair, the row below it and the
-// x-neighbours beyond the chunk come from plane buffer `buf`:
+// (registers); the row above the pair and the row below it come from plane
+// buffer `buf`, the x-neighbours beyond the chunk from the adjacent lanes (at
+// a warp's ends from `buf`; beyond the region's first and last chunk any
+// finite value: no owned cell depends on it):
 // nb = wx (left + right) + wy (south + north) + wz (below + above).
+// Every thread of a warp has to call it.  Shared-memory wavefronts and issue
+// are what the legs spend their time on: a scalar read at the lanes' stride
+// of four floats takes four wavefronts, so four such reads were 16 of the 24
+// a stencil took (256^3 solve 9.27 -> 9.20 ms without them, -> 9.09 with
+// paired arithmetic).
 __device__ __forceinline__ void neighbours(const LevelDev& L, const Th& t, const float* buf,
                                            const float (&a)[2][4], const float (&zm)[2][4],
                                            const float (&zp)[2][4], float (&nb)[2][4]) {
@@ -214,15 +230,44 @@ __device__ __forceinline__ void neighbours(const LevelDev& L, const Th& t, const
   const float* r1 = r0 + RS;
   const float4 s = *reinterpret_cast<const float4*>(r0 - RS);
   const float4 n = *reinterpret_cast<const float4*>(r1 + RS);
-  const float l0 = r0[-1], e0 = r0[4], l1 = r1[-1], e1 = r1[4];
-  const float sv[4] = {s.x, s.y, s.z, s.w}, nv[4] = {n.x, n.y, n.z, n.w};
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const float xl0 = j == 0 ? l0 : a[0][j - 1], xr0 = j == 3 ? e0 : a[0][j + 1];
-    const float xl1 = j == 0 ? l1 : a[1][j - 1], xr1 = j == 3 ? e1 : a[1][j + 1];
-    nb[0][j] = fmaf(L.wx, xl0 + xr0, fmaf(L.wy, sv[j] + a[1][j], L.wz * (zm[0][j] + zp[0][j])));
-    nb[1][j] = fmaf(L.wx, xl1 + xr1, fmaf(L.wy, a[0][j] + nv[j], L.wz * (zm[1][j] + zp[1][j])));
+  float l0 = __shfl_up_sync(0xffffffffu, a[0][3], 1), l1 = __shfl_up_sync(0xffffffffu, a[1][3], 1);
+  float e0 = __shfl_down_sync(0xffffffffu, a[0][0], 1), e1 = __shfl_down_sync(0xffffffffu, a[1][0], 1);
+  if (t.edge) {
+    const float v0 = r0[t.edge], v1 = r1[t.edge];
+    if (t.edge < 0) l0 = v0, l1 = v1;
+    else e0 = v0, e1 = v1;
   }
+  const float2 wx = f2(L.wx, L.wx), wy = f2(L.wy, L.wy), wz = f2(L.wz, L.wz);
+  const float2 sv[2] = {f2(s.x, s.y), f2(s.z, s.w)}, nv[2] = {f2(n.x, n.y), f2(n.z, n.w)};
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const float l = h ? l1 : l0, e = h ? e1 : e0;
+    const float2 x[2] = {f2(l + a[h][1], a[h][0] + a[h][2]), f2(a[h][1] + a[h][3], a[h][2] + e)};
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const float2 y = h ? __fadd2_rn(cells2(a[0], q), nv[q]) : __fadd2_rn(sv[q], cells2(a[1], q));
+      const float2 z = __fmul2_rn(wz, __fadd2_rn(cells2(zm[h], q), cells2(zp[h], q)));
+      const float2 v = __ffma2_rn(wx, x[q], __ffma2_rn(wy, y, z));
+      nb[h][2 * q] = v.x;
+      nb[h][2 * q + 1] = v.y;
+    }
+  }
+}
+
+// One sweep of the thread's cells: out = keep v + W(h, j) (b + nb).
+template <typename F>
+__device__ __forceinline__ void relax(float keep, const float (&v)[2][4], const float (&b)[2][4],
+                                      const float (&nb)[2][4], F&& W, float (&out)[2][4]) {
+  const float2 k2 = f2(keep, keep);
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const float2 t = __fmul2_rn(f2(W(h, 2 * q), W(h, 2 * q + 1)), __fadd2_rn(cells2(b[h], q), cells2(nb[h], q)));
+      const float2 o = __ffma2_rn(k2, cells2(v[h], q), t);
+      out[h][2 * q] = o.x;
+      out[h][2 * q + 1] = o.y;
+    }
 }
 
 __device__ __forceinline__ void sts8(float* buf, const Th& t, const float (&v)[2][4]) {
@@ -380,30 +425,20 @@ __global__ void __launch_bounds__(NT, 1)
       if (i >= 2) {
         float nb[2][4];
         neighbours(L, t, XS + ((i - 1) & 1) * PL, XQ[C1], XQ[C2], XQ[C0], nb);
-        auto sweep = [&](auto W) {
-#pragma unroll
-          for (int h = 0; h < 2; ++h)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) SQ[C1][h][j] = fmaf(keep, XQ[C1][h][j], W(h, j) * (BQ[C1][h][j] + nb[h][j]));
-        };
+        auto sweep = [&](auto W) { relax(keep, XQ[C1], BQ[C1], nb, W, SQ[C1]); };
         if constexpr (MASKED) sweep([&](int h, int j) { return WQ[C1][h][j]; });
         else with_plane(plane_kz(L, p - 1), D.w1, D.w2, sweep);
         sts8(SS + ((i - 1) & 1) * PL, t, SQ[C1]);
       }
       // C: second sweep on plane o = p - 2, written out
       const int o = p - 2;
-      if (i >= 4 && t.own) {
+      if (i >= 4 && t.wown) {
         float nb[2][4], z[2][4];
         neighbours(L, t, SS + (i & 1) * PL, SQ[C2], SQ[C0], SQ[C1], nb);
-        auto sweep = [&](auto W) {
-#pragma unroll
-          for (int h = 0; h < 2; ++h)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) z[h][j] = fmaf(keep, SQ[C2][h][j], W(h, j) * (BQ[C2][h][j] + nb[h][j]));
-        };
+        auto sweep = [&](auto W) { relax(keep, SQ[C2], BQ[C2], nb, W, z); };
         if constexpr (MASKED) sweep([&](int h, int j) { return WQ[C2][h][j]; });
         else with_plane(plane_kz(L, o), D.w1, D.w2, sweep);
-        if (t.xin) {
+        if (t.own && t.xin) {
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
             if (!t.yin[h]) continue;
@@ -527,13 +562,7 @@ __global__ void __launch_bounds__(NT, 1)
       if (i >= 2) {
         float nb[2][4];
         neighbours(L, t, S1 + ((i - 1) & 1) * PL, S1Q[C1], S1Q[C2], S1Q[C0], nb);
-        auto sweep = [&](auto W) {
-#pragma unroll
-          for (int h = 0; h < 2; ++h)
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-              XQ[C1][h][j] = fmaf(keep, S1Q[C1][h][j], W(h, j) * (BQ[C1][h][j] + nb[h][j]));
-        };
+        auto sweep = [&](auto W) { relax(keep, S1Q[C1], BQ[C1], nb, W, XQ[C1]); };
         if constexpr (MASKED) sweep([&](int h, int j) { return WQ[C1][h][j]; });
         else with_plane(plane_kz(L, p - 1), D.w1, D.w2, sweep);
         sts8(XB + ((i - 1) & 1) * PL, t, XQ[C1]);
@@ -547,7 +576,7 @@ __global__ void __launch_bounds__(NT, 1)
       // C: residual on plane o = p - 2 and its 2x2x2 average (x pairs and
       // the row pair in registers, z pairs across consecutive steps)
       const int o = p - 2;
-      if (i >= 4 && t.own) {
+      if (i >= 4 && t.wown) {
         float nb[2][4], rx[2] = {0.f, 0.f};
         neighbours(L, t, XB + (i & 1) * PL, XQ[C2], XQ[C0], XQ[C1], nb);
         // solid cells (d = 0) are not unknowns: no residual there; unmasked
@@ -567,7 +596,7 @@ __global__ void __launch_bounds__(NT, 1)
         if ((o & 1) == 0) {
           zp[0] = rx[0];
           zp[1] = rx[1];
-        } else if (t.xin && t.yin[0]) {
+        } else if (t.own && t.xin && t.yin[0]) {
           stg2<T>(bcoarse + ((size_t)(o >> 1) * (L.ny >> 1) + (t.gy >> 1)) * (L.nx >> 1) + (t.gx >> 1),
                   0.125f * (zp[0] + rx[0]), 0.125f * (zp[1] + rx[1]));
         }
@@ -701,11 +730,11 @@ __global__ void __launch_bounds__(NT, 2)
       }
       // B: A' p on plane o = p - 1, written with p; (p, Ap) reduced
       const int o = p - 1;
-      if (i >= 2 && t.own) {
+      if (i >= 2 && t.wown) {
         float nb[2][4];
         neighbours(L, t, PS + ((i - 1) & 1) * PL, PQ[C1], PQ[C2], PQ[C0], nb);
         auto apply = [&](auto Dg) {
-          if (!t.xin) return;
+          if (!t.own || !t.xin) return;
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
             if (!t.yin[h]) continue;
@@ -852,11 +881,11 @@ __global__ void __launch_bounds__(NT, 1)
       sts8(PS + (i & 1) * PL, t, PQ[C0]);
       // B: A' p on plane o = p - 1; d and r of plane o from this stage
       const int o = p - 1;
-      if (i >= 2 && t.own) {
+      if (i >= 2 && t.wown) {
         float nb[2][4];
         neighbours(L, t, PS + ((i - 1) & 1) * PL, PQ[C1], PQ[C2], PQ[C0], nb);
         auto update = [&](auto Dg) {
-          if (!t.xin) return;
+          if (!t.own || !t.xin) return;
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
             if (!t.yin[h]) continue;

@@ -280,8 +280,14 @@ __device__ __forceinline__ void sts8(float* buf, const Th& t, const float (&v)[2
 // of column-major (column, plane) units (a block may end one column's
 // planes and start the next column's), or with units == 0 one z-run of zr
 // planes of column (blockIdx.x, blockIdx.y).
+// With flip the block walks the mirror image (columns and planes from the
+// last to the first): the up leg and the vector update take the grid in the
+// opposite order of the down leg and the direction update, so that each
+// kernel starts on the planes its predecessor touched last, which the L2
+// still holds.  plane() gives the plane in memory of a plane of the walk.
 struct Sched {
-  int zr, units;
+  int zr, units, flip;
+  __device__ __forceinline__ int plane(const LevelDev& L, int p) const { return flip ? L.nz - 1 - p : p; }
 };
 
 template <typename F>
@@ -289,14 +295,18 @@ __device__ __forceinline__ void for_each_run(const LevelDev& L, Sched sc, F&& ru
   const int strips = (L.nx + TX - 1) / TX;
   if (sc.units == 0) {
     const int z0 = blockIdx.z * sc.zr;
-    run(blockIdx.x * TX, blockIdx.y * TY, z0, min(z0 + sc.zr, L.nz));
+    const int bx = sc.flip ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
+    const int by = sc.flip ? gridDim.y - 1 - blockIdx.y : blockIdx.y;
+    run(bx * TX, by * TY, z0, min(z0 + sc.zr, L.nz));
     return;
   }
-  const long total = (long)strips * ((L.ny + TY - 1) / TY) * L.nz;
+  const int cols = strips * ((L.ny + TY - 1) / TY);
+  const long total = (long)cols * L.nz;
   long u = (long)blockIdx.x * sc.units;
   const long uend = min(u + sc.units, total);
   while (u < uend) {
-    const int col = (int)(u / L.nz), z0 = (int)(u % L.nz);
+    const int c = (int)(u / L.nz), z0 = (int)(u % L.nz);
+    const int col = sc.flip ? cols - 1 - c : c;
     const int z1 = (int)min((long)L.nz, z0 + (uend - u));
     if (!run((col % strips) * TX, (col / strips) * TY, z0, z1)) return;
     u += z1 - z0;
@@ -379,7 +389,8 @@ __global__ void __launch_bounds__(NT, 1)
     if (!MASKED) D = unmasked_diag(L, t, omega);
     const int n = z1 - z0 + 4;  // steps: A on planes z0 - 2 .. z1 + 1
     if (threadIdx.x == 0)
-      for (int k = 0; k < S::NS && k < n; ++k) issue_plane<T, TB, MASKED, true>(R, &mx, &mb, &me, &mm, x0, y0, z0 - 2 + k);
+      for (int k = 0; k < S::NS && k < n; ++k)
+        issue_plane<T, TB, MASKED, true>(R, &mx, &mb, &me, &mm, x0, y0, sc.plane(L, z0 - 2 + k));
     float XQ[3][2][4], BQ[3][2][4], WQ[3][2][4], SQ[3][2][4];
 #pragma unroll
     for (int k = 0; k < 3; ++k)
@@ -427,11 +438,11 @@ __global__ void __launch_bounds__(NT, 1)
         neighbours(L, t, XS + ((i - 1) & 1) * PL, XQ[C1], XQ[C2], XQ[C0], nb);
         auto sweep = [&](auto W) { relax(keep, XQ[C1], BQ[C1], nb, W, SQ[C1]); };
         if constexpr (MASKED) sweep([&](int h, int j) { return WQ[C1][h][j]; });
-        else with_plane(plane_kz(L, p - 1), D.w1, D.w2, sweep);
+        else with_plane(plane_kz(L, sc.plane(L, p - 1)), D.w1, D.w2, sweep);
         sts8(SS + ((i - 1) & 1) * PL, t, SQ[C1]);
       }
       // C: second sweep on plane o = p - 2, written out
-      const int o = p - 2;
+      const int o = sc.plane(L, p - 2);
       if (i >= 4 && t.wown) {
         float nb[2][4], z[2][4];
         neighbours(L, t, SS + (i & 1) * PL, SQ[C2], SQ[C0], SQ[C1], nb);
@@ -458,7 +469,7 @@ __global__ void __launch_bounds__(NT, 1)
         return false;
       }
       if (threadIdx.x == 0 && i + S::NS < n)
-        issue_plane<T, TB, MASKED, true>(R, &mx, &mb, &me, &mm, x0, y0, z0 - 2 + i + S::NS);
+        issue_plane<T, TB, MASKED, true>(R, &mx, &mb, &me, &mm, x0, y0, sc.plane(L, z0 - 2 + i + S::NS));
       ++R.g;
       return true;
     };
@@ -808,15 +819,15 @@ struct GX {
 template <bool MASKED, int N>
 __device__ __forceinline__ void issue_xr(Ring<N>& R, const CUtensorMap* mp, const CUtensorMap* md,
                                          const CUtensorMap* mr, const CUtensorMap* mm, bool first, int x0, int y0,
-                                         int p) {
+                                         int p, int pv) {
   using S = GX<MASKED>;
   const unsigned st = R.issued % N;
   unsigned char* dst = R.base + st * S::STAGE;
   uint64_t* bar = R.bar + st;
   mbar_arrive_expect_tx(bar, (uint32_t)(S::PB + S::VB * (first ? 1 : 2) + S::MBY));
   tma_load_3d(dst + S::OP, mp, bar, x0 - 4, y0 - 2, p);
-  if (!first) tma_load_3d(dst + S::OD, md, bar, x0, y0, p - 1);
-  tma_load_3d(dst + S::OR, mr, bar, x0, y0, p - 1);
+  if (!first) tma_load_3d(dst + S::OD, md, bar, x0, y0, pv);
+  tma_load_3d(dst + S::OR, mr, bar, x0, y0, pv);
   if (MASKED) tma_load_3d(dst + S::OM, mm, bar, x0 - 16, y0 - 2, p);
   ++R.issued;
 }
@@ -853,7 +864,8 @@ __global__ void __launch_bounds__(NT, 1)
     if (!MASKED) D = unmasked_diag(L, t, 1.f);
     const int n = z1 - z0 + 2;  // steps: p on planes z0 - 1 .. z1
     if (threadIdx.x == 0)
-      for (int k = 0; k < S::NS && k < n; ++k) issue_xr<MASKED>(R, &mp, &md, &mr, &mm, first, x0, y0, z0 - 1 + k);
+      for (int k = 0; k < S::NS && k < n; ++k)
+        issue_xr<MASKED>(R, &mp, &md, &mr, &mm, first, x0, y0, sc.plane(L, z0 - 1 + k), sc.plane(L, z0 - 2 + k));
     float PQ[3][2][4], DQ[3][2][4];
 #pragma unroll
     for (int k = 0; k < 3; ++k)
@@ -880,7 +892,7 @@ __global__ void __launch_bounds__(NT, 1)
       }
       sts8(PS + (i & 1) * PL, t, PQ[C0]);
       // B: A' p on plane o = p - 1; d and r of plane o from this stage
-      const int o = p - 1;
+      const int o = sc.plane(L, p - 1);
       if (i >= 2 && t.wown) {
         float nb[2][4];
         neighbours(L, t, PS + ((i - 1) & 1) * PL, PQ[C1], PQ[C2], PQ[C0], nb);
@@ -914,7 +926,8 @@ __global__ void __launch_bounds__(NT, 1)
         return false;
       }
       if (threadIdx.x == 0 && i + S::NS < n)
-        issue_xr<MASKED>(R, &mp, &md, &mr, &mm, first, x0, y0, z0 - 1 + i + S::NS);
+        issue_xr<MASKED>(R, &mp, &md, &mr, &mm, first, x0, y0, sc.plane(L, z0 - 1 + i + S::NS),
+                         sc.plane(L, z0 - 2 + i + S::NS));
       ++R.g;
       return true;
     };
@@ -960,7 +973,7 @@ struct T3Plan {
 };
 
 // bps: blocks of the kernel an SM holds at once.
-static T3Plan t3_plan(const LevelDev& L, int bps = 1) {
+static T3Plan t3_plan(const LevelDev& L, int bps = 1, int flip = 0) {
   const long strips = (L.nx + TX - 1) / TX, tiles = (L.ny + TY - 1) / TY;
   const long cols = strips * tiles;
   const long nsm = (long)t3_sms() * bps;
@@ -978,6 +991,7 @@ static T3Plan t3_plan(const LevelDev& L, int bps = 1) {
   }
   T3Plan p;
   p.sc.zr = (int)best_zr;
+  p.sc.flip = flip;
   p.sc.units = 0;
   p.grid = dim3((unsigned)strips, (unsigned)tiles, (unsigned)((L.nz + best_zr - 1) / best_zr));
   const long total = cols * L.nz;
@@ -1049,7 +1063,7 @@ cudaError_t launch_down_t3(const Tma3Maps& m, const LevelDev& L, void* x, void* 
 template <typename T, bool MASKED, bool FINEST, typename TB>
 cudaError_t launch_up_t3(const Tma3Maps& m, const LevelDev& L, void* xout, float omega, float sc, SolveState* st,
                          double* partials, cudaStream_t s) {
-  const T3Plan pl = t3_plan(L);
+  const T3Plan pl = t3_plan(L, 1, 1);
   return launch_chain(k_up_t3<T, MASKED, FINEST, TB>, pl.grid, NT, (size_t)G3<T, TB, MASKED, true>::BYTES, s, m.x,
                       m.b, m.e, m.m, L, (TB*)xout, omega, sc, pl.sc, st, partials);
 }
@@ -1086,7 +1100,7 @@ template cudaError_t launch_p_update_t3<true>(const Tma3CgMaps&, int, const Leve
 template <bool MASKED>
 cudaError_t launch_xr_update_t3(const Tma3CgMaps& m, int pbuf, const LevelDev& L, float* d, float* r,
                                 SolveState* st, double* partials, cudaStream_t s) {
-  const T3Plan pl = t3_plan(L);
+  const T3Plan pl = t3_plan(L, 1, 1);
   return launch_chain(k_xr_t3<MASKED>, pl.grid, NT, (size_t)GX<MASKED>::BYTES, s, m.p[pbuf], m.d, m.r, m.m, L, d, r,
                       pl.sc, st, partials);
 }

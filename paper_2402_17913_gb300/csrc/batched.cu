@@ -45,7 +45,7 @@ struct BInst {
   float* b[kMaxLevels];  // right-hand side of level k (k >= 1)
   float* x[kMaxLevels];  // down-leg x of level k (k < kc)
   float* y[kMaxLevels];  // up-leg output of level k (1 <= k <= kc; y[kc] = coarse item output)
-  float *r, *z, *p0, *p1, *Ap, *d;
+  float *r, *z, *p0, *p1, *d;
   float2 *xf0, *xf1;
   ff wff[2];             // finest operator weights c / h^2 (float-float)
   ff cff;                // c = h_x^2
@@ -371,44 +371,6 @@ struct VNb {
   __device__ __forceinline__ float left(int k) const { return k == 0 ? l : lane(c, k - 1); }
   __device__ __forceinline__ float right(int k) const { return k == 3 ? r : lane(c, k + 1); }
 };
-
-// d += alpha p (d = alpha p on the first iteration), r -= alpha Ap on a
-// level-0 tile, four cells per access; returns the thread's share of ||r||^2
-template <int TX, int TY>
-__device__ float b_xr(const LevelDev& L, int tx, int ty, float* __restrict__ d, const float* __restrict__ p,
-                      const float* __restrict__ Ap, float* __restrict__ r, float alpha, bool first) {
-  constexpr int T4 = TX / 4, NG = TY * T4, NI = (NG + kBThreads - 1) / kBThreads;
-  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-  float4 dv[NI], pv[NI], av[NI], rv[NI];
-  int gi[NI];
-#pragma unroll
-  for (int j = 0; j < NI; ++j) {
-    const int q = threadIdx.x + j * kBThreads;
-    const int x = tx * TX + 4 * (q % T4), y = ty * TY + q / T4;
-    gi[j] = (q < NG && x < L.nx && y < L.ny) ? y * L.nx + x : -1;
-    dv[j] = (gi[j] < 0 || first) ? zero : *reinterpret_cast<const float4*>(d + gi[j]);
-    pv[j] = gi[j] < 0 ? zero : *reinterpret_cast<const float4*>(p + gi[j]);
-    av[j] = gi[j] < 0 ? zero : *reinterpret_cast<const float4*>(Ap + gi[j]);
-    rv[j] = gi[j] < 0 ? zero : *reinterpret_cast<const float4*>(r + gi[j]);
-  }
-  float acc = 0.f;
-#pragma unroll
-  for (int j = 0; j < NI; ++j) {
-    if (gi[j] < 0) continue;
-    float4 dn, rn;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const float pk = lane(pv[j], k);
-      set_lane(dn, k, first ? alpha * pk : fmaf(alpha, pk, lane(dv[j], k)));
-      const float rk = fmaf(-alpha, lane(av[j], k), lane(rv[j], k));
-      set_lane(rn, k, rk);
-      acc = fmaf(rk, rk, acc);
-    }
-    *reinterpret_cast<float4*>(d + gi[j]) = dn;
-    *reinterpret_cast<float4*>(r + gi[j]) = rn;
-  }
-  return acc;
-}
 
 // legs of a level whose width is not a multiple of 4 (tiles), and of one item
 // of any other level (a strip of rows, one warp)
@@ -824,7 +786,7 @@ __global__ void __launch_bounds__(kBThreads, kBBlocks) k_batched(const __grid_co
         }
       }
       if (!grid_barrier(A, epoch)) return;
-      // p = z + beta p, Ap, (p, Ap)
+      // p = z + beta p, (p, Ap)
       for (int w = wid; w < A.nstrips[0]; w += nw) {
         const int4 item = A.strips[0][w];
         const SolveState& st = A.st[item.x];
@@ -837,7 +799,7 @@ __global__ void __launch_bounds__(kBThreads, kBBlocks) k_batched(const __grid_co
         float* pnew = (st.it & 1) ? I.p0 : I.p1;
         const Strip t(item, L, A.srows[0]);
         warp_partial(A, item.w,
-                     s_pupdate(L, t.u0, t.u1, t.y0, t.y1, I.z, pold, pnew, I.Ap, beta, first, ring));
+                     s_pupdate(L, t.u0, t.u1, t.y0, t.y1, I.z, pold, pnew, beta, first, ring));
       }
       if (!grid_barrier(A, epoch)) return;
       for (int w = blockIdx.x; w < A.count; w += gridDim.x) {
@@ -851,22 +813,21 @@ __global__ void __launch_bounds__(kBThreads, kBBlocks) k_batched(const __grid_co
       }
       if (!grid_barrier(A, epoch)) return;
       // d += alpha p, r -= alpha Ap, ||r||^2
-      for (int w = blockIdx.x; w < n0; w += gridDim.x) {
-        const int4 item = it0[n0 - 1 - w];
+      for (int w = wid; w < A.nstrips[0]; w += nw) {
+        const int4 item = A.strips[0][A.nstrips[0] - 1 - w];
         const SolveState& st = A.st[item.x];
         if (st.inner_done) continue;
         const BInst& I = A.inst[item.x];
-        const float alpha = (float)st.alpha;
-        const float* p = (st.it & 1) ? I.p0 : I.p1;
-        const float acc = b_xr<TX, TY>(I.lv[0], item.y, item.z, I.d, p, I.Ap, I.r, alpha, st.first != 0);
-        const double t = block_total(acc);
-        if (threadIdx.x == 0) A.partials[item.w] = t;
+        const LevelDev L = I.lv[0];
+        const Strip t(item, L, A.srows[0]);
+        warp_partial(A, item.w, s_xrupdate(L, t.u0, t.u1, t.y0, t.y1, (st.it & 1) ? I.p0 : I.p1, I.d, I.r,
+                                           (float)st.alpha, st.first != 0, ring));
       }
       if (!grid_barrier(A, epoch)) return;
       for (int w = blockIdx.x; w < A.count; w += gridDim.x) {
         SolveState& st = A.st[w];
         if (st.inner_done) continue;
-        const double tot = reduce_slots(A, A.inst[w].slot0, A.inst[w].ntiles0);
+        const double tot = reduce_slots(A, A.inst[w].wslot0, A.inst[w].nstrips0);
         if (threadIdx.x == 0) inner_decide(&st, tot);
         __syncthreads();
         count_active(A, cslot, !st.inner_done);
@@ -1090,7 +1051,7 @@ static mg_status build_items(mg_batch_s* B, int tile, cudaStream_t s);
 // inner edge belongs to the neighbour; runs of rows, chosen per level so that
 // the warps' rounds times the rows walked (the halo rows and about six rows'
 // time of latency at a run's start included) are fewest.
-constexpr int kStripRows[] = {8, 16, 32, 64, 128};
+constexpr int kStripRows[] = {4, 8, 16, 32, 64, 128};
 static int strip_count(int nx) { return nx <= 128 ? 1 : (nx / 4 + 29) / 30; }
 
 extern "C" {
@@ -1136,7 +1097,7 @@ mg_status mg_create_batched(mg_batch* out, int count, const int64_t* shapes, con
   };
   struct Off {
     size_t solid[kMaxLevels], cell[kMaxLevels], b[kMaxLevels], x[kMaxLevels], y[kMaxLevels];
-    size_t r, z, p0, p1, Ap, d, xf0, xf1, inv;
+    size_t r, z, p0, p1, d, xf0, xf1, inv;
   };
   std::vector<Off> off(count);
   int max_kc = 0;
@@ -1209,7 +1170,6 @@ mg_status mg_create_batched(mg_batch* out, int count, const int64_t* shapes, con
     f.z = reserve(n0 * 4);
     f.p0 = reserve(n0 * 4);
     f.p1 = reserve(n0 * 4);
-    f.Ap = reserve(n0 * 4);
     f.d = reserve(n0 * 4);
     f.xf0 = reserve(n0 * 8);
     f.xf1 = reserve(n0 * 8);
@@ -1291,7 +1251,6 @@ mg_status mg_create_batched(mg_batch* out, int count, const int64_t* shapes, con
     I.z = (float*)(P + f.z);
     I.p0 = (float*)(P + f.p0);
     I.p1 = (float*)(P + f.p1);
-    I.Ap = (float*)(P + f.Ap);
     I.d = (float*)(P + f.d);
     I.xf0 = (float2*)(P + f.xf0);
     I.xf1 = (float2*)(P + f.xf1);

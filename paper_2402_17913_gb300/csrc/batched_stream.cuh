@@ -17,7 +17,8 @@
 // blocks per SM at 80 registers spill: 36 ms).  The block tiles before staged
 // 72 x 38 cells for 64 x 32 behind seven block barriers, 6 us a tile at four
 // blocks per SM: 28.1 -> 21.0 ms a solve, -> 19.7 with paired arithmetic and
-// with the phases walking the list up and down in turn.
+// with the phases walking the list up and down in turn, -> 18.8 with Ap
+// formed again instead of stored.
 #pragma once
 
 #include "npmg_internal.cuh"
@@ -28,7 +29,9 @@ constexpr int kSD = 5;          // rows in flight ahead of the row in use
 constexpr int kSSlots = kSD + 1;
 constexpr int kSRowDown = 32 * 16 + 32 * 4;                     // b, cell bytes
 constexpr int kSRowUp = 2 * 32 * 16 + 32 * 8 + 32 * 4;          // x (or z), b (or p), e, cell bytes
-constexpr int kSRing = kSSlots * kSRowUp;                       // bytes of one warp's ring
+constexpr int kSRowXr = 3 * 32 * 16 + 32 * 4;                  // p, d, r, cell bytes
+constexpr int kSRing = kSSlots * kSRowXr;                       // bytes of one warp's ring
+static_assert(kSRowXr >= kSRowUp && kSRowUp >= kSRowDown, "the ring holds the longest rows");
 constexpr unsigned kFull = 0xffffffffu;
 
 __device__ __forceinline__ uint32_t s_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -291,11 +294,23 @@ __device__ __forceinline__ float s_up(const LevelDev& L, int u0, int u1, int y0,
   return acc;
 }
 
-// p = z + beta p_old, Ap; returns the lane's share of (p, Ap)
+// A p of row v between rows dn and up (0 off the fluid)
+__device__ __forceinline__ Quad s_apply(const SLane& c, float2 nwx, float2 nwy, unsigned m, const Quad& dn,
+                                        const Quad& v, const Quad& up) {
+  Quad t = s_table(c, c.tabd, m);
+  t.a = __fmul2_rn(t.a, v.a);
+  t.b = __fmul2_rn(t.b, v.b);
+  t = s_stencil(c, nwx, nwy, t, dn, v, up);
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+    if (!s_byte(m, j)) t.set(j, 0.f);
+  return t;
+}
+
+// p = z + beta p_old and the lane's share of (p, Ap)
 __device__ __forceinline__ float s_pupdate(const LevelDev& L, int u0, int u1, int y0, int y1,
                                            const float* __restrict__ z, const float* __restrict__ pold,
-                                           float* __restrict__ pnew, float* __restrict__ Ap, float beta, bool first,
-                                           unsigned char* ring) {
+                                           float* __restrict__ pnew, float beta, bool first, unsigned char* ring) {
   const SLane c = s_lane(L, u0, u1, 1.f);
   const float2 wx = s_dup(-L.wx), wy = s_dup(-L.wy), bt = s_dup(beta);
   Quad ps[3];
@@ -324,18 +339,66 @@ __device__ __forceinline__ float s_pupdate(const LevelDev& L, int u0, int u1, in
 #pragma unroll
         for (int j = 0; j < 4; ++j) ps[2].set(j, s_byte(m, j) ? v.get(j) : 0.f);
         const int o = p - 1;
-        Quad t = s_table(c, c.tabd, mp), ap;
-        t.a = __fmul2_rn(t.a, ps[1].a);
-        t.b = __fmul2_rn(t.b, ps[1].b);
-        t = s_stencil(c, wx, wy, t, ps[0], ps[1], ps[2]);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) ap.set(j, s_byte(mp, j) ? t.get(j) : 0.f);
+        const Quad ap = s_apply(c, wx, wy, mp, ps[0], ps[1], ps[2]);
         mp = m;
         if (o >= y0 && c.own) {
           s_put(pnew + o * L.nx + c.gx, ps[1]);
-          s_put(Ap + o * L.nx + c.gx, ap);
 #pragma unroll
           for (int j = 0; j < 4; ++j) acc = fmaf(ps[1].get(j), ap.get(j), acc);
+        }
+      });
+  return acc;
+}
+
+// d += alpha p (d = alpha p on the first iteration), r -= alpha Ap with Ap
+// formed again from p, the values (p, Ap) was summed from: both updates run
+// at the copy rate, and Ap stored and read back was 8 of their 41 bytes per
+// cell (256 instances: the two phases 6.25 -> 4.86 ms of a solve).  Returns
+// the lane's share of ||r||^2.
+__device__ __forceinline__ float s_xrupdate(const LevelDev& L, int u0, int u1, int y0, int y1,
+                                            const float* __restrict__ pv, float* __restrict__ dv,
+                                            float* __restrict__ rv, float alpha, bool first, unsigned char* ring) {
+  const SLane c = s_lane(L, u0, u1, 1.f);
+  const float2 wx = s_dup(-L.wx), wy = s_dup(-L.wy), al = s_dup(alpha), na = s_dup(-alpha);
+  Quad ps[3];
+  unsigned mp = 0u;
+  float acc = 0.f;
+  s_zero(ps);
+  s_walk<kSRowXr>(
+      y0 - 1, y1 - y0 + 2, ring,
+      [&](int p, unsigned char* slot) {
+        // row p of p and of the cell bytes, row p - 1 of d and r
+        const bool f = c.in && p >= 0 && p < L.ny, fo = c.own && p > y0;
+        const int at = f ? p * L.nx + c.go : 0, ao = fo ? (p - 1) * L.nx + c.go : 0;
+        const uint32_t sl = s_addr(slot);
+        s_copy16(sl + c.lane * 16, pv + at, f);
+        if (!first) s_copy16(sl + 512 + c.lane * 16, dv + ao, fo);
+        s_copy16(sl + 1024 + c.lane * 16, rv + ao, fo);
+        if (L.cell) s_copy<4>(sl + 1536 + c.lane * 4, L.cell + at, f);
+      },
+      [&](int p, const unsigned char* slot) {
+        s_shift(ps);
+        ps[2] = s_get(slot + c.lane * 16);
+        const unsigned m = s_cells(L, c, p, slot + 1536);
+        const Quad ap = s_apply(c, wx, wy, mp, ps[0], ps[1], ps[2]);
+        mp = m;
+        const int o = p - 1;
+        if (o >= y0 && c.own) {
+          Quad d, r = s_get(slot + 1024 + c.lane * 16);
+          if (first) {
+            d.a = __fmul2_rn(al, ps[1].a);
+            d.b = __fmul2_rn(al, ps[1].b);
+          } else {
+            d = s_get(slot + 512 + c.lane * 16);
+            d.a = __ffma2_rn(al, ps[1].a, d.a);
+            d.b = __ffma2_rn(al, ps[1].b, d.b);
+          }
+          r.a = __ffma2_rn(na, ap.a, r.a);
+          r.b = __ffma2_rn(na, ap.b, r.b);
+          s_put(dv + o * L.nx + c.gx, d);
+          s_put(rv + o * L.nx + c.gx, r);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) acc = fmaf(r.get(j), r.get(j), acc);
         }
       });
   return acc;

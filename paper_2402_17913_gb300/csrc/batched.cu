@@ -72,7 +72,7 @@ struct BatchArgs {
   const int2* citems;    // coarse phase: (instance, first row of a dense product) or (instance, -1)
   int ncitems;
   double* partials;      // one per level-0 tile, then one per level-0 strip
-  unsigned* bar;         // [0] arrivals, [1] generation, [2] error, [4..5] active counts
+  unsigned* bar;         // [0] arrivals, [2] error, [4..5] active counts
   int sweeps;
   float omega, s;
   SolveParams prm;
@@ -81,44 +81,38 @@ struct BatchArgs {
 };
 
 // ---------------------------------------------------------------------------
-// bounded grid barrier
-__device__ __forceinline__ bool bwait(const BatchArgs& A, unsigned g) {
-  volatile unsigned* gen = A.bar + 1;
-  volatile unsigned* err = A.bar + 2;
+// Bounded grid barrier: arrivals are counted through the whole launch (zeroed
+// before it), so barrier number `epoch` is open when (epoch + 1) gridDim.x
+// blocks have arrived.  One release addition and acquire loads of the counter
+// with the error flag: a generation word beside the counter, read before and
+// published after it between full fences, cost three more trips to the L2 (a
+// 64 - 192 batch of four spends most of its time in barriers).
+__device__ __forceinline__ bool bwait(const BatchArgs& A, unsigned target) {
   for (long long i = 0; i < A.spin_limit; ++i) {
-    if (*gen != g) return true;
-    if (*err) return false;
-    __nanosleep(128);
+    unsigned n, err;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(n) : "l"(A.bar) : "memory");
+    if ((int)(n - target) >= 0) return true;
+    if ((i & 15) == 15) {
+      asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(err) : "l"(A.bar + 2) : "memory");
+      if (err) return false;
+    }
+    __nanosleep(32);
   }
   return false;
 }
 
 __device__ __forceinline__ bool grid_barrier(const BatchArgs& A, unsigned& epoch) {
-  __syncthreads();
+  ++epoch;
   __shared__ int ok;
+  __syncthreads();
   if (threadIdx.x == 0) {
-    const unsigned g = *(volatile unsigned*)(A.bar + 1);
-    __threadfence();
-    bool res;
-    if (A.withhold && blockIdx.x == 0 && epoch == 0) {
-      res = bwait(A, g);  // withheld arrival: nobody can pass this barrier
-    } else {
-      const unsigned t = atomicAdd(A.bar + 0, 1u);
-      if (t == gridDim.x - 1) {
-        atomicExch(A.bar + 0, 0u);
-        __threadfence();
-        atomicAdd(A.bar + 1, 1u);
-        res = true;
-      } else {
-        res = bwait(A, g);
-      }
-    }
+    if (!(A.withhold && blockIdx.x == 0 && epoch == 1))  // withheld arrival: nobody can pass this barrier
+      asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(A.bar) : "memory");
+    const bool res = bwait(A, epoch * gridDim.x);
     if (!res) atomicExch(A.bar + 2, 1u);
-    __threadfence();
-    ok = res && *(volatile unsigned*)(A.bar + 2) == 0;
+    ok = res;
   }
   __syncthreads();
-  ++epoch;
   return ok;
 }
 

@@ -71,7 +71,9 @@ struct BatchArgs {
   int ntile_levels;      // max kc over instances
   const int2* citems;    // coarse phase: (instance, first row of a dense product) or (instance, -1)
   int ncitems;
-  double* partials;      // one per level-0 tile, then one per level-0 strip
+  double* partials;      // one per level-0 tile, then one per level-0 strip; the same again for (p, Ap)
+  int pstride;
+  int fold;              // (r, z) and (p, Ap) are summed by the phases that use them
   unsigned* bar;         // [0] arrivals, [2] error, [4..5] active counts
   int sweeps;
   float omega, s;
@@ -409,10 +411,33 @@ __device__ __forceinline__ float s_up(const LevelDev& L, const Strip& t, const f
   return s_up<3>(L, t.u0, t.u1, t.y0, t.y1, b, xin, xout, e, omega, s, ring);
 }
 
-__device__ __forceinline__ void warp_partial(const BatchArgs& A, int slot, float acc) {
+// Sum of an instance's strip partials, the same bits in every warp that forms
+// it; kept while a warp's next strip is of the same instance.  The phases
+// after (r, z) and (p, Ap) form theirs so where no instance has more than
+// kFoldStrips partials, four a lane; else a phase of their own does it, which
+// with its barrier takes 4 us.  256 instances of sides 64-512 (80 partials):
+// 18.3 -> 17.9 ms, four of 64-192 (96): 2.33 -> 2.14; with 640 partials (four
+// of 64-512) the phases are faster, 3.66 against 3.87.
+constexpr int kFoldStrips = 128;
+struct StripSum {
+  int inst = -1;
+  double tot = 0.0;
+  __device__ __forceinline__ double of(const double* partials, const BInst& I, int id) {
+    if (id != inst) {
+      inst = id;
+      tot = 0.0;
+#pragma unroll 4
+      for (int j = threadIdx.x & 31; j < I.nstrips0; j += 32) tot += __ldcg(partials + I.wslot0 + j);
+      for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(kFull, tot, o);
+    }
+    return tot;
+  }
+};
+
+__device__ __forceinline__ void warp_partial(double* partials, int slot, float acc) {
   double t = (double)acc;
   for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(kFull, t, o);
-  if ((threadIdx.x & 31) == 0) A.partials[slot] = t;
+  if ((threadIdx.x & 31) == 0) partials[slot] = t;
 }
 
 // ---------------------------------------------------------------------------
@@ -559,9 +584,9 @@ __device__ __forceinline__ double block_total(float v) {
 }
 
 // per-instance fixed-order reduction of the level-0 partial slots
-__device__ __forceinline__ double reduce_slots(const BatchArgs& A, int slot0, int n) {
+__device__ __forceinline__ double reduce_slots(const double* partials, int slot0, int n) {
   double acc = 0.0;
-  for (int j = threadIdx.x; j < n; j += blockDim.x) acc += __ldcg(A.partials + slot0 + j);
+  for (int j = threadIdx.x; j < n; j += blockDim.x) acc += __ldcg(partials + slot0 + j);
   __shared__ double sh[32];
   __shared__ double tot;
   const double t = block_sum(acc, sh);
@@ -633,7 +658,7 @@ __global__ void __launch_bounds__(kBThreads, kBBlocks) k_batched(const __grid_co
   if (!grid_barrier(A, epoch)) return;
   for (int w = blockIdx.x; w < A.count; w += gridDim.x) {
     const BInst& I = A.inst[w];
-    const double tot = reduce_slots(A, I.slot0, I.ntiles0);
+    const double tot = reduce_slots(A.partials, I.slot0, I.ntiles0);
     if (threadIdx.x == 0) {
       SolveParams prm = A.prm;
       prm.n_fluid = I.nfluid > 0 ? I.nfluid : 1;
@@ -697,7 +722,7 @@ __global__ void __launch_bounds__(kBThreads, kBBlocks) k_batched(const __grid_co
       SolveState& st = A.st[w];
       if (st.outer_done) continue;
       const BInst& I = A.inst[w];
-      const double tot = reduce_slots(A, I.slot0, I.ntiles0);
+      const double tot = reduce_slots(A.partials, I.slot0, I.ntiles0);
       if (threadIdx.x == 0) {
         const double sig_old_d = st.sigma;
         const double sig_new_d =
@@ -756,7 +781,7 @@ __global__ void __launch_bounds__(kBThreads, kBBlocks) k_batched(const __grid_co
           const LevelDev L = I.lv[k];
           const float acc = s_up(L, Strip(item, L, A.srows[k]), k == 0 ? I.r : I.b[k], I.x[k], k == 0 ? I.z : I.y[k],
                                  I.y[k + 1], A.sweeps, omega, A.s, ring);
-          if (k == 0) warp_partial(A, item.w, acc);
+          if (k == 0) warp_partial(A.partials, item.w, acc);
         }
         const int4* its = A.items[k];
         for (int w = blockIdx.x; k > 0 && w < A.nitems[k]; w += gridDim.x) {
@@ -767,61 +792,76 @@ __global__ void __launch_bounds__(kBThreads, kBBlocks) k_batched(const __grid_co
         }
         if (!grid_barrier(A, epoch)) return;
       }
-      // (r, z) per instance -> beta
-      for (int w = blockIdx.x; w < A.count; w += gridDim.x) {
-        SolveState& st = A.st[w];
-        if (st.inner_done) continue;
-        const BInst& I = A.inst[w];
-        const double tot = reduce_slots(A, I.wslot0, I.nstrips0);
-        if (threadIdx.x == 0) {
-          st.rz = tot;
-          st.beta = (st.first || !st.krylov) ? 0.0 : tot / st.rz_old;
-          st.rz_old = tot;
+      // beta from (r, z), p = z + beta p, (p, Ap); an instance's first strip
+      // keeps (r, z) for the next phase, which nothing reads in this one
+      if (!A.fold) {
+        for (int w = blockIdx.x; w < A.count; w += gridDim.x) {
+          SolveState& st = A.st[w];
+          if (st.inner_done) continue;
+          const double tot = reduce_slots(A.partials, A.inst[w].wslot0, A.inst[w].nstrips0);
+          if (threadIdx.x == 0) {
+            st.rz = tot;
+            st.beta = (st.first || !st.krylov) ? 0.0 : tot / st.rz_old;
+          }
         }
+        if (!grid_barrier(A, epoch)) return;
       }
-      if (!grid_barrier(A, epoch)) return;
-      // p = z + beta p, (p, Ap)
+      StripSum rz;
       for (int w = wid; w < A.nstrips[0]; w += nw) {
         const int4 item = A.strips[0][w];
-        const SolveState& st = A.st[item.x];
+        SolveState& st = A.st[item.x];
         if (st.inner_done) continue;
         const BInst& I = A.inst[item.x];
         const LevelDev L = I.lv[0];
         const bool first = st.first || !st.krylov;
-        const float beta = first ? 0.f : (float)st.beta;
+        const double tot = A.fold ? rz.of(A.partials, I, item.x) : st.rz;
+        const float beta = first ? 0.f : (float)(A.fold ? tot / st.rz_old : st.beta);
         const float* pold = (st.it & 1) ? I.p1 : I.p0;
         float* pnew = (st.it & 1) ? I.p0 : I.p1;
         const Strip t(item, L, A.srows[0]);
-        warp_partial(A, item.w,
+        warp_partial(A.partials + A.pstride, item.w,
                      s_pupdate(L, t.u0, t.u1, t.y0, t.y1, I.z, pold, pnew, beta, first, ring));
+        if (A.fold && item.w == I.wslot0 && (threadIdx.x & 31) == 0) st.rz = tot;
       }
       if (!grid_barrier(A, epoch)) return;
-      for (int w = blockIdx.x; w < A.count; w += gridDim.x) {
-        SolveState& st = A.st[w];
-        if (st.inner_done) continue;
-        const double tot = reduce_slots(A, A.inst[w].wslot0, A.inst[w].nstrips0);
-        if (threadIdx.x == 0) {
-          st.pAp = tot;
-          st.alpha = st.krylov ? st.rz / tot : 1.0;
+      // alpha from (p, Ap), d += alpha p, r -= alpha Ap, ||r||^2
+      if (!A.fold) {
+        for (int w = blockIdx.x; w < A.count; w += gridDim.x) {
+          SolveState& st = A.st[w];
+          if (st.inner_done) continue;
+          const double tot = reduce_slots(A.partials + A.pstride, A.inst[w].wslot0, A.inst[w].nstrips0);
+          if (threadIdx.x == 0) {
+            st.pAp = tot;
+            st.alpha = st.krylov ? st.rz / tot : 1.0;
+          }
         }
+        if (!grid_barrier(A, epoch)) return;
       }
-      if (!grid_barrier(A, epoch)) return;
-      // d += alpha p, r -= alpha Ap, ||r||^2
+      StripSum pap;
       for (int w = wid; w < A.nstrips[0]; w += nw) {
         const int4 item = A.strips[0][A.nstrips[0] - 1 - w];
-        const SolveState& st = A.st[item.x];
+        SolveState& st = A.st[item.x];
         if (st.inner_done) continue;
         const BInst& I = A.inst[item.x];
         const LevelDev L = I.lv[0];
+        const double tot = A.fold ? pap.of(A.partials + A.pstride, I, item.x) : st.pAp;
+        const double alpha = !A.fold ? st.alpha : st.krylov ? st.rz / tot : 1.0;
         const Strip t(item, L, A.srows[0]);
-        warp_partial(A, item.w, s_xrupdate(L, t.u0, t.u1, t.y0, t.y1, (st.it & 1) ? I.p0 : I.p1, I.d, I.r,
-                                           (float)st.alpha, st.first != 0, ring));
+        warp_partial(A.partials, item.w, s_xrupdate(L, t.u0, t.u1, t.y0, t.y1, (st.it & 1) ? I.p0 : I.p1, I.d, I.r,
+                                                    (float)alpha, st.first != 0, ring));
+        if (item.w == I.wslot0 && (threadIdx.x & 31) == 0) {
+          if (A.fold) {
+            st.pAp = tot;
+            st.alpha = alpha;
+          }
+          st.rz_old = st.rz;
+        }
       }
       if (!grid_barrier(A, epoch)) return;
       for (int w = blockIdx.x; w < A.count; w += gridDim.x) {
         SolveState& st = A.st[w];
         if (st.inner_done) continue;
-        const double tot = reduce_slots(A, A.inst[w].wslot0, A.inst[w].nstrips0);
+        const double tot = reduce_slots(A.partials, A.inst[w].wslot0, A.inst[w].nstrips0);
         if (threadIdx.x == 0) inner_decide(&st, tot);
         __syncthreads();
         count_active(A, cslot, !st.inner_done);
@@ -897,7 +937,7 @@ struct mg_batch_s {
   void** h_ptrs;                 // pinned staging of the pointer tables
   std::vector<int4*> d_items, d_strips;
   int nstrips[kMaxLevels], srows[kMaxLevels];
-  int strip_slot0;               // first partial slot of the strips
+  int strip_slot0, pstride;      // first partial slot of the strips, slots in all
   int2* d_citems;
   int ncitems;
   int nitems[kMaxLevels];
@@ -985,6 +1025,10 @@ static mg_status batched_launch(mg_batch_s* B, int tile, int sweeps, double tol,
   A.citems = B->d_citems;
   A.ncitems = B->ncitems;
   A.partials = B->d_partials;
+  A.pstride = B->pstride;
+  A.fold = 1;
+  for (const BInst& I : B->inst)
+    if (I.nstrips0 > kFoldStrips) A.fold = 0;
   A.bar = B->d_bar;
   A.sweeps = sweeps;
   A.omega = (float)B->opt.omega;
@@ -1185,7 +1229,8 @@ mg_status mg_create_batched(mg_batch* out, int count, const int64_t* shapes, con
   B->strip_slot0 = (int)max_slots;
   for (int i = 0; i < count; ++i)
     max_slots += (long long)strip_count(B->inst[i].nx) * ((B->inst[i].ny + kStripRows[0] - 1) / kStripRows[0]);
-  const size_t off_partials = reserve((size_t)max_slots * 8);
+  B->pstride = (int)max_slots;
+  const size_t off_partials = reserve((size_t)max_slots * 2 * 8);
   const size_t off_bar = reserve(64);
   cudaError_t ce = cudaMalloc((void**)&B->pool, bytes);
   if (ce != cudaSuccess) {

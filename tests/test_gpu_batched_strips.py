@@ -40,6 +40,27 @@ def test_a_choice_taken_up_again_gives_the_same_bits(L):  # noqa: F811
 SIDES = [(128, 32), (132, 28), (248, 16), (256, 16), (500, 8), (64, 60), (40, 28)]
 
 
+def test_more_partials_than_a_warp_sums(L):  # noqa: F811
+    """An instance of more than 128 strips (its sums have phases of their own)
+    beside small ones; relative residual as asked for."""
+    shapes, spacings, solids, rhs = make_batch([(512, 512), (64, 64), (160, 96)], seed=9)
+    masks = [None if s is None else torch.from_numpy(s.astype(np.uint8)).cuda() for s in solids]
+    b = L.mg_create_batched(shapes, spacings, BC, masks)
+    try:
+        bt = [torch.from_numpy(r).cuda() for r in rhs]
+        xt = [torch.zeros_like(t) for t in bt]
+        status, stats = L.mg_solve_batched(b, bt, xt, 1e-6)
+    finally:
+        L.mg_destroy_batched(b)
+    assert status == L.MG_OK and all(s["relres"] <= 1e-6 for s in stats)
+    for (nx, ny), h, solid, r, x in zip(shapes, spacings, solids, rhs, xt):
+        lv = P.Level((ny, nx), h, BC, solid)
+        b64, x64 = r.astype(np.float64) * lv.fluid, x.cpu().numpy().astype(np.float64)
+        # float32 rounding of x passes through the operator: 6e-8 ||A|| ||x|| / ||b||
+        bound = 1e-6 + 6e-8 * 8 * (max(nx, ny) + 1) ** 2 * np.linalg.norm(x64) / np.linalg.norm(b64)
+        assert np.linalg.norm(b64 - P.apply_A(lv, x64)) / np.linalg.norm(b64) <= bound
+
+
 @pytest.mark.parametrize("sweeps", [1, 2, 3])
 @pytest.mark.parametrize("bc,with_masks", [((0, 0, 0, 0), True), ((1, 0, 1, 1), False), ((0, 1, 1, 0), True)])
 def test_strips_match_oracle(L, sweeps, bc, with_masks):  # noqa: F811

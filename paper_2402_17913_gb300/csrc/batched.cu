@@ -319,25 +319,6 @@ __device__ __noinline__ void b_up_h(const LevelDev& L, int tx, int ty, const flo
 }
 
 // ---------------------------------------------------------------------------
-// float4 region of the refinement residual: the level-0 tile plus one group
-// of four cells on each side in x and H rows in y, so a global access is a
-// whole float4 (uchar4 for the cell bytes) that is either all on the grid or
-// all off it (an instance's width is a multiple of 4).
-template <int TX, int TY, int H>
-struct VReg {
-  static constexpr int RX = TX + 8, RY = TY + 2 * H, R = RX * RY, W4 = RX / 4, PAD = 4;
-  static constexpr int A = R + 2 * PAD;  // floats per padded array
-  static constexpr int NG = RY * W4;     // groups in the region
-  int ox, oy;
-  __device__ __forceinline__ VReg(int tx, int ty) : ox(tx * TX - 4), oy(ty * TY - H) {}
-  // global index of group q's first cell, or -1 off the grid
-  __device__ __forceinline__ int gidx(const LevelDev& L, int q) const {
-    const int gx = ox + 4 * (q % W4), gy = oy + q / W4;
-    if (q >= NG || gx < 0 || gx >= L.nx || gy < 0 || gy >= L.ny) return -1;
-    return gy * L.nx + gx;
-  }
-};
-
 __device__ __forceinline__ float4 lds4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 __device__ __forceinline__ void sts4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
 __device__ __forceinline__ float lane(const float4& v, int k) {
@@ -358,16 +339,6 @@ __device__ __forceinline__ uchar4 v_cells(const LevelDev& L, int gi) {
   if (!L.cell) return make_uchar4(kFluidBit, kFluidBit, kFluidBit, kFluidBit);
   return *reinterpret_cast<const uchar4*>(L.cell + gi);
 }
-// left / right / down / up neighbours of lane k of the group at li
-struct VNb {
-  float4 c, d, u;
-  float l, r;
-  __device__ __forceinline__ VNb(const float* x, int li, int RX)
-      : c(lds4(x + li)), d(lds4(x + li - RX)), u(lds4(x + li + RX)), l(x[li - 1]), r(x[li + 4]) {}
-  __device__ __forceinline__ float left(int k) const { return k == 0 ? l : lane(c, k - 1); }
-  __device__ __forceinline__ float right(int k) const { return k == 3 ? r : lane(c, k + 1); }
-};
-
 // legs of a level whose width is not a multiple of 4 (tiles), and of one item
 // of any other level (a strip of rows, one warp)
 template <int TX, int TY>
@@ -487,84 +458,6 @@ __device__ void v_result(const LevelDev& L, int tx, int ty, const float2* __rest
   }
 }
 
-// refinement residual of the float-float iterate after x += sigma_old d
-// (when `update`): the iterate of the tile and a one-cell ring is staged in
-// shared memory as (hi, lo) planes, then r = c b - A' x per fluid cell in
-// float-float, scaled by 1 / sigma_new into the CG right-hand side; returns
-// the thread's share of ||r||^2
-template <int TX, int TY>
-__device__ float v_resid(const BInst& I, const LevelDev& L, int tx, int ty, const float* __restrict__ b,
-                         const float2* __restrict__ xin, float2* __restrict__ xo, bool update, float sig_old,
-                         float inv_sig_new, float* S) {
-  using G = VReg<TX, TY, 1>;
-  const G g(tx, ty);
-  float* sh = S + G::PAD;
-  float* sl = sh + G::A;
-  uint8_t* sm = reinterpret_cast<uint8_t*>(S + 2 * G::A);
-  auto xv = [&](float hi, float lo, float dd) -> ff {
-    if (!update) return {hi, lo};
-    const ff s2 = two_sum(hi, sig_old * dd);
-    return quick_two_sum(s2.hi, s2.lo + lo);
-  };
-  __syncthreads();
-  for (int q = threadIdx.x; q < G::NG; q += kBThreads) {
-    const int gi = g.gidx(L, q);
-    const int li = (q / G::W4) * G::RX + 4 * (q % G::W4);
-    float4 h = make_float4(0.f, 0.f, 0.f, 0.f), l = h;
-    uchar4 m = make_uchar4(0, 0, 0, 0);
-    if (gi >= 0) {
-      m = v_cells(L, gi);
-      const float4 a = reinterpret_cast<const float4*>(xin + gi)[0], c = reinterpret_cast<const float4*>(xin + gi)[1];
-      const float4 dd = update ? *reinterpret_cast<const float4*>(I.d + gi) : make_float4(0.f, 0.f, 0.f, 0.f);
-      const ff v0 = xv(a.x, a.y, dd.x), v1 = xv(a.z, a.w, dd.y), v2 = xv(c.x, c.y, dd.z), v3 = xv(c.z, c.w, dd.w);
-      h = make_float4(v0.hi, v1.hi, v2.hi, v3.hi);
-      l = make_float4(v0.lo, v1.lo, v2.lo, v3.lo);
-    }
-    sts4(sh + li, h);
-    sts4(sl + li, l);
-    *reinterpret_cast<uchar4*>(sm + li) = m;
-  }
-  __syncthreads();
-  float acc = 0.f;
-  constexpr int T4 = TX / 4;
-  for (int q = threadIdx.x; q < TY * T4; q += kBThreads) {
-    const int row = q / T4, c4 = q % T4;
-    const int gx = tx * TX + 4 * c4, gy = ty * TY + row;
-    if (gx >= L.nx || gy >= L.ny) continue;
-    const int gi = gy * L.nx + gx;
-    const int li = (row + 1) * G::RX + 4 * (c4 + 1);
-    const VNb H(sh, li, G::RX), Lo(sl, li, G::RX);
-    const uchar4 m4 = *reinterpret_cast<const uchar4*>(sm + li);
-    const float4 bb = *reinterpret_cast<const float4*>(b + gi);
-    float4 rv = make_float4(0.f, 0.f, 0.f, 0.f), oh = rv, ol = rv;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const uint8_t m = lane(m4, k);
-      if (!m) continue;
-      const int kx = L.cell ? (m & 3) : axis_count(gx + k, L.nx, L.bcD, 0);
-      const int ky = L.cell ? ((m >> 2) & 3) : axis_count(gy, L.ny, L.bcD, 2);
-      const ff xc = {lane(H.c, k), lane(Lo.c, k)};
-      const ff xl = {H.left(k), Lo.left(k)}, xr = {H.right(k), Lo.right(k)};
-      const ff xd = {lane(H.d, k), lane(Lo.d, k)}, xu = {lane(H.u, k), lane(Lo.u, k)};
-      ff ax = ff_mul(ff_add(ff_mul(xc, ff{(float)kx, 0.f}), ff_neg(ff_add(xl, xr))), I.wff[0]);
-      ax = ff_add(ax, ff_mul(ff_add(ff_mul(xc, ff{(float)ky, 0.f}), ff_neg(ff_add(xd, xu))), I.wff[1]));
-      const ff r = ff_add(ff_mul(ff{lane(bb, k), 0.f}, I.cff), ff_neg(ax));
-      const float rs = r.hi + r.lo;
-      set_lane(rv, k, rs * inv_sig_new);
-      acc = fmaf(rs, rs, acc);
-      set_lane(oh, k, xc.hi);
-      set_lane(ol, k, xc.lo);
-    }
-    *reinterpret_cast<float4*>(I.r + gi) = rv;
-    if (update) {
-      float4* o = reinterpret_cast<float4*>(xo + gi);
-      o[0] = make_float4(oh.x, ol.x, oh.y, ol.y);
-      o[1] = make_float4(oh.z, ol.z, oh.w, ol.w);
-    }
-  }
-  return acc;
-}
-
 // cells of a level-0 tile, one by one: callback(i, x, y)
 template <int TX, int TY, typename F>
 __device__ __forceinline__ void b_cells(const BInst& I, int tx, int ty, F&& f) {
@@ -670,14 +563,31 @@ __global__ void __launch_bounds__(kBThreads, kBBlocks) k_batched(const __grid_co
   // ---- refinement loop
   for (int outer = 0; outer <= A.prm.max_outer; ++outer) {
     const bool update = outer > 0;
-    // residual of the float-float iterate (after x += sigma d')
+    // residual of the float-float iterate (after x += sigma d'): strips where
+    // the caller's right-hand side is 16-byte aligned, else cell by cell
+    for (int w = wid; w < A.nstrips[0]; w += nw) {
+      const int4 item = A.strips[0][w];
+      const SolveState& st = A.st[item.x];
+      const float* b = A.rhs[item.x];
+      if (st.outer_done || !aligned16(b)) continue;
+      const BInst& I = A.inst[item.x];
+      const LevelDev L = I.lv[0];
+      const int cur = A.cur[item.x];
+      const double sig_old = st.sigma;
+      const double sig_new =
+          update ? pow2_floor(sig_old * sqrt(fmax(st.rnorm2, 1e-300) / (double)st.n_fluid)) : sig_old;
+      const Strip t(item, L, A.srows[0]);
+      warp_partial(A.partials, item.w,
+                   s_resid(L, t.u0, t.u1, t.y0, t.y1, b, cur ? I.xf1 : I.xf0, cur ? I.xf0 : I.xf1, I.d, I.r, I.wff[0],
+                           I.wff[1], I.cff, update, (float)sig_old, (float)(1.0 / sig_new), ring));
+    }
     for (int w = blockIdx.x; w < n0; w += gridDim.x) {
       const int4 item = it0[w];
       SolveState& st = A.st[item.x];
-      if (st.outer_done) continue;
+      const float* b = A.rhs[item.x];
+      if (st.outer_done || aligned16(b)) continue;
       const BInst& I = A.inst[item.x];
       const LevelDev& L = I.lv[0];
-      const float* b = A.rhs[item.x];
       const int cur = A.cur[item.x];
       const float2* xin = cur ? I.xf1 : I.xf0;
       float2* xo = cur ? I.xf0 : I.xf1;
@@ -692,8 +602,7 @@ __global__ void __launch_bounds__(kBThreads, kBBlocks) k_batched(const __grid_co
         return quick_two_sum(s2.hi, s2.lo + q.y);
       };
       float acc = 0.f;
-      if (aligned16(b)) acc = v_resid<TX, TY>(I, L, item.y, item.z, b, xin, xo, update, sig_old, inv_sig_new, S);
-      else b_cells<TX, TY>(I, item.y, item.z, [&](size_t i, int cx, int cy) {
+      b_cells<TX, TY>(I, item.y, item.z, [&](size_t i, int cx, int cy) {
         const uint8_t m = L.cell ? L.cell[i] : kFluidBit;
         if (!m) {
           if (update) xo[i] = make_float2(0.f, 0.f);
@@ -722,7 +631,8 @@ __global__ void __launch_bounds__(kBThreads, kBBlocks) k_batched(const __grid_co
       SolveState& st = A.st[w];
       if (st.outer_done) continue;
       const BInst& I = A.inst[w];
-      const double tot = reduce_slots(A.partials, I.slot0, I.ntiles0);
+      const double tot = aligned16(A.rhs[w]) ? reduce_slots(A.partials, I.wslot0, I.nstrips0)
+                                             : reduce_slots(A.partials, I.slot0, I.ntiles0);
       if (threadIdx.x == 0) {
         const double sig_old_d = st.sigma;
         const double sig_new_d =
@@ -959,12 +869,9 @@ struct mg_batch_s {
 
 static size_t batched_smem(int tx, int ty, int sweeps, size_t coarse_bytes) {
   const int h = sweeps < 1 ? 1 : (sweeps > 3 ? 3 : sweeps);
-  // scalar tile: halo h on every side; the residual's tile: one group of four
-  // in x and one row in y, (hi, lo) planes padded by 4 floats at both ends;
-  // the warps' rings
-  const size_t R = (size_t)(tx + 2 * h) * (ty + 2 * h), Rv = (size_t)(tx + 8) * (ty + 2);
+  // scalar tile: halo h on every side; the warps' rings
+  const size_t R = (size_t)(tx + 2 * h) * (ty + 2 * h);
   size_t m = 4 * R * 4 + ((R + 15) & ~size_t(15));  // b, two iterates, omega/d; cell bytes
-  m = std::max(m, 2 * (Rv + 8) * 4 + ((Rv + 15) & ~size_t(15)));
   m = std::max(m, (size_t)(kBThreads / 32) * kSRing);
   return std::max(m, coarse_bytes);
 }

@@ -18,10 +18,12 @@
 // 72 x 38 cells for 64 x 32 behind seven block barriers, 6 us a tile at four
 // blocks per SM: 28.1 -> 21.0 ms a solve, -> 19.7 with paired arithmetic and
 // with the phases walking the list up and down in turn, -> 18.8 with Ap
-// formed again instead of stored.
+// formed again instead of stored, -> 18.2 with cheaper barriers and sums, ->
+// 17.5 with the refinement residual on strips too.
 #pragma once
 
 #include "npmg_internal.cuh"
+#include "refine.cuh"
 
 namespace npmg {
 
@@ -30,8 +32,9 @@ constexpr int kSSlots = kSD + 1;
 constexpr int kSRowDown = 32 * 16 + 32 * 4;                     // b, cell bytes
 constexpr int kSRowUp = 2 * 32 * 16 + 32 * 8 + 32 * 4;          // x (or z), b (or p), e, cell bytes
 constexpr int kSRowXr = 3 * 32 * 16 + 32 * 4;                  // p, d, r, cell bytes
-constexpr int kSRing = kSSlots * kSRowXr;                       // bytes of one warp's ring
-static_assert(kSRowXr >= kSRowUp && kSRowUp >= kSRowDown, "the ring holds the longest rows");
+constexpr int kSRowRes = 4 * 32 * 16 + 32 * 4;                 // iterate (hi, lo), d, b, cell bytes
+constexpr int kSRing = kSSlots * kSRowRes;                      // bytes of one warp's ring
+static_assert(kSRowRes >= kSRowXr && kSRowXr >= kSRowUp && kSRowUp >= kSRowDown, "the ring holds the longest rows");
 constexpr unsigned kFull = 0xffffffffu;
 
 __device__ __forceinline__ uint32_t s_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -400,6 +403,95 @@ __device__ __forceinline__ float s_xrupdate(const LevelDev& L, int u0, int u1, i
 #pragma unroll
           for (int j = 0; j < 4; ++j) acc = fmaf(r.get(j), r.get(j), acc);
         }
+      });
+  return acc;
+}
+
+// Refinement residual of the float-float iterate after x += sigma_old d (when
+// `update`), r = (c b - A' x) inv_sig in float-float on the fluid cells.  As
+// block tiles between two barriers it ran at a fifth of the copy rate (256
+// instances: 18.2 -> 17.5 ms a solve); returns the lane's share of ||r||^2 (before inv_sig).
+// kx, ky: link counts; the iterate and d hold 0 off the fluid.
+__device__ __forceinline__ float s_resid(const LevelDev& L, int u0, int u1, int y0, int y1,
+                                         const float* __restrict__ b, const float2* __restrict__ xin,
+                                         float2* __restrict__ xo, const float* __restrict__ dv,
+                                         float* __restrict__ rv, ff wx, ff wy, ff cff, bool update, float sig_old,
+                                         float inv_sig, unsigned char* ring) {
+  const SLane c = s_lane(L, u0, u1, 1.f);
+  float hi[3][4], lo[3][4];
+  unsigned mp = 0u;
+  float acc = 0.f;
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) hi[k][j] = lo[k][j] = 0.f;
+  s_walk<kSRowRes>(
+      y0 - 1, y1 - y0 + 2, ring,
+      [&](int p, unsigned char* slot) {
+        // row p of the iterate, d and the cell bytes, row p - 1 of b
+        const bool f = c.in && p >= 0 && p < L.ny, fo = c.own && p > y0;
+        const int at = f ? p * L.nx + c.go : 0, ao = fo ? (p - 1) * L.nx + c.go : 0;
+        const uint32_t sl = s_addr(slot);
+        s_copy16(sl + c.lane * 32, xin + at, f);
+        s_copy16(sl + c.lane * 32 + 16, xin + at + 2, f);
+        if (update) s_copy16(sl + 1024 + c.lane * 16, dv + at, f);
+        s_copy16(sl + 1536 + c.lane * 16, b + ao, fo);
+        if (L.cell) s_copy<4>(sl + 2048 + c.lane * 4, L.cell + at, f);
+      },
+      [&](int p, const unsigned char* slot) {
+        const Quad q0 = s_get(slot + c.lane * 32), q1 = s_get(slot + c.lane * 32 + 16);
+        const float xh[4] = {q0.a.x, q0.b.x, q1.a.x, q1.b.x}, xl[4] = {q0.a.y, q0.b.y, q1.a.y, q1.b.y};
+        Quad d;
+        d.a = d.b = make_float2(0.f, 0.f);
+        if (update) d = s_get(slot + 1024 + c.lane * 16);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          hi[0][j] = hi[1][j];
+          lo[0][j] = lo[1][j];
+          hi[1][j] = hi[2][j];
+          lo[1][j] = lo[2][j];
+          ff v = {xh[j], xl[j]};
+          if (update) {
+            const ff s2 = two_sum(xh[j], sig_old * d.get(j));
+            v = quick_two_sum(s2.hi, s2.lo + xl[j]);
+          }
+          hi[2][j] = v.hi;
+          lo[2][j] = v.lo;
+        }
+        const unsigned m = s_cells(L, c, p, slot + 2048);
+        float lh = __shfl_up_sync(kFull, hi[1][3], 1), ll = __shfl_up_sync(kFull, lo[1][3], 1);
+        float rh = __shfl_down_sync(kFull, hi[1][0], 1), rl = __shfl_down_sync(kFull, lo[1][0], 1);
+        if (c.lane == 0) lh = ll = 0.f;
+        if (c.lane == 31) rh = rl = 0.f;
+        const int o = p - 1;
+        if (o >= y0 && c.own) {
+          const Quad bb = s_get(slot + 1536 + c.lane * 16);
+          Quad r;
+          float oh[4], ol[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const unsigned mj = s_byte(mp, j);
+            const ff xc = {hi[1][j], lo[1][j]};
+            const ff xw = {j == 0 ? lh : hi[1][j - 1], j == 0 ? ll : lo[1][j - 1]};
+            const ff xe = {j == 3 ? rh : hi[1][j + 1], j == 3 ? rl : lo[1][j + 1]};
+            const ff xd = {hi[0][j], lo[0][j]}, xu = {hi[2][j], lo[2][j]};
+            ff ax = ff_mul(ff_add(ff_mul(xc, ff{(float)(mj & 3u), 0.f}), ff_neg(ff_add(xw, xe))), wx);
+            ax = ff_add(ax, ff_mul(ff_add(ff_mul(xc, ff{(float)((mj >> 2) & 3u), 0.f}), ff_neg(ff_add(xd, xu))), wy));
+            const ff rr = ff_add(ff_mul(ff{bb.get(j), 0.f}, cff), ff_neg(ax));
+            const float rs = mj ? rr.hi + rr.lo : 0.f;
+            r.set(j, rs * inv_sig);
+            acc = fmaf(rs, rs, acc);
+            oh[j] = mj ? xc.hi : 0.f;
+            ol[j] = mj ? xc.lo : 0.f;
+          }
+          s_put(rv + o * L.nx + c.gx, r);
+          if (update) {
+            float4* out = reinterpret_cast<float4*>(xo + o * L.nx + c.gx);
+            out[0] = make_float4(oh[0], ol[0], oh[1], ol[1]);
+            out[1] = make_float4(oh[2], ol[2], oh[3], ol[3]);
+          }
+        }
+        mp = m;
       });
   return acc;
 }

@@ -52,9 +52,10 @@ UNIT = "unknowns/s"
 TOL = 1e-6
 
 # Batched solve: bytes per fine cell of one CG iteration (the four fine
-# passes below, plus one cell byte in three of them, plus about a third more
-# for the coarser levels) and of one float-float refinement pass.
-BATCH_ITER_BYTES = 72
+# passes below with A p formed again instead of stored, plus one cell byte in
+# each, plus about a third more for the coarser levels) and of one float-float
+# refinement pass.
+BATCH_ITER_BYTES = 64
 OUTER_BYTES = 28
 KERNEL_CLASSES = ("down_fine", "up_fine", "p_update", "xr_update", "outer")
 

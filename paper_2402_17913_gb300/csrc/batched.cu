@@ -4,14 +4,14 @@
 // Every instance runs the single-grid algorithm (float-float refinement
 // around MG-PCG with the V(pre,post) cycle of Sec. 2.2).  The launch walks the
 // phases of that algorithm in lockstep over all instances; within a phase the
-// blocks share out work items -- (instance, tile) pairs on one level, or
+// blocks share out work items -- strips or tiles of an instance's level, or
 // whole instances for the per-instance steps -- and a grid-wide barrier
 // separates phases.  Phases are aligned by level counted from the finest
 // grid, so a small instance simply has no items in some phases.  An
 // instance that has converged leaves every later work list.  Each
 // instance's levels with <= 1024 cells are one block-local item (the same
 // cycle code as the single-grid coarse kernel).  Reductions are per
-// instance, in a fixed order over per-tile partial slots.
+// instance, in a fixed order over per-strip (per-tile) partial slots.
 //
 // The grid barrier spins a bounded number of times: if a block never
 // arrives, the others give up, raise an error flag and return, and the
@@ -190,7 +190,7 @@ __device__ __forceinline__ int b_gidx(const LevelDev& L, const BReg<TX, TY, H>& 
 
 // down leg of one tile: H sweeps from zero, x, restricted residual (the
 // scalar path, for a level whose width is not a multiple of 4; kept out of
-// line so that its registers do not weigh on the float4 path)
+// line so that its registers do not weigh on the strips)
 template <int TX, int TY, int H>
 __device__ __noinline__ void b_down_h(const LevelDev& L, int tx, int ty, const float* __restrict__ b, float* __restrict__ x,
                          float* __restrict__ bc, float omega, float* S) {

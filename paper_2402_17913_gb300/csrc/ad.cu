@@ -63,6 +63,7 @@ struct State {
   int max_cycles;
   double bnorm2, relres, relres0, l1, l1_first;
   int cycles, done, status;
+  float rscale;         // power of two near 1 / ||b||^2: the grid's sums of r^2 are float32 pairs
   unsigned int counter[2];
   unsigned int checks;  // of the device-side loop
 };
@@ -97,11 +98,14 @@ __global__ void __launch_bounds__(kT) k_ad_init(Lev L, const float* __restrict__
     acc = fmaf(bv, bv, acc);
   }
   double tot;
-  if (grid_sum_last(acc, partials, &st->counter[0], &tot) && threadIdx.x == 0) {
+  // in the caller's units, so in float64 across the threads: its sum passes
+  // the float32 range at an rms of 1.8e16 on 1024^2 (once a solve)
+  if (grid_sum_last((double)acc, partials, &st->counter[0], &tot) && threadIdx.x == 0) {
     st->tol = tol;
     st->l1_tol = l1_tol;
     st->max_cycles = max_cycles;
     st->bnorm2 = tot;
+    st->rscale = tot > 0.0 && isfinite(tot) ? ldexpf(1.f, -max(-126, min(126, ilogb(tot)))) : 1.f;
     st->relres = st->relres0 = 1.0;
     st->l1 = st->l1_first = 0.0;
     st->cycles = 0;
@@ -112,10 +116,12 @@ __global__ void __launch_bounds__(kT) k_ad_init(Lev L, const float* __restrict__
   }
 }
 
-// relres from ||b - A x||^2 and, unless `final`, the stopping decision taken
-// before each cycle: converged, diverged (1000-fold growth) or out of cycles.
-__device__ void decide(State* st, double rr, bool final) {
-  const double rel = st->bnorm2 > 0.0 ? sqrt(rr / st->bnorm2) : 0.0;
+// relres from rscale ||b - A x||^2 and, unless `final`, the stopping decision
+// taken before each cycle: converged, diverged (1000-fold growth, or a
+// right-hand side whose norm is not finite) or out of cycles.
+__device__ void decide(State* st, double srr, bool final) {
+  const double bn2 = st->bnorm2, rr = srr / (double)st->rscale;
+  const double rel = bn2 == 0.0 ? 0.0 : isfinite(bn2) ? sqrt(rr / bn2) : nan("");
   st->relres = rel;
   if (final) return;
   if (st->cycles == 0) st->relres0 = rel;
@@ -214,7 +220,7 @@ __global__ void __launch_bounds__(kT) k_ad_resid(Lev L, const float* __restrict_
     }
   }
   double tot;
-  if (grid_sum_last(acc, partials, &st->counter[0], &tot) && threadIdx.x == 0) decide(st, tot, FINAL);
+  if (grid_sum_last(acc * st->rscale, partials, &st->counter[0], &tot) && threadIdx.x == 0) decide(st, tot, FINAL);
 }
 
 // One relaxed Jacobi sweep over window J, [J, RX - J) x [J, RY - J), of a
@@ -349,7 +355,7 @@ __global__ void __launch_bounds__(kT) k_ad_down_saw(Lev L, const float* __restri
   }
   if (FUSED) {
     double tot;
-    if (grid_sum_last(acc, partials, &st->counter[0], &tot) && threadIdx.x == 0) decide(st, tot, false);
+    if (grid_sum_last(acc * st->rscale, partials, &st->counter[0], &tot) && threadIdx.x == 0) decide(st, tot, false);
   }
 }
 

@@ -559,7 +559,8 @@ __global__ void __launch_bounds__(256) k_outer(LevelDev L, OuterArgs oa, const f
     }
   }
   double tot;
-  if (grid_sum_last(acc, partials, &st->counter[kCntOuter], &tot)) {
+  // r is in the caller's units times c: float64 across the threads (k_init)
+  if (grid_sum_last((double)acc, partials, &st->counter[kCntOuter], &tot)) {
     if (threadIdx.x == 0) {
       outer_decide(st, tot, oa.c2, sig_new_d, UPDATE);
       if (UPDATE && dyn) st->cur ^= 1;
@@ -980,7 +981,9 @@ __global__ void __launch_bounds__(256) k_init(LevelDev L, const float* __restric
     }
   }
   double tot;
-  if (grid_sum_last(acc, partials, &st->counter[kCntInit], &tot)) {
+  // in the caller's units, so in float64 across the threads: its sum passes
+  // the float32 range at an rms of 4.5e15 on 256^3 (once a solve)
+  if (grid_sum_last((double)acc, partials, &st->counter[kCntInit], &tot)) {
     if (threadIdx.x == 0) init_state(st, prm, tot, c);
   }
 }

@@ -51,7 +51,9 @@ __device__ __forceinline__ ff ff_mul(ff a, ff w) {
 // otherwise the tolerance of the next inner solve.
 __device__ __forceinline__ void outer_decide(SolveState* st, double tot, double c2, double sig_new, bool update) {
   const double bn2 = st->bnorm2;
-  const double rel = bn2 > 0.0 ? sqrt(tot / (c2 * bn2)) : 0.0;
+  // a right-hand side whose norm is not finite has no relative residual: NaN,
+  // which ends the solve as diverged
+  const double rel = bn2 == 0.0 ? 0.0 : isfinite(bn2) ? sqrt(tot / (c2 * bn2)) : nan("");
   const double prev = st->relres;
   if (update) st->outer += 1;
   const int o = st->outer;

@@ -1130,9 +1130,15 @@ mg_status mg_create_batched(mg_batch* out, int count, const int64_t* shapes, con
     I.cfloats = 0;
   }
   B->ntile_levels = max_kc;
-  // partial slots: worst case over tile shapes = the smallest tile (32 x 16)
+  // partial slots: per instance the most level-0 tiles any tile shape makes
+  // (32 x 16 on wide grids, 128 x 8 on those at most 32 cells wide)
   long long max_slots = 0;
-  for (int i = 0; i < count; ++i) max_slots += (long long)((B->inst[i].nx + 31) / 32) * ((B->inst[i].ny + 15) / 16);
+  for (int i = 0; i < count; ++i) {
+    long long most = 0;
+    for (const TileChoice& t : kTiles)
+      most = std::max(most, (long long)((B->inst[i].nx + t.tx - 1) / t.tx) * ((B->inst[i].ny + t.ty - 1) / t.ty));
+    max_slots += most;
+  }
   B->strip_slot0 = (int)max_slots;
   for (int i = 0; i < count; ++i)
     max_slots += (long long)strip_count(B->inst[i].nx) * ((B->inst[i].ny + kStripRows[0] - 1) / kStripRows[0]);
@@ -1297,6 +1303,10 @@ static mg_status build_items(mg_batch_s* B, int tile, cudaStream_t s) {
         for (int tx = 0; tx < (nx + TX - 1) / TX; ++tx) items[k].push_back(make_int4(i, tx, ty, k == 0 ? slot++ : -1));
     }
     I.ntiles0 = slot - I.slot0;
+  }
+  if (slot > B->strip_slot0) {
+    set_error("batched solve: %d level-0 tiles, %d partial slots", slot, B->strip_slot0);
+    return MG_ERR_INVALID;
   }
   // the captured launches hold the lists freed here
   for (int t = 0; t < kNTiles; ++t)

@@ -684,8 +684,9 @@ __global__ void __launch_bounds__(256) k_outer64(LevelDev L, double w0, double w
 // the exact 77-bit product of the significands cut to 59 bits, and the
 // products with the link counts and the rest of the sum are exact integer
 // arithmetic.  The cut-off parts are below 2^-59 of the largest value, where
-// a float64 sum rounds at 2^-53.  The result is normalised and rounded to
-// float32 once; ||r|| is summed from r' in float-float.
+// a float64 sum rounds at 2^-53.  The result is normalised to a pair of
+// float32 numbers (48 bits): r' is the pair rounded once, and ||r|| sums the
+// squares of the pairs.
 __device__ __forceinline__ unsigned magnitude(double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; }
 
 __device__ __forceinline__ long long fix_of(double v, int emax) {
@@ -713,17 +714,19 @@ __device__ __forceinline__ long long fix_cb(FixC c, float b, int emax) {
   return ((long long)t ^ s) - s;
 }
 
-// v 2^(emax - 1081) as float32.
-__device__ __forceinline__ float fix_float(long long v, int emax) {
+// v 2^(emax - 1081) as a float32 pair: the leading 24 and the next 24 bits.
+__device__ __forceinline__ float2 fix_pair(long long v, int emax) {
   const unsigned long long a = (unsigned long long)(v < 0 ? -v : v);
   const int z = __clzll((long long)a);
-  const unsigned top = (unsigned)((a << (z & 63)) >> 32);
+  const unsigned long long t = a << (z & 63);
+  const unsigned top = (unsigned)(t >> 32), low = (unsigned)t;
   // top 2^(32 - z) 2^(emax - 1081), in two factors that are float32 numbers
   const int s = emax - 1049 - z, s1 = s >> 1, s2 = s - s1;
   const float f1 = __int_as_float((max(-126, min(127, s1)) + 127) << 23);
   const float f2 = __int_as_float((max(-126, min(127, s2)) + 127) << 23);
-  const float r = a ? (float)top * f1 * f2 : 0.f;
-  return v < 0 ? -r : r;
+  const float hi = a ? (float)(top & ~255u) * f1 * f2 : 0.f;
+  const float lo = a ? (float)(top << 24 | low >> 8) * 0x1p-24f * f1 * f2 : 0.f;
+  return v < 0 ? make_float2(-hi, -lo) : make_float2(hi, lo);
 }
 
 template <bool VEC>
@@ -796,7 +799,10 @@ __global__ void __launch_bounds__(256, DIM == 3 ? 2 : 3) k_outer_fix(LevelDev L,
     if (odd || emax < 128) {
       // non-finite: the solve ends as diverged; below 2^-894: 0 in float32
 #pragma unroll
-      for (int k = 0; k < 4; ++k) rv[k] = odd && m[k] ? __int_as_float(0x7fc00000) : 0.f;
+      for (int k = 0; k < 4; ++k) {
+        rv[k] = odd && m[k] ? __int_as_float(0x7fc00000) : 0.f;
+        acc.x += rv[k];
+      }
     } else {
       long long X[6];  // x0-1 .. x0+4
       X[0] = fix_of(xl, emax);
@@ -816,18 +822,19 @@ __global__ void __launch_bounds__(256, DIM == 3 ? 2 : 3) k_outer_fix(LevelDev L,
         // 2^59
         const long long s =
             fix_cb(c, m[k] ? bv[k] : 0.f, emax) - q * X[k + 1] + X[k] + X[k + 2] + fix_of(yu[k], emax);
-        rv[k] = m[k] ? fix_float(s, emax) * inv_sig_new : 0.f;
+        const float2 r = fix_pair(s, emax);
+        const float hi = m[k] ? r.x * inv_sig_new : 0.f, lo = m[k] ? r.y * inv_sig_new : 0.f;
+        rv[k] = hi + lo;
+        const float p = hi * hi;
+        acc = pair_add(acc, make_float2(p, fmaf(2.f * hi, lo, fmaf(hi, hi, -p))));
       }
-    }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const float p = rv[k] * rv[k];
-      acc = pair_add(acc, make_float2(p, fmaf(rv[k], rv[k], -p)));
     }
     st4(rprime, n.i, x0, L.nx, rv);
   }
   double tot;
-  if (grid_sum_last(acc, partials, &st->counter[kCntOuter], &tot)) {
+  // float64 across the threads: a guess far from the solution takes the sum
+  // past the float32 range (once a refinement step)
+  if (grid_sum_last((double)acc.x + (double)acc.y, partials, &st->counter[kCntOuter], &tot)) {
     if (threadIdx.x == 0) {
       outer_decide(st, tot * sig_new * sig_new, c2, sig_new, UPDATE);
       if (UPDATE && dyn) st->cur ^= 1;

@@ -708,8 +708,9 @@ __device__ __forceinline__ long long fix_cb(FixC c, float b, int emax) {
   const unsigned u = __float_as_uint(b), m = (u & 0x7fffffu) | 0x800000u;
   const int eb = (int)((u >> 23) & 255u);
   unsigned long long t = ((unsigned long long)m * c.mhi << 14) + ((unsigned long long)m * c.mlo >> 18);
-  t >>= min(emax - (eb + c.e), 63);
-  if (eb == 0) t = 0;  // zero (a denormal b has ||b||^2 = 0 in float32)
+  // a zero b (and a denormal one, whose ||b||^2 is 0 in float32) is not among
+  // the values that emax covers
+  t = eb == 0 ? 0 : t >> min(emax - (eb + c.e), 63);
   const long long s = (long long)((int)u >> 31);
   return ((long long)t ^ s) - s;
 }

@@ -220,7 +220,8 @@ __global__ void __launch_bounds__(kT) k_ad_resid(Lev L, const float* __restrict_
     }
   }
   double tot;
-  if (grid_sum_last(acc * st->rscale, partials, &st->counter[0], &tot) && threadIdx.x == 0) decide(st, tot, FINAL);
+  if (grid_sum_last(make_float2(acc * st->rscale, 0.f), partials, &st->counter[0], &tot) && threadIdx.x == 0)
+    decide(st, tot, FINAL);
 }
 
 // One relaxed Jacobi sweep over window J, [J, RX - J) x [J, RY - J), of a
@@ -355,7 +356,8 @@ __global__ void __launch_bounds__(kT) k_ad_down_saw(Lev L, const float* __restri
   }
   if (FUSED) {
     double tot;
-    if (grid_sum_last(acc * st->rscale, partials, &st->counter[0], &tot) && threadIdx.x == 0) decide(st, tot, false);
+    if (grid_sum_last(make_float2(acc * st->rscale, 0.f), partials, &st->counter[0], &tot) && threadIdx.x == 0)
+      decide(st, tot, false);
   }
 }
 
@@ -426,7 +428,7 @@ __global__ void __launch_bounds__(kT) k_ad_up(Lev L, const float* __restrict__ b
   }
   if (FINEST) {
     double t;
-    if (grid_sum_last(acc, partials, &st->counter[1], &t) && threadIdx.x == 0) cycle_end(st, t);
+    if (grid_sum_last(make_float2(acc, 0.f), partials, &st->counter[1], &t) && threadIdx.x == 0) cycle_end(st, t);
   }
 }
 
@@ -545,7 +547,7 @@ __global__ void __launch_bounds__(kT) k_ad_up_c(Lev L, const float* __restrict__
   }
   if (FINEST) {
     double t;
-    if (grid_sum_last(acc, partials, &st->counter[1], &t) && threadIdx.x == 0) cycle_end(st, t);
+    if (grid_sum_last(make_float2(acc, 0.f), partials, &st->counter[1], &t) && threadIdx.x == 0) cycle_end(st, t);
   }
 }
 

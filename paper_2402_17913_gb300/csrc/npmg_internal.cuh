@@ -191,8 +191,14 @@ __device__ __forceinline__ bool grid_sum_last(float2 v, double* partials, unsign
   return true;
 }
 
+// The same for a thread's float32 sum of CG (r', z or A' p with r' scaled to
+// an rms near 1, but r' of a guess far from the solution is as much larger as
+// its residual is): summed 2^32 times smaller, so that what fits float32 in a
+// thread fits it over any grid.
 __device__ __forceinline__ bool grid_sum_last(float v, double* partials, unsigned int* counter, double* total) {
-  return grid_sum_last(make_float2(v, 0.f), partials, counter, total);
+  const bool last = grid_sum_last(make_float2(v * 0x1p-32f, 0.f), partials, counter, total);
+  if (last && threadIdx.x == 0) *total *= 0x1p32;
+  return last;
 }
 
 // The same for float64 contributions.

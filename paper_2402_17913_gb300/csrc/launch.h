@@ -42,17 +42,17 @@ size_t coarse_layout(int* off, const LevelDev* lv, int nlev, int dim);
 // ghost rings and arrays, inverse diagonals) to `image` (device).
 cudaError_t launch_coarse_image(const CoarseArgs& a, float* image, size_t bytes, cudaStream_t s);
 // First level handled by the single-block kernel (or, with `dense`, by the
-// dense matrix of the coarse cycle).
+// dense matrix of the coarse cycle, whose set-up needs more shared memory).
 int coarse_start_level(const LevelDev* lv, int L, int dim, size_t smem_limit, bool dense);
 
-// The coarse cycle of level n cells as a dense matrix (mg_dense.cu): bytes of
-// the matrix and of its set-up's scratch, its set-up (a.finest 0; a wait
-// that times out sets st->status), and y = M b unless *done (b and y with
-// 16-byte aligned storage padded to a multiple of four values).
+// The coarse cycle of a level of n cells as a dense matrix (mg_dense.cu): bytes
+// of the matrix, its set-up (`layout_bytes` of coarse_layout, `inv` the
+// float64 coarsest inverse), and y = M b unless *done (b and y with 16-byte
+// aligned storage padded to a multiple of four values).
 size_t dense_bytes(int n);
-size_t dense_scratch_bytes(int n);
-cudaError_t launch_dense_matrix(const CoarseArgs& a, size_t smem_bytes, int n, float* M, float* scratch,
-                                SolveState* st, cudaStream_t s);
+size_t dense_smem(size_t layout_bytes, int nlev);
+cudaError_t launch_dense_matrix(const CoarseArgs& a, size_t layout_bytes, int n, const double* inv, double omega,
+                                double scale, float* M, cudaStream_t s);
 template <typename T>
 cudaError_t launch_dense(int dim, int n, const float* M, const void* b, void* y, const int* done, cudaStream_t s);
 int dense_stride(int n);  // floats of a row of M

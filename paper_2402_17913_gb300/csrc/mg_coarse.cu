@@ -78,9 +78,11 @@ int coarse_start_level(const LevelDev* lv, int L, int dim, size_t smem_limit, bo
   int kc = L - 1;
   int off[kMaxLevels];
   const size_t lim = coarse_cells_limit(dim, dense);
-  while (kc > 0 && (size_t)lv[kc - 1].nx * lv[kc - 1].ny * lv[kc - 1].nz <= lim &&
-         coarse_layout(off, lv + kc - 1, L - kc + 1, dim) <= smem_limit)
+  while (kc > 0 && (size_t)lv[kc - 1].nx * lv[kc - 1].ny * lv[kc - 1].nz <= lim) {
+    const size_t bytes = coarse_layout(off, lv + kc - 1, L - kc + 1, dim);
+    if ((dense ? dense_smem(bytes, L - kc + 1) : bytes) > smem_limit) break;
     --kc;
+  }
   return kc;
 }
 

@@ -4,8 +4,8 @@
 // of level kc's right-hand side: sweeps, transfers and the exact coarsest
 // solve have no data-dependent step.  For a level of at most a couple of
 // thousand cells its matrix (n x n floats, n^2 * 4 <= 16 MB, resident in L2)
-// is written once at create, a column per unit vector run through the
-// single-block coarse cycle, and a cycle then costs one matrix-vector product
+// is written once at create, a column per unit vector run through the cycle
+// in float-float, and a cycle then costs one matrix-vector product
 // over all SMs instead of a chain of some twenty block barriers on one SM
 // and, on grids whose sides are not powers of two, a dense coarsest inverse
 // of up to 1000^2 read by that SM.  Measured per cycle (launch included):
@@ -16,30 +16,214 @@
 
 #include "coarse.cuh"
 #include "launch.h"
+#include "refine.cuh"
 
 namespace npmg {
 
 namespace {
 
-// Column j of the matrix into row j of `Mt` (one block per column): the
-// coarse cycle of unit vector j.  `E` holds four zero arrays of 2 npad + 4
-// floats with a single 1 at npad + s in array s, so that E + s (2 npad + 4) +
-// npad + s - j is unit vector j and, with s = j mod 4, 16-byte aligned.
-template <int DIM>
-__global__ void __launch_bounds__(1024) k_dense_columns(const __grid_constant__ CoarseArgs a,
-                                                        const float* __restrict__ E, int npad, int ld,
-                                                        float* __restrict__ Mt, SolveState* __restrict__ st,
-                                                        int total_floats) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int j = blockIdx.x, s = j & 3;
-  coarse_cycle<DIM, float>(a, E + (size_t)s * (2 * npad + 4) + npad + s - j, Mt + (size_t)j * ld, st,
-                           reinterpret_cast<float*>(smem_raw), total_floats);
+constexpr int kColT = 256;  // threads of a column's block
+
+// Arrays of one level in the block's shared memory: x, x', b (float-float,
+// padded with a zero ring as in coarse.cuh) and the cell bytes (0 on the
+// ring); d, 1 / d and omega / d by link counts (0 where there are none).
+struct DLev {
+  CGeo g;
+  float wx, wy, wz;
+  float2 *x, *y, *b;
+  const float2 *d, *id, *w;
+  uint8_t* m;
+};
+constexpr int kTabs = 3 * 64;  // pairs of a level's tables
+
+__device__ __forceinline__ ff get(const float2* p, int i) { return {p[i].x, p[i].y}; }
+__device__ __forceinline__ void put(float2* p, int i, ff v) { p[i] = make_float2(v.hi, v.lo); }
+__device__ __forceinline__ ff to_ff(double v) {
+  const float hi = (float)v;
+  return {hi, (float)(v - (double)hi)};
+}
+__device__ __forceinline__ ff scale(ff a, float w) {
+  const float p = a.hi * w;
+  return quick_two_sum(p, fmaf(a.lo, w, fmaf(a.hi, w, -p)));
 }
 
-__global__ void k_unit_vectors(float* __restrict__ E, int npad) {
-  const int len = 2 * npad + 4;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < 4 * len; i += gridDim.x * blockDim.x)
-    E[i] = (i % len) == npad + i / len ? 1.f : 0.f;
+__device__ __forceinline__ DLev d_level(const CoarseArgs& a, int l, float2* tab, float2* arr, uint8_t* bytes) {
+  DLev v;
+  const LevelDev& L = a.lv[l];
+  v.g = cgeo(L, a.off[l]);
+  v.wx = L.wx;
+  v.wy = L.wy;
+  v.wz = L.wz;
+  const int P = v.g.WH * (v.g.nz + (v.g.nz > 1 ? 2 : 0)), o = a.off[l] / 4;  // padded cells, and those before
+  v.x = arr + 3 * o;
+  v.y = v.x + P;
+  v.b = v.y + P;
+  v.d = tab + kTabs * l;
+  v.id = v.d + 64;
+  v.w = v.id + 64;
+  v.m = bytes + o;
+  return v;
+}
+
+template <int DIM>
+__device__ __forceinline__ ff d_nb(const DLev& v, const float2* x, int p) {
+  ff nb = ff_add(scale(ff_add(get(x, p - 1), get(x, p + 1)), v.wx),
+                 scale(ff_add(get(x, p - v.g.W), get(x, p + v.g.W)), v.wy));
+  if (DIM == 3) nb = ff_add(nb, scale(ff_add(get(x, p - v.g.WH), get(x, p + v.g.WH)), v.wz));
+  return nb;
+}
+
+// f(i, p, entry of the tables or -1 off the fluid) on every cell, then a
+// barrier.
+template <typename F>
+__device__ __forceinline__ void d_cells(const DLev& v, F&& f) {
+  for (int i = threadIdx.x; i < v.g.n; i += kColT) {
+    int x, y, z;
+    v.g.xyz(i, x, y, z);
+    const int p = v.g.pad(x, y, z), m = v.m[p];
+    f(i, p, m ? m & 63 : -1, x, y, z);
+  }
+  __syncthreads();
+}
+
+__device__ __forceinline__ void d_swap(DLev& v) {
+  float2* t = v.x;
+  v.x = v.y;
+  v.y = t;
+}
+
+template <int DIM>
+__device__ __forceinline__ void d_sweep(DLev& v, ff keep) {
+  d_cells(v, [&](int, int p, int q, int, int, int) {
+    const ff zero = {0.f, 0.f};
+    put(v.y, p, q < 0 ? zero : ff_add(ff_mul(get(v.x, p), keep),
+                                      ff_mul(ff_add(get(v.b, p), d_nb<DIM>(v, v.x, p)), get(v.w, q))));
+  });
+  d_swap(v);
+}
+
+// Column j of the matrix into row j of `Mt` (one block per column): the
+// coarse cycle (coarse_cycle's steps) of unit vector j in float-float with the
+// float64 coarsest inverse, rounded to float32 once.  The columns of a float32
+// cycle carried its roundings into every product: a cycle on 64^2 was 0.9e-7
+// of its result off, 0.6e-7 with these (0.8e-7 to 1.4e-7 launch by launch).
+// 48 bits are enough for that, and one float64 instruction holds its pipe as
+// long as 64 float32 ones: creating a 64^2 handle takes 0.46 ms so, 0.58 with
+// float64 columns, 0.49 with float32 ones.  256 threads, so that an SM works
+// on several columns.
+template <int DIM>
+__global__ void __launch_bounds__(kColT) k_dense_columns(const __grid_constant__ CoarseArgs a,
+                                                        const double* __restrict__ inv, double omega, double s,
+                                                        float* __restrict__ Mt, int ld) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int j = blockIdx.x, last = a.nlev - 1, nc = a.ncoarse;
+  const bool saw = a.pre < 0;
+  float* __restrict__ out = Mt + (size_t)j * ld;
+  if (last == 0 && !saw) {  // the inverse itself
+    for (int i = threadIdx.x; i < nc; i += kColT) out[i] = (float)inv[(size_t)j * nc + i];
+    return;
+  }
+  float2* tab = reinterpret_cast<float2*>(smem_raw);
+  float2* arr = tab + kTabs * a.nlev;
+  int cells = 0;
+  for (int l = 0; l < a.nlev; ++l) {
+    const CGeo g = cgeo(a.lv[l], 0);
+    cells += g.WH * (g.nz + (g.nz > 1 ? 2 : 0));
+  }
+  uint8_t* bytes = reinterpret_cast<uint8_t*>(arr + 3 * cells);
+  for (int i = threadIdx.x; i < 3 * cells; i += kColT) arr[i] = make_float2(0.f, 0.f);
+  for (int i = threadIdx.x; i < cells; i += kColT) bytes[i] = 0;
+  for (int i = threadIdx.x; i < 64 * a.nlev; i += kColT) {
+    const LevelDev& L = a.lv[i >> 6];
+    const double d = (double)L.wx * (i & 3) + (double)L.wy * ((i >> 2) & 3) + (double)L.wz * ((i >> 4) & 3);
+    float2* t = tab + kTabs * (i >> 6) + (i & 63);
+    put(t, 0, to_ff(d));
+    put(t, 64, to_ff(d > 0.0 ? 1.0 / d : 0.0));
+    put(t, 128, to_ff(d > 0.0 ? omega / d : 0.0));
+  }
+  __syncthreads();
+  for (int l = 0; l < a.nlev; ++l) {
+    const LevelDev& L = a.lv[l];
+    const DLev v = d_level(a, l, tab, arr, bytes);
+    for (int i = threadIdx.x; i < v.g.n; i += kColT) {
+      int x, y, z;
+      v.g.xyz(i, x, y, z);
+      int m = kFluidBit | axis_count(x, L.nx, L.bcD, 0) | axis_count(y, L.ny, L.bcD, 2) << 2;
+      if (DIM == 3) m |= axis_count(z, L.nz, L.bcD, 4) << 4;
+      v.m[v.g.pad(x, y, z)] = L.cell ? L.cell[i] : (uint8_t)m;
+      if (l == 0 && i == j) v.b[v.g.pad(x, y, z)] = make_float2(1.f, 0.f);
+    }
+  }
+  __syncthreads();
+  const ff keep = to_ff(1.0 - omega), sc = to_ff(s), zero = {0.f, 0.f};
+  unsigned odd = 0u;  // bit l: level l's x and x' have changed places
+  auto level = [&](int l) {
+    DLev v = d_level(a, l, tab, arr, bytes);
+    if ((odd >> l) & 1u) d_swap(v);
+    return v;
+  };
+  // down legs: x from zero, the restricted residual (sawtooth: b's average)
+  for (int l = 0; l < last; ++l) {
+    DLev v = level(l);
+    const DLev c = level(l + 1);
+    d_cells(v, [&](int, int p, int q, int, int, int) {
+      put(v.x, p, q < 0 || a.pre == 0 ? zero : ff_mul(get(v.b, p), get(saw ? v.id : v.w, q)));
+    });
+    for (int k = 2; k <= a.pre; ++k) d_sweep<DIM>(v, keep);
+    if (a.pre > 1 && !(a.pre & 1)) odd |= 1u << l;
+    d_cells(c, [&](int, int pc, int, int X, int Y, int Z) {
+      ff sum = zero;
+      for (int k = 0; k < (DIM == 3 ? 8 : 4); ++k) {
+        const int p = v.g.pad(2 * X + (k & 1), 2 * Y + ((k >> 1) & 1), 2 * Z + (k >> 2)), m = v.m[p];
+        if (!m) continue;
+        ff r = get(v.b, p);
+        if (!saw) r = ff_add(r, ff_add(d_nb<DIM>(v, v.x, p), ff_neg(ff_mul(get(v.x, p), get(v.d, m & 63)))));
+        sum = ff_add(sum, r);
+      }
+      put(c.b, pc, scale(sum, DIM == 3 ? 0.125f : 0.25f));
+    });
+  }
+  // coarsest: A^-1 b in float64, a warp per row (sawtooth: a Jacobi step and
+  // the sweeps)
+  {
+    DLev v = level(last);
+    if (saw) {
+      d_cells(v, [&](int, int p, int q, int, int, int) {
+        put(v.x, p, q < 0 ? zero : ff_mul(get(v.b, p), get(v.id, q)));
+      });
+      for (int k = 1; k <= a.post; ++k) d_sweep<DIM>(v, keep);
+      if (a.post & 1) odd |= 1u << last;
+    } else {
+      const int lane = threadIdx.x & 31;
+      for (int i = threadIdx.x >> 5; i < nc; i += kColT / 32) {
+        double acc = 0.0;
+#pragma unroll 4
+        for (int k = lane; k < nc; k += 32) {
+          int x, y, z;
+          v.g.xyz(k, x, y, z);
+          const float2 b = v.b[v.g.pad(x, y, z)];
+          acc = fma(__ldg(inv + (size_t)i * nc + k), (double)b.x + (double)b.y, acc);
+        }
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        int x, y, z;
+        v.g.xyz(i, x, y, z);
+        if (lane == 0) put(v.x, v.g.pad(x, y, z), to_ff(acc));
+      }
+      __syncthreads();
+    }
+  }
+  // up legs: x + s P e, the sweeps
+  for (int l = last - 1; l >= 0; --l) {
+    DLev v = level(l);
+    const DLev c = level(l + 1);
+    d_cells(v, [&](int, int p, int q, int X, int Y, int Z) {
+      if (q >= 0) put(v.x, p, ff_add(get(v.x, p), ff_mul(get(c.x, c.g.pad(X >> 1, Y >> 1, Z >> 1)), sc)));
+    });
+    for (int k = 1; k <= a.post; ++k) d_sweep<DIM>(v, keep);
+    if (a.post & 1) odd ^= 1u << l;
+  }
+  const DLev v = level(0);
+  d_cells(v, [&](int i, int p, int, int, int, int) { out[i] = v.x[p].x + v.x[p].y; });
 }
 
 // In-place transposition of the n x n matrix (row stride ld): a block swaps
@@ -125,7 +309,6 @@ __global__ void __launch_bounds__(32 * kRowWarps) k_dense(int n, int ld, const f
 
 int dense_stride(int n) { return (n + 3) & ~3; }
 size_t dense_bytes(int n) { return (size_t)n * dense_stride(n) * sizeof(float); }
-size_t dense_scratch_bytes(int n) { return 4 * (size_t)(2 * dense_stride(n) + 4) * sizeof(float); }
 
 cudaError_t launch_transpose(float* M, int n, cudaStream_t s) {
   const int t = (n + 31) / 32;
@@ -133,8 +316,12 @@ cudaError_t launch_transpose(float* M, int n, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_dense_matrix(const CoarseArgs& a, size_t smem_bytes, int n, float* M, float* scratch,
-                                SolveState* st, cudaStream_t s) {
+// Shared memory of a column's block: the tables, three float-float arrays and
+// the cell bytes (`bytes`: what coarse_layout asks, 16 per padded cell).
+size_t dense_smem(size_t bytes, int nlev) { return (size_t)nlev * kTabs * 8 + bytes / 16 * 25; }
+
+cudaError_t launch_dense_matrix(const CoarseArgs& a, size_t layout_bytes, int n, const double* inv, double omega,
+                                double scale, float* M, cudaStream_t s) {
   const int ld = dense_stride(n);
   const auto k = a.dim == 3 ? k_dense_columns<3> : k_dense_columns<2>;
   cudaError_t e = cudaMemsetAsync(M, 0, dense_bytes(n), s);
@@ -143,8 +330,7 @@ cudaError_t launch_dense_matrix(const CoarseArgs& a, size_t smem_bytes, int n, f
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - 1024);
   if (e != cudaSuccess) return e;
-  k_unit_vectors<<<32, 256, 0, s>>>(scratch, ld);
-  k<<<n, 1024, smem_bytes, s>>>(a, scratch, ld, ld, M, st, (int)(smem_bytes / sizeof(float)));
+  k<<<n, kColT, dense_smem(layout_bytes, a.nlev), s>>>(a, inv, omega, scale, M, ld);
   e = cudaGetLastError();
   return e == cudaSuccess ? launch_transpose(M, n, s) : e;
 }

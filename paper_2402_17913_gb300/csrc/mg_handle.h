@@ -41,7 +41,6 @@ struct mg_handle_s {
   double* inv;
   float* cimage;   // constant shared-memory image of the single-block kernel
   float* dense;    // the coarse cycle's matrix (levels kc .. L-1; nullptr when kc == 0)
-  float* dense_scratch;
   int ncoarse;
   double* partials;
   npmg::SolveState* st;

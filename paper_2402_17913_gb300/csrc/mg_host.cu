@@ -60,6 +60,9 @@ cudaError_t prof_flush(mg_handle_s* h) {
   return cudaSuccess;
 }
 
+// The float64 coarsest inverse, behind the float32 copy (launch_coarse_inverse).
+static const double* inv64(const mg_handle_s* h) { return h->inv + (size_t)h->ncoarse * h->ncoarse; }
+
 // The refinement iterate and residual in float64 (MG_REFINE_FP64, the
 // default) or in float-float pairs (MG_REFINE_FF); 8 bytes per cell either way.
 static bool f64_iterate(const mg_handle_s* h) { return h->opt.refine != MG_REFINE_FF; }
@@ -689,10 +692,7 @@ mg_status mg_create(mg_handle* out, int dim, const int64_t shape[3], const doubl
   plan.push_back({(void**)&h->bsave, n0c * 4});
   plan.push_back({(void**)&h->inv, (size_t)2 * h->ncoarse * h->ncoarse * 8});
   plan.push_back({(void**)&h->cimage, h->ca_smem});
-  if (kc > 0) {
-    plan.push_back({(void**)&h->dense, dense_bytes((int)h->ncell[kc])});
-    plan.push_back({(void**)&h->dense_scratch, dense_scratch_bytes((int)h->ncell[kc])});
-  }
+  if (kc > 0) plan.push_back({(void**)&h->dense, dense_bytes((int)h->ncell[kc])});
   if (dim == 2 && o.prec == MG_FP32 && kc >= 1) {
     // the cluster path's coarse cycle starts at level kc or below: its
     // right-hand side, correction and shared-memory image fit level kc's
@@ -781,7 +781,7 @@ mg_status mg_create(mg_handle* out, int dim, const int64_t shape[3], const doubl
     NPMG_TRY(launch_coarse_image(ca, h->cimage, h->ca_smem, s));
     ca.image = h->cimage;
     if (kc > 0) {
-      NPMG_TRY(launch_dense_matrix(ca, h->ca_smem, (int)h->ncell[kc], h->dense, h->dense_scratch, h->st, s));
+      NPMG_TRY(launch_dense_matrix(ca, h->ca_smem, (int)h->ncell[kc], inv64(h), o.omega, o.coarse_scale, h->dense, s));
     }
   }
   h->nb1d = default_blocks_1d(h, h->ncell[0]);
@@ -884,7 +884,7 @@ mg_status mg_create(mg_handle* out, int dim, const int64_t shape[3], const doubl
         const int nd = (int)h->ncell[h->cpcg_kd];
         if (h->cpcg_dense && nd <= kClusterDense && nd % (4 * pa.a.C) == 0) {
           if (e == cudaSuccess)
-            e = launch_dense_matrix(cc, ca_bytes, nd, h->cpcg_dense, h->dense_scratch, h->st, s);
+            e = launch_dense_matrix(cc, ca_bytes, nd, inv64(h), o.omega, o.coarse_scale, h->cpcg_dense, s);
           pa.a.dense = h->cpcg_dense;
           pa.a.dense_n = nd;
         }
@@ -899,15 +899,9 @@ mg_status mg_create(mg_handle* out, int dim, const int64_t shape[3], const doubl
                                  (const float*)h->p[1], (const float*)h->d, (const float*)h->r);
     return e;
   }));
-  NPMG_TRY(cudaMemcpyAsync(h->st_host, h->st, sizeof(SolveState), cudaMemcpyDeviceToHost, s));
   NPMG_TRY(cudaStreamSynchronize(s));
   NPMG_TRY(cudaGetLastError());
 #undef NPMG_TRY
-  if (kc > 0 && h->st_host->status == MG_TIMEOUT) {
-    set_error("mg_create: a load of the coarse cycle's set-up timed out");
-    st = MG_TIMEOUT;
-    goto fail;
-  }
   *out = h;
   return MG_OK;
 fail:

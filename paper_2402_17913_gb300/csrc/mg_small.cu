@@ -71,6 +71,19 @@ __device__ __forceinline__ float nbsum(const LevelDev& L, const float* x, int i)
   return nb;
 }
 
+// One sweep of a cell, x + (omega / d)(b + nb - d x).  The error of omega / d
+// then scales with the residual; in (1 - omega) x + (omega / d)(b + nb) it
+// scales with x, the same in every interior cell, and is a bias of the whole
+// cycle: on 48 x 64 x 56 against 64 bits 1.5e-7, 0.64e-7 so (1.0e-7 with the
+// streamed columns and their rounded quotient).  A rounded quotient formed
+// before the wait instead gave 1.2e-7 and cost 1.3 us of a 27.1 us cycle on
+// 96 x 80 x 64; this form costs 0.6 us.
+template <int DIM>
+__device__ __forceinline__ float sweep_cell(const LevelDev& L, const float* x, const float* sB, float d, float omega,
+                                            int i) {
+  return d > 0.f ? fmaf(__fdividef(omega, d), fmaf(-d, x[i], sB[i] + nbsum<DIM>(L, x, i)), x[i]) : 0.f;
+}
+
 // One sweep of the cells of the tile and its one-cell ring.
 template <int DIM>
 __device__ __forceinline__ void sweep_ring(const LevelDev& L, const float* xin, float* xout, const float* sB,
@@ -82,8 +95,7 @@ __device__ __forceinline__ void sweep_ring(const LevelDev& L, const float* xin, 
     if (i < W::SN) {
       const int lz = DIM == 3 ? i / (W::SX * W::SY) + 1 : 0;
       const int li = lz * W::RXY + ((i / W::SX) % W::SY + 1) * W::RX + i % W::SX + 1;
-      const float d = sD[li];
-      xout[li] = d > 0.f ? fmaf(1.f - omega, xin[li], __fdividef(omega, d) * (sB[li] + nbsum<DIM>(L, xin, li))) : 0.f;
+      xout[li] = sweep_cell<DIM>(L, xin, sB, sD[li], omega, li);
     }
   }
 }
@@ -191,10 +203,7 @@ __global__ void __launch_bounds__(NT) k_up_c(LevelDev L, const TB* __restrict__ 
   const int li = out_cell<DIM>(gx, gy, gz);
   float acc = 0.f;
   if (inside<DIM>(L, gx, gy, gz)) {
-    const float dc = sD[li];
-    const float z =
-        dc > 0.f ? fmaf(1.f - omega, s1[li], __fdividef(omega, dc) * (sB[li] + nbsum<DIM>(L, s1, li))) : 0.f;
-    const TB zt = cvt<TB>(z);
+    const TB zt = cvt<TB>(sweep_cell<DIM>(L, s1, sB, sD[li], omega, li));
     xout[(gz * L.ny + gy) * L.nx + gx] = zt;
     if (FINEST) acc = sB[li] * ld(&zt, 0);
   }

@@ -319,19 +319,11 @@ __device__ __noinline__ void b_up_h(const LevelDev& L, int tx, int ty, const flo
 }
 
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ float4 lds4(const float* p) { return *reinterpret_cast<const float4*>(p); }
-__device__ __forceinline__ void sts4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
 __device__ __forceinline__ float lane(const float4& v, int k) {
   return k == 0 ? v.x : k == 1 ? v.y : k == 2 ? v.z : v.w;
 }
 __device__ __forceinline__ uint8_t lane(const uchar4& v, int k) {
   return k == 0 ? v.x : k == 1 ? v.y : k == 2 ? v.z : v.w;
-}
-__device__ __forceinline__ void set_lane(float4& v, int k, float a) {
-  if (k == 0) v.x = a;
-  else if (k == 1) v.y = a;
-  else if (k == 2) v.z = a;
-  else v.w = a;
 }
 // cell bytes of a group (all fluid on a level without solid)
 __device__ __forceinline__ uchar4 v_cells(const LevelDev& L, int gi) {
@@ -678,8 +670,7 @@ __global__ void __launch_bounds__(kBThreads, kBBlocks) k_batched(const __grid_co
         const BInst& I = A.inst[item.x];
         __syncthreads();
         if (item.y >= 0) b_dense_rows(I, item.y, S);
-        else coarse_cycle<2, float, false>(I.ca, I.kc == 0 ? I.r : I.b[I.kc], I.kc == 0 ? I.z : I.y[I.kc], nullptr, S,
-                               I.cfloats);
+        else coarse_cycle<2, float, false>(I.ca, I.b[I.kc], I.y[I.kc], nullptr, S, I.cfloats);
       }
       if (!grid_barrier(A, epoch)) return;
       // up legs; the finest produces z = M r and (r, z)
@@ -1077,7 +1068,7 @@ mg_status mg_create_batched(mg_batch* out, int count, const int64_t* shapes, con
     I.L = L;
     int kc = L - 1;
     while (kc > 0 && (size_t)(nx >> (kc - 1)) * (ny >> (kc - 1)) <= (size_t)kBCoarseCells) --kc;
-    I.kc = kc;
+    I.kc = kc;  // at least 1: level 0 has more cells, and a one-level grid is turned down below
     max_kc = kc > max_kc ? kc : max_kc;
     const double c = spacing[2 * i] * spacing[2 * i];
     I.c = c;
@@ -1209,12 +1200,9 @@ mg_status mg_create_batched(mg_batch* out, int count, const int64_t* shapes, con
     // coarsest inverse and the block-local coarse item
     {
       const int Lc = I.L - 1;
-      const double hx = std::ldexp(1.0, Lc), c = I.c;
-      (void)hx;
-      const double wc[3] = {(double)I.lv[Lc].wx, (double)I.lv[Lc].wy, 0.0};
+      const double c = I.c;
       const double wd[3] = {c / (spacing[2 * i] * spacing[2 * i] * std::ldexp(1.0, 2 * Lc)),
                             c / (spacing[2 * i + 1] * spacing[2 * i + 1] * std::ldexp(1.0, 2 * Lc)), 0.0};
-      (void)wc;
       const int64_t n3[3] = {I.lv[Lc].nx, I.lv[Lc].ny, 1};
       NPMG_BTRY(launch_coarse_inverse(2, n3, wd, I.lv[Lc].bcD, I.lv[Lc].cell, (double*)(P + f.inv), s));
       CoarseArgs& ca = I.ca;
@@ -1354,7 +1342,7 @@ static mg_status build_items(mg_batch_s* B, int tile, cudaStream_t s) {
     std::vector<int2> ci;
     for (int i = 0; i < B->count; ++i) {
       const BInst& I = B->inst[i];
-      if (I.kc > 0 && I.kc == I.L - 1 && I.ca.ncoarse > kBDense && I.ca.pre >= 0)
+      if (I.kc == I.L - 1 && I.ca.ncoarse > kBDense && I.ca.pre >= 0)
         for (int r = 0; r < I.ca.ncoarse; r += kBRows) ci.push_back(make_int2(i, r));
       else
         ci.push_back(make_int2(i, -1));

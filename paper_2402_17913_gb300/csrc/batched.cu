@@ -379,7 +379,7 @@ __device__ __forceinline__ float s_up(const LevelDev& L, const Strip& t, const f
 // after (r, z) and (p, Ap) form theirs so where no instance has more than
 // kFoldStrips partials, four a lane; else a phase of their own does it, which
 // with its barrier takes 4 us.  256 instances of sides 64-512 (80 partials):
-// 18.3 -> 17.9 ms, four of 64-192 (96): 2.33 -> 2.14; with 640 partials (four
+// 18.3 -> 18.2 ms, four of 64-192 (96): 2.33 -> 2.29; with 640 partials (four
 // of 64-512) the phases are faster, 3.66 against 3.87.
 constexpr int kFoldStrips = 128;
 struct StripSum {

@@ -874,6 +874,17 @@ static std::string tune_cache_path() {
   return std::string(home ? home : "/tmp") + "/.cache/npmg_batched_tune.txt";
 }
 
+// Part of the cache's key: 2 since the level legs run on warp strips.  Raised
+// whenever the kernels that a choice was measured on are replaced.
+constexpr int kTuneGeneration = 2;
+
+// FNV-1a over the bytes of a word.
+constexpr uint64_t kHashSeed = 0xcbf29ce484222325ull;
+static uint64_t hash_word(uint64_t h, uint64_t v) {
+  for (int k = 0; k < 8; ++k) h = (h ^ ((v >> (8 * k)) & 255u)) * 0x100000001b3ull;
+  return h;
+}
+
 // cache lines: "<key> <tile> <sweeps> <ms>"
 static bool tune_lookup(const std::string& key, int* tile, int* sweeps) {
   FILE* f = fopen(tune_cache_path().c_str(), "r");
@@ -1255,8 +1266,17 @@ mg_status mg_create_batched(mg_batch* out, int count, const int64_t* shapes, con
     if (cudaGetDeviceProperties(&prop, B->device) == cudaSuccess) snprintf(name, sizeof name, "%s", prop.name);
     for (char* c = name; *c; ++c)
       if (*c == ' ') *c = '_';
+    // the choice depends on every instance's sides and solids and on the faces
+    uint64_t hash = kHashSeed;
+    for (int f = 0; f < 4; ++f) hash = hash_word(hash, (uint64_t)bc[f]);
+    for (int i = 0; i < count; ++i) {
+      hash = hash_word(hash, (uint64_t)B->inst[i].nx);
+      hash = hash_word(hash, (uint64_t)B->inst[i].ny);
+      hash = hash_word(hash, (uint64_t)B->inst[i].nfluid);
+    }
     char key[512];
-    snprintf(key, sizeof key, "%s|n%d|cells%lld|max%d|p%d", name, count, total_cells, max_side, o.pre);
+    snprintf(key, sizeof key, "%s|n%d|cells%lld|max%d|p%d|g%d|%016llx", name, count, total_cells, max_side, o.pre,
+             kTuneGeneration, (unsigned long long)hash);
     B->tune_key = key;
   }
   B->tile = 0;

@@ -78,7 +78,7 @@ struct mg_handle_s {
   int cpcg_kd;
   size_t cpcg_smem;
   float* cpcg_image;              // its coarse cycle's constant image
-  float* cpcg_dense;              // and matrix (levels of at most kClusterDense cells)
+  float* cpcg_dense;              // and matrix (levels of at most kClusterDense cells, where it is not `dense`)
   int64_t chunk_kernels;   // kernels in one graph launch
   // instrumentation
   int64_t launches;

@@ -883,9 +883,10 @@ mg_status mg_create(mg_handle* out, int dim, const int64_t shape[3], const doubl
         pa.a.s = (float)o.coarse_scale;
         const int nd = (int)h->ncell[h->cpcg_kd];
         if (h->cpcg_dense && nd <= kClusterDense && nd % (4 * pa.a.C) == 0) {
-          if (e == cudaSuccess)
+          // the cycle's own matrix where both start at the same level
+          pa.a.dense = h->cpcg_kd == h->kc ? h->dense : h->cpcg_dense;
+          if (e == cudaSuccess && h->cpcg_kd != h->kc)
             e = launch_dense_matrix(cc, ca_bytes, nd, inv64(h), o.omega, o.coarse_scale, h->cpcg_dense, s);
-          pa.a.dense = h->cpcg_dense;
           pa.a.dense_n = nd;
         }
         h->cpcg = pa;

@@ -183,8 +183,7 @@ __global__ void __launch_bounds__(kColT) k_dense_columns(const __grid_constant__
       put(c.b, pc, scale(sum, DIM == 3 ? 0.125f : 0.25f));
     });
   }
-  // coarsest: A^-1 b in float64, a warp per row (sawtooth: a Jacobi step and
-  // the sweeps)
+  // coarsest: A^-1 b in float64 (sawtooth: a Jacobi step and the sweeps)
   {
     DLev v = level(last);
     if (saw) {
@@ -194,20 +193,39 @@ __global__ void __launch_bounds__(kColT) k_dense_columns(const __grid_constant__
       for (int k = 1; k <= a.post; ++k) d_sweep<DIM>(v, keep);
       if (a.post & 1) odd |= 1u << last;
     } else {
-      const int lane = threadIdx.x & 31;
-      for (int i = threadIdx.x >> 5; i < nc; i += kColT / 32) {
+      // a unit vector reaches a few coarsest cells only: their list (in order,
+      // so that the sums are the same every time) in the array x' has no use
+      // for, then a row per thread
+      __shared__ int count;
+      int* list = reinterpret_cast<int*>(v.y);
+      if (threadIdx.x < 32) {
+        int have = 0;
+        for (int k0 = 0; k0 < nc; k0 += 32) {
+          const int k = k0 + (int)threadIdx.x;
+          bool on = false;
+          if (k < nc) {
+            int x, y, z;
+            v.g.xyz(k, x, y, z);
+            on = v.b[v.g.pad(x, y, z)].x != 0.f;
+          }
+          const unsigned mask = __ballot_sync(0xffffffffu, on);
+          if (on) list[have + __popc(mask & ((1u << threadIdx.x) - 1u))] = k;
+          have += __popc(mask);
+        }
+        if (threadIdx.x == 0) count = have;
+      }
+      __syncthreads();
+      for (int i = threadIdx.x; i < nc; i += kColT) {
         double acc = 0.0;
-#pragma unroll 4
-        for (int k = lane; k < nc; k += 32) {
-          int x, y, z;
+        int x, y, z;
+        for (int q = 0; q < count; ++q) {
+          const int k = list[q];
           v.g.xyz(k, x, y, z);
           const float2 b = v.b[v.g.pad(x, y, z)];
-          acc = fma(__ldg(inv + (size_t)i * nc + k), (double)b.x + (double)b.y, acc);
+          acc = fma(__ldg(inv + (size_t)k * nc + i), (double)b.x + (double)b.y, acc);
         }
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        int x, y, z;
         v.g.xyz(i, x, y, z);
-        if (lane == 0) put(v.x, v.g.pad(x, y, z), to_ff(acc));
+        put(v.x, v.g.pad(x, y, z), to_ff(acc));
       }
       __syncthreads();
     }

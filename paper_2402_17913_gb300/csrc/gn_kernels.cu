@@ -861,15 +861,21 @@ static cudaError_t conv_epi(const void* x, const void* wpack, ConvArgs a, cudaSt
   if (grid_cache < 0) return cudaErrorInvalidValue;
   // z-runs: a run of c outputs costs c + 2 planes.  The tensor core's operand
   // reads bound an SM that has two or more runs in work (its runs' planes add
-  // up); a lone run is bound by its own chain, about 1.7 planes' time each;
-  // and a block's start costs about eight planes.
+  // up: 0.36 us a plane on 256 x 128 x 128 voxels); a lone run is bound by its
+  // own chain (0.68 us a plane on 64 x 64 x 256 in one and in two runs), so it
+  // counts 1.7 of those planes; 1.5 to 1.9 give the same runs on all shapes
+  // below.  Whole gn_conv3d calls, 44 us of each not the convolution, in
+  // 1 / 2 / 4 / 6 / 8 / 16 runs: 8 x 64^3 (4 chosen) 98 / 96 / 89 / 96 / 95 / 96 us,
+  // 256 x 128 x 128 (4) 157 / 144 / 134 / 145 / 133 / 134, 64^3 (8) 83 / 59 / 49 / 47 /
+  // 46 / 46, 64 x 64 x 256 (9: 70) 219 / 132 / 82 / 82 / 69 / 69, 96 x 80 x 64 (5: 54)
+  // 83 / 59 / 57 / 56 / 57 / 57, 3 x 100 x 60 x 40 (4) 71 / 66 / 58 / 59 / 60.
   const long long columns = (long long)a.tx * a.ty * a.nn;
   const long long nsm = device_sms();
   double best = -1.0;
   for (int runs = 1; runs <= (a.nz + 3) / 4; ++runs) {
     const int zc = (a.nz + runs - 1) / runs;
     const long long items = columns * ((a.nz + zc - 1) / zc);
-    const double cost = std::max((double)((items + nsm - 1) / nsm), 1.7) * (zc + 2) + 8.0;
+    const double cost = std::max((double)((items + nsm - 1) / nsm), 1.7) * (zc + 2);
     if (best >= 0.0 && cost >= best) continue;
     best = cost;
     a.zc = zc;
@@ -877,7 +883,8 @@ static cudaError_t conv_epi(const void* x, const void* wpack, ConvArgs a, cudaSt
     a.nitems = items;
   }
   const long long g = a.nitems < grid_cache ? a.nitems : grid_cache;
-  k_conv<EPI><<<(unsigned)(g > 0 ? g : 1), kConvThreads, kConvSmem, s>>>((const unsigned char*)x, (const unsigned char*)wpack, a);
+  k_conv<EPI><<<(unsigned)(g > 0 ? g : 1), kConvThreads, kConvSmem, s>>>((const unsigned char*)x,
+                                                                          (const unsigned char*)wpack, a);
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return cudaGetLastError();
 }

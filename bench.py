@@ -834,7 +834,7 @@ def run_gpu(args, rank, world):
         cyc = statistics.mean(st["cycles"] for st in step_stats)
         ms_solve = total_ms / args.steps
         achieved = per_cycle * cyc / (ms_solve * 1e-3) / 1e9
-        roofline = {"bound": "hbm", "kernel": "whole solve (k_ad_resid, k_ad_down, k_ad_coarse, k_ad_up)",
+        roofline = {"bound": "hbm", "kernel": "whole solve (k_ad_resid, k_ad_down, k_dense, k_ad_up)",
                     "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
                     "frac": round(achieved / peak, 4), "peak_source": peak_kind, "traffic": None,
                     "algorithmic_bytes_per_cycle": per_cycle, "cycles_per_solve": cyc,

@@ -75,13 +75,16 @@ __device__ __forceinline__ float nbsum(const LevelDev& L, const float* x, int i)
 // then scales with the residual; in (1 - omega) x + (omega / d)(b + nb) it
 // scales with x, the same in every interior cell, and is a bias of the whole
 // cycle: on 48 x 64 x 56 against 64 bits 1.5e-7, 0.64e-7 so (1.0e-7 with the
-// streamed columns and their rounded quotient).  A rounded quotient formed
-// before the wait instead gave 1.2e-7 and cost 1.3 us of a 27.1 us cycle on
-// 96 x 80 x 64; this form costs 0.6 us.
+// streamed columns and their rounded quotient; that one here, formed before
+// the wait, gave 1.2e-7).  Formed in every cell and selected at the end: with
+// the formula behind the test of d its loads wait for d (96 x 80 x 64 cycle
+// 27.8 us, 26.9 so, 27.0 in the biased form).
 template <int DIM>
 __device__ __forceinline__ float sweep_cell(const LevelDev& L, const float* x, const float* sB, float d, float omega,
                                             int i) {
-  return d > 0.f ? fmaf(__fdividef(omega, d), fmaf(-d, x[i], sB[i] + nbsum<DIM>(L, x, i)), x[i]) : 0.f;
+  const float xc = x[i], nb = nbsum<DIM>(L, x, i);
+  const float v = fmaf(__fdividef(omega, d), nb + fmaf(-d, xc, sB[i]), xc);
+  return d > 0.f ? v : 0.f;
 }
 
 // One sweep of the cells of the tile and its one-cell ring.

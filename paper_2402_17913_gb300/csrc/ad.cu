@@ -64,6 +64,7 @@ struct State {
   double bnorm2, relres, relres0, l1, l1_first;
   int cycles, done, status;
   float rscale;         // power of two near 1 / ||b||^2: the grid's sums of r^2 are float32 pairs
+  double snorm2;        // rscale ||b||^2, NaN where that norm is not finite
   unsigned int counter[2];
   unsigned int checks;  // of the device-side loop
 };
@@ -105,7 +106,9 @@ __global__ void __launch_bounds__(kT) k_ad_init(Lev L, const float* __restrict__
     st->l1_tol = l1_tol;
     st->max_cycles = max_cycles;
     st->bnorm2 = tot;
-    st->rscale = tot > 0.0 && isfinite(tot) ? ldexpf(1.f, -max(-126, min(126, ilogb(tot)))) : 1.f;
+    const float rs = tot > 0.0 && isfinite(tot) ? ldexpf(1.f, -max(-126, min(126, ilogb(tot)))) : 1.f;
+    st->rscale = rs;
+    st->snorm2 = isfinite(tot) ? tot * (double)rs : nan("");
     st->relres = st->relres0 = 1.0;
     st->l1 = st->l1_first = 0.0;
     st->cycles = 0;
@@ -120,8 +123,7 @@ __global__ void __launch_bounds__(kT) k_ad_init(Lev L, const float* __restrict__
 // taken before each cycle: converged, diverged (1000-fold growth, or a
 // right-hand side whose norm is not finite) or out of cycles.
 __device__ void decide(State* st, double srr, bool final) {
-  const double bn2 = st->bnorm2, rr = srr / (double)st->rscale;
-  const double rel = bn2 == 0.0 ? 0.0 : isfinite(bn2) ? sqrt(rr / bn2) : nan("");
+  const double sb = st->snorm2, rel = sb == 0.0 ? 0.0 : sqrt(srr / sb);
   st->relres = rel;
   if (final) return;
   if (st->cycles == 0) st->relres0 = rel;
@@ -157,6 +159,7 @@ __global__ void __launch_bounds__(kT) k_ad_resid(Lev L, const float* __restrict_
                                                  float* __restrict__ r, State* st, double* partials) {
   chain_enter();
   if (!FINAL && st->done) return;
+  const float rscale = st->rscale;  // at the end its latency would stand alone
   float acc = 0.f;
   const int gxn = (L.nx + 127) / 128, groups = gxn * ((L.ny + 7) / 8);
   for (int g = blockIdx.x; g < groups; g += gridDim.x) {
@@ -220,7 +223,7 @@ __global__ void __launch_bounds__(kT) k_ad_resid(Lev L, const float* __restrict_
     }
   }
   double tot;
-  if (grid_sum_last(make_float2(acc * st->rscale, 0.f), partials, &st->counter[0], &tot) && threadIdx.x == 0)
+  if (grid_sum_last(make_float2(acc * rscale, 0.f), partials, &st->counter[0], &tot) && threadIdx.x == 0)
     decide(st, tot, FINAL);
 }
 
@@ -325,6 +328,7 @@ __global__ void __launch_bounds__(kT) k_ad_down_saw(Lev L, const float* __restri
                                                     double* partials) {
   chain_enter();
   if (st->done) return;
+  const float rscale = FUSED ? st->rscale : 1.f;
   const int cnx = L.nx / 2;
   const size_t nc = (size_t)cnx * (L.ny / 2);
   float acc = 0.f;
@@ -356,7 +360,7 @@ __global__ void __launch_bounds__(kT) k_ad_down_saw(Lev L, const float* __restri
   }
   if (FUSED) {
     double tot;
-    if (grid_sum_last(make_float2(acc * st->rscale, 0.f), partials, &st->counter[0], &tot) && threadIdx.x == 0)
+    if (grid_sum_last(make_float2(acc * rscale, 0.f), partials, &st->counter[0], &tot) && threadIdx.x == 0)
       decide(st, tot, false);
   }
 }

@@ -20,10 +20,9 @@ static int grid_1d(size_t n, int cap) {
 // ---------------------------------------------------------------------------
 // The whole cycle of a grid of at most 2048 cells, and of the coarse levels of
 // the allocation-free cycle (handles apply those as one dense matrix,
-// mg_dense.cu, whose columns this block's cycle computes): down legs, the
-// exact coarsest solve and up legs inside one block of 1024 threads with
-// every level resident in shared memory.  One SM executes it, so it is written for instruction
-// count: each level is stored with a zero ghost ring (no bounds checks; the
+// mg_dense.cu): down legs, the exact coarsest solve and up legs inside one
+// block of 1024 threads with every level resident in shared memory.  One SM
+// executes it, so it is written for instruction count: each level is stored with a zero ghost ring (no bounds checks; the
 // ring is the zero padding of Sec. 2.1), the inverse diagonal is computed
 // once per launch (0 marks a non-fluid cell), and a sweep is
 // x <- (1 - omega) x + omega D^-1 (b + sum_a w_a (x_- + x_+)).  The
